@@ -123,12 +123,13 @@ typedef struct crn_grid crn_grid;
  * Returns CRN_E_ARG if d is NULL. */
 int crn_grid_desc_default(crn_grid_desc* d, int32_t n_r, int32_t n_theta, int32_t n_phi);
 
-/* Radial planes per CTA that crn_grid_create gives the tiled residual: the
- * chunk whose CTAs, list-scheduled in launch order (all `ntiles` (theta, phi)
- * tiles of chunk 0, then chunk 1, ...) onto `slots` resident CTAs, each costing
- * its planes plus `overhead` planes (crn_grid_create uses 3), finish first;
- * ties go to the larger chunk; at least 4 planes (n_r if smaller).  Pure host
- * function; -1 on a non-positive argument. */
+/* Radial planes per CTA from a plain makespan model (the chunk crn_grid_create
+ * gives the TMA-staged kernel; the tiled residual's comes from a simulation of
+ * its launch that also goes below 4 planes): the chunk whose CTAs,
+ * list-scheduled in launch order (all `ntiles` (theta, phi) tiles of chunk 0,
+ * then chunk 1, ...) onto `slots` resident CTAs, each costing its planes plus
+ * `overhead` planes, finish first; ties go to the larger chunk; at least 4
+ * planes (n_r if smaller).  Pure host function; -1 on a non-positive argument. */
 int32_t crn_tiled_radial_chunk(int32_t n_r, int64_t ntiles, int64_t slots, int32_t overhead);
 
 /* Create a grid on the current CUDA device: validates *d (CRN_E_ARG with a
@@ -418,7 +419,8 @@ int crn_ensemble_pseudo_time_step(crn_ensemble* e, double* const* U64_dev, int32
 int crn_ensemble_autotune(crn_ensemble* e, const void* const* U_dev, void* const* R_dev, void* stream,
                           int32_t* kchunk_out);
 
-/* Tile shape (0: 8 x 32, 1: 16 x 16 (theta, phi) columns per CTA) and radial
+/* Tile shape (0: 8 x 32, 1: 16 x 16, 2: 8 x 16 (theta, phi) columns per CTA; 2
+ * is the own shape of FP64 members and theirs only, 0 of FP32 members) and radial
  * chunk (planes per work item; 0 = the member's own single-launch chunk) of
  * member m in the persistent launch.  CRN_E_ARG for an index, shape or chunk
  * out of range; a chunk that gives a member more work items than its

@@ -516,7 +516,7 @@ class Ensemble:
     def last_launch_count(self):
         return int(_lib.crn_ensemble_launch_count(self._h))
 
-    TILES = {0: (8, 32), 1: (16, 16)}
+    TILES = {0: (8, 32), 1: (16, 16), 2: (8, 16)}
 
     def member_config(self, m):
         """(tile shape (theta, phi), radial chunk) member m runs with."""
@@ -525,7 +525,7 @@ class Ensemble:
         return self.TILES[t.value], k.value
 
     def set_member_config(self, m, tile=(8, 32), kchunk=0):
-        """Tile shape ((8, 32) or (16, 16)) and radial chunk (0: the member's own) of member m."""
+        """Tile shape ((8, 32), (16, 16) or, in FP64, (8, 16)) and radial chunk (0: the member's own) of member m."""
         code = {v: c for c, v in self.TILES.items()}[tuple(tile)]
         _check(_lib.crn_ensemble_set_member_config(self._h, int(m), code, int(kchunk)))
 

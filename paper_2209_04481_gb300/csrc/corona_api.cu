@@ -337,17 +337,18 @@ int crn_grid_create(const crn_grid_desc* d, crn_grid** out) {
   g->ph64 = make_phys<double>(*d, h);
   g->ph32 = make_phys<float>(*d, h);
   // opt the kernels in to their shared memory, then size the tiled launch:
-  // radial chunk from the makespan model over the resident CTA slots
+  // radial chunk from the simulated launch
   e = d->precision == CRN_FP64 ? crn::prepare_fp64() : crn::prepare_fp32();
   if (e != cudaSuccess) { delete g; return cuda_fail(e, "kernel attributes"); }
   {
-    const int tt = 8, tp = 32;
+    const int tile = crn::own_tile(d->precision == CRN_FP64);
+    const int tt = crn::ens_tt(tile), tp = crn::ens_tp(tile);
     const int64_t ntiles = (int64_t)((d->n_theta + tt - 1) / tt) * ((d->n_phi + tp - 1) / tp);
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, g->device);
     const int per_sm = d->precision == CRN_FP64 ? crn::tiled_ctas_per_sm_fp64(d->limiter)
                                                  : crn::tiled_ctas_per_sm_fp32(d->limiter);
-    int kc = crn::choose_kchunk_balanced(d->n_r, ntiles, (long long)std::max(nsm, 1) * std::max(per_sm, 1));
+    int kc = crn::choose_radial_chunk(d->n_r, ntiles, std::max(nsm, 1), per_sm, d->precision == CRN_FP64);
     if (const char* env = std::getenv("CRN_KCHUNK")) {  // tuning override
       const int v = std::atoi(env);
       if (v >= 1) kc = v;

@@ -126,18 +126,11 @@ bool staged_shape_ok(int nt, int np);
 int staged_tiles(int nt, int np);
 int staged_ctas_per_sm_fp32(int limiter);
 
-// Radial planes per CTA of the tiled kernel: the largest chunk count whose
-// CTAs all fit in one wave of `slots` resident CTAs (fewer planes per CTA
-// only add preamble work), at least 4 planes per CTA.
-inline int choose_kchunk(int nr, long long ntiles, long long slots) {
-  if (ntiles <= 0 || slots <= 0 || ntiles >= slots) return nr;
-  long long nch = slots / ntiles;
-  if (nch > nr) nch = nr;
-  int kc = (int)((nr + nch - 1) / nch);
-  return kc < 4 ? (nr < 4 ? nr : 4) : kc;
-}
+// Radial planes per CTA of the tiled kernel (plan.cu): the chunk with the
+// shortest simulated run of its CTAs on `nsm` SMs of `per_sm` resident CTAs.
+int choose_radial_chunk(int nr, long long ntiles, int nsm, int per_sm, bool fp64);
 
-// Radial planes per CTA of the tiled kernel from a makespan model: the CTAs
+// Radial planes per CTA of the TMA-staged kernel from a makespan model: the CTAs
 // of each candidate chunk, in launch order (all tiles of chunk 0, then chunk
 // 1, ...), are list-scheduled onto `slots` resident CTAs, each taking its
 // planes plus `overhead` planes of preamble; the chunk with the shortest

@@ -23,7 +23,7 @@ struct crn_ensemble {
   std::vector<crn_grid*> g;
   int precision = 0, limiter = 0, device = 0;
   int kchunk = 0;          // last chunk set for all members (0: each member's own)
-  std::vector<int> tile;   // per member: tile shape (0: 8 x 32, 1: 16 x 16)
+  std::vector<int> tile;   // per member: tile shape (0: 8 x 32, 1: 16 x 16, 2: 8 x 16, FP64 only)
   std::vector<int> kc;     // per member: radial chunk (0: the member's own)
   unsigned cfg_version = 1;  // bumped whenever tile or kc changes
   int nctas[crn::kEnsTileCount] = {};  // persistent grid per tile shape
@@ -181,14 +181,15 @@ int crn_ensemble_create(crn_grid* const* grids, int32_t n, crn_ensemble** out) {
   }
   crn_ensemble* e = new crn_ensemble();
   e->g.assign(grids, grids + n);
-  e->tile.assign(n, 0);
   e->kc.assign(n, 0);
   e->precision = grids[0]->d.precision;
+  e->tile.assign(n, crn::own_tile(e->precision == CRN_FP64));
   e->limiter = grids[0]->d.limiter;
   e->device = grids[0]->device;
   e->msz = e->precision == CRN_FP64 ? crn::ens_member_bytes_fp64() : crn::ens_member_bytes_fp32();
   e->usz = crn::ens_update_bytes();
   for (int t = 0; t < crn::kEnsTileCount; ++t) {
+    if (t == 2 && e->precision != CRN_FP64) continue;
     const int per_sm = e->precision == CRN_FP64 ? crn::ensemble_ctas_per_sm_fp64(e->limiter, t)
                                                 : crn::ensemble_ctas_per_sm_fp32(e->limiter, t);
     if (per_sm < 1) { free_ens(e); return report(CRN_E_CUDA, "ensemble kernel: no resident CTA fits"); }
@@ -227,7 +228,8 @@ int crn_ensemble_set_kchunk(crn_ensemble* e, int32_t kchunk) {
 int crn_ensemble_set_member_config(crn_ensemble* e, int32_t m, int32_t tile, int32_t kchunk) {
   if (!e) return report(CRN_E_ARG, "ensemble is NULL");
   if (m < 0 || m >= (int)e->g.size()) return report(CRN_E_ARG, "member index out of range");
-  if (tile < 0 || tile >= crn::kEnsTileCount) return report(CRN_E_ARG, "tile must be 0 (8 x 32) or 1 (16 x 16)");
+  if (tile != 0 && tile != 1 && tile != crn::own_tile(e->precision == CRN_FP64))
+    return report(CRN_E_ARG, "tile must be 0 (8 x 32), 1 (16 x 16) or, for FP64 members, 2 (8 x 16)");
   if (kchunk < 0 || kchunk > 4096) return report(CRN_E_ARG, "kchunk must be in [0, 4096]");
   e->tile[m] = tile;
   e->kc[m] = kchunk;
@@ -347,7 +349,7 @@ int crn_ensemble_autotune(crn_ensemble* e, const void* const* U_dev, void* const
     if (cells > big_cells) { big_cells = cells; big_class = (int)c; }
     float best_ms = INFINITY;
     int best_tile = 0, bestk = 0;
-    for (int tile = 0; tile < crn::kEnsTileCount; ++tile)
+    for (int tile = 0; tile < 2; ++tile)
       for (int k : cand) {
         if (k > 0 && k > nr_max) continue;
         for (int m : mem) { e->tile[m] = tile; e->kc[m] = k; }

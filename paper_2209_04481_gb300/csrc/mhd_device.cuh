@@ -65,18 +65,61 @@ struct Shape {
   int64_t ncell;
 };
 
-// (theta, phi) tile shapes of the ensemble kernel, all of 256 threads:
-// tile t has ens_tt(t) x ens_tp(t) columns per CTA
-constexpr int kEnsTileCount = 2;
-__host__ __device__ constexpr int ens_tt(int t) { return t == 0 ? 8 : 16; }
+// (theta, phi) tile shapes of the tiled kernels: tile t has ens_tt(t) x
+// ens_tp(t) columns per CTA.  A grid's own launch takes tile own_tile(): 8 x 32
+// in FP32; 8 x 16 in FP64, whose CTA is bound by the FP64 pipe: half the
+// columns cost 1.5 % more halo work per cell and give twice the CTAs to
+// spread over the SMs.
+constexpr int kEnsTileCount = 3;
+__host__ __device__ constexpr int ens_tt(int t) { return t == 1 ? 16 : 8; }
 __host__ __device__ constexpr int ens_tp(int t) { return t == 0 ? 32 : 16; }
+__host__ __device__ constexpr int own_tile(bool fp64) { return fp64 ? 2 : 0; }
 
+template <class T> __device__ __forceinline__ T fmat(T a, T b, T c);
+template <> __device__ __forceinline__ double fmat<double>(double a, double b, double c) { return fma(a, b, c); }
+template <> __device__ __forceinline__ float fmat<float>(float a, float b, float c) { return fmaf(a, b, c); }
+
+// Reciprocal and square root.  The FP64 pipe runs at 1/64 of the FP32 rate, so
+// their FP64 operations are counted: both start from the approximate PTX
+// instructions (about 20 bits, not on the FP64 pipe) and take one cubic step.
+//   1/x: y0 (1 + e + e^2) with e = 1 - x y0 (Newton's series cut after e^2:
+//        error e^3 ~ 2^-60), 3 operations, within one unit in the last place;
+//        x finite and nonzero.
+//   sqrt x: g (1 + e/2 + 3 e^2/8) with g = x y0, e = 1 - g y0 (the binomial
+//        series of (1 - e)^(-1/2)), 5 operations, within one unit in the last
+//        place; 0 below the normal range, NaN for x < 0.
 template <class T> __device__ __forceinline__ T frcp(T x);
-template <> __device__ __forceinline__ double frcp<double>(double x) { return 1.0 / x; }
+template <> __device__ __forceinline__ double frcp<double>(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
 template <> __device__ __forceinline__ float frcp<float>(float x) { return __fdividef(1.0f, x); }
 template <class T> __device__ __forceinline__ T fsqrt(T x);
-template <> __device__ __forceinline__ double fsqrt<double>(double x) { return sqrt(x); }
+template <> __device__ __forceinline__ double fsqrt<double>(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double g = x * y;
+  const double e = fma(-g, y, 1.0);
+  const double r = fma(g * e, fma(e, 0.375, 0.5), g);
+  return (__double2hiint(x) & 0x7ff00000) == 0 ? 0.0 : r;
+}
 template <> __device__ __forceinline__ float fsqrt<float>(float x) { return sqrtf(x); }
+
+// Comparisons of FP64 values on the integer pipe (an FP64 compare takes a slot
+// of the FP64 pipe): positive doubles order as their bit patterns.
+// positive(x): x > 0; greater(x, y): x > y for y >= 0; both false for a NaN x.
+__device__ __forceinline__ bool positive(float x) { return x > 0.f; }
+__device__ __forceinline__ bool positive(double x) {
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool greater(float x, float y) { return x > y; }
+__device__ __forceinline__ bool greater(double x, double y) {
+  const long long b = __double_as_longlong(x);
+  return b > __double_as_longlong(y) && b <= 0x7ff0000000000000ll;
+}
 
 // ---------------------------------------------------------------------------
 // primitive recovery [Sect. 2.2: E = p/(gamma-1) + rho V^2/2 + B^2/2]
@@ -86,14 +129,14 @@ template <> __device__ __forceinline__ float fsqrt<float>(float x) { return sqrt
 // E - B^2/2 cancels and the internal energy is recomputed in FP64.
 __device__ __forceinline__ void recover(const double (&u)[NV], const Phys<double>& ph,
                                         double (&w)[NV]) {
-  const double ir = 1.0 / u[0];
+  const double ir = frcp(u[0]);
   const double vx = u[1] * ir, vy = u[2] * ir, vz = u[3] * ir;
-  const double ek = 0.5 * (u[1] * vx + u[2] * vy + u[3] * vz);
-  const double eb = 0.5 * (u[4] * u[4] + u[5] * u[5] + u[6] * u[6]);
+  // twice the kinetic and magnetic energy
+  const double t = fma(u[1], vx, fma(u[2], vy, fma(u[3], vz, fma(u[4], u[4], fma(u[5], u[5], u[6] * u[6])))));
   w[0] = u[0];
   w[1] = vx; w[2] = vy; w[3] = vz;
   w[4] = u[4]; w[5] = u[5]; w[6] = u[6];
-  w[7] = ph.gm1 * (u[7] - ek - eb);
+  w[7] = ph.gm1 * fma(-0.5, t, u[7]);
   w[8] = u[8];
 }
 
@@ -222,10 +265,6 @@ __device__ __forceinline__ void outer_ghost(const T (&wi)[NV], T ex, T ey, T ez,
 // ---------------------------------------------------------------------------
 // slope limiters on the two one-sided slopes a (backward), b (forward)
 // ---------------------------------------------------------------------------
-template <class T> __device__ __forceinline__ T fmat(T a, T b, T c);
-template <> __device__ __forceinline__ double fmat<double>(double a, double b, double c) { return fma(a, b, c); }
-template <> __device__ __forceinline__ float fmat<float>(float a, float b, float c) { return fmaf(a, b, c); }
-
 template <int LIM, class T>
 __device__ __forceinline__ T limited_slope(T a, T b, T eps) {
   if (LIM == 0) {  // unlimited central
@@ -253,27 +292,6 @@ __device__ __forceinline__ T limited_slope(T a, T b, T eps) {
   }
 }
 
-// Two limited slopes at once.  FP64 van Albada shares one division between
-// them, 1/(d1 d2) times d2 and d1 (three multiplies and one IEEE division in
-// place of two divisions on the slow FP64 pipe); d >= 2 eps > 0 and the
-// slopes' squares keep d1 d2 far inside the binary64 range.  Every other case
-// is two calls of limited_slope.
-template <int LIM, class T>
-__device__ __forceinline__ void limited_slope2(T a1, T b1, T a2, T b2, T eps, T& s1, T& s2) {
-  if (LIM == 2 && sizeof(T) == 8) {
-    const T n1 = (a1 + b1) * fmat(a1, b1, eps);
-    const T d1 = fmat(a1, a1, fmat(b1, b1, (T)2 * eps));
-    const T n2 = (a2 + b2) * fmat(a2, b2, eps);
-    const T d2 = fmat(a2, a2, fmat(b2, b2, (T)2 * eps));
-    const T inv = frcp(d1 * d2);
-    s1 = n1 * (inv * d2);
-    s2 = n2 * (inv * d1);
-  } else {
-    s1 = limited_slope<LIM>(a1, b1, eps);
-    s2 = limited_slope<LIM>(a2, b2, eps);
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Rusanov + GLM face flux through the unit normal n, times the face area.
 // F* = (F(W_L) + F(W_R))/2 - lambda (U_R - U_L)/2,
@@ -281,66 +299,151 @@ __device__ __forceinline__ void limited_slope2(T a1, T b1, T a2, T b2, T eps, T&
 // F_rho = rho u_n, F_m = rho V u_n + (p + B^2/2) n - B B_n,
 // F_B = u_n B - B_n V + psi n, F_E = (E + p + B^2/2) u_n - B_n (V.B),
 // F_psi = c_h^2 B_n.
+//
+// FP64: the flux is the longest chain of the residual (three per cell) on the
+// slowest pipe, so its operations are counted: h = |S|/2 is multiplied into
+// u_n, B_n and rho u_n once per side instead of into each of the nine sums, and
+// the pressure and GLM gradient terms of both sides are added before they meet
+// the normal (159 operations against about 200; every FMA explicit).  FP32
+// keeps the sums by side: there the regrouping saved 3 % and moved the momentum
+// of the polar cells, whose opposite faces nearly cancel, by 1e-7 per step.
 // ---------------------------------------------------------------------------
 template <class T>
 struct Side {
-  T un, bn, pt, en, sp;
+  T un, bn, pt, en, vb, sp;
 };
 
-template <class T>
-__device__ __forceinline__ Side<T> side_terms(const T (&w)[NV], T nx, T ny, T nz,
-                                               const Phys<T>& ph) {
-  Side<T> s;
-  const T ir = frcp(w[0]);
-  s.un = w[1] * nx + w[2] * ny + w[3] * nz;
-  s.bn = w[4] * nx + w[5] * ny + w[6] * nz;
-  const T b2 = w[4] * w[4] + w[5] * w[5] + w[6] * w[6];
-  const T v2 = w[1] * w[1] + w[2] * w[2] + w[3] * w[3];
-  s.pt = w[7] + (T)0.5 * b2;
-  s.en = w[7] * ph.igm1 + (T)0.5 * (w[0] * v2 + b2);
-  const T a2 = ph.gamma * w[7] * ir;
-  const T sum = a2 + b2 * ir;
-  T disc = sum * sum - (T)4 * a2 * s.bn * s.bn * ir;
-  disc = disc > (T)0 ? disc : (T)0;
-  const T cf = fsqrt((T)0.5 * (sum + fsqrt(disc)));
+// NZ: the normal has a z component (phi faces have none)
+template <bool NZ>
+__device__ __forceinline__ Side<float> side_terms(const float (&w)[NV], float nx, float ny, float nz,
+                                                  const Phys<float>& ph) {
+  Side<float> s;
+  const float ir = frcp(w[0]);
+  s.un = w[1] * nx + w[2] * ny;
+  s.bn = w[4] * nx + w[5] * ny;
+  if (NZ) {
+    s.un += w[3] * nz;
+    s.bn += w[6] * nz;
+  }
+  const float b2 = w[4] * w[4] + w[5] * w[5] + w[6] * w[6];
+  const float v2 = w[1] * w[1] + w[2] * w[2] + w[3] * w[3];
+  s.vb = w[1] * w[4] + w[2] * w[5] + w[3] * w[6];
+  s.pt = w[7] + 0.5f * b2;
+  s.en = w[7] * ph.igm1 + 0.5f * (w[0] * v2 + b2);
+  const float a2 = ph.gamma * w[7] * ir;
+  const float sum = a2 + b2 * ir;
+  float disc = sum * sum - 4.f * a2 * s.bn * s.bn * ir;
+  disc = disc > 0.f ? disc : 0.f;
+  const float cf = fsqrt(0.5f * (sum + fsqrt(disc)));
+  s.sp = fabsf(s.un) + cf;
+  return s;
+}
+
+template <bool NZ>
+__device__ __forceinline__ double dot_n(const double* w, double nx, double ny, double nz) {
+  return NZ ? fma(w[0], nx, fma(w[1], ny, w[2] * nz)) : fma(w[0], nx, w[1] * ny);
+}
+__device__ __forceinline__ double dot3(const double* a, const double* b) {
+  return fma(a[0], b[0], fma(a[1], b[1], a[2] * b[2]));
+}
+
+template <bool NZ>
+__device__ __forceinline__ Side<double> side_terms(const double (&w)[NV], double nx, double ny, double nz,
+                                                   const Phys<double>& ph) {
+  Side<double> s;
+  s.un = dot_n<NZ>(w + 1, nx, ny, nz);
+  s.bn = dot_n<NZ>(w + 4, nx, ny, nz);
+  s.vb = dot3(w + 1, w + 4);
+  const double b2 = dot3(w + 4, w + 4);
+  const double v2 = dot3(w + 1, w + 1);
+  s.pt = fma(0.5, b2, w[7]);
+  s.en = fma(0.5, fma(w[0], v2, b2), w[7] * ph.igm1);
+  // fast speed: c_f^2 = (q + sqrt(q^2 - 4 a^2 B_n^2 / rho)) / 2, q = a^2 + B^2 / rho
+  const double ir = frcp(w[0]);
+  const double a2 = (ph.gamma * w[7]) * ir;
+  const double q = fma(b2, ir, a2);
+  const double disc = fma(-4.0 * (a2 * ir), s.bn * s.bn, q * q);
+  const double cf = fsqrt(0.5 * (q + fsqrt(positive(disc) ? disc : 0.0)));
   s.sp = fabs(s.un) + cf;
   return s;
 }
 
-template <class T>
-__device__ __forceinline__ void rusanov(const T (&wl)[NV], const T (&wr)[NV], T nx, T ny, T nz,
-                                        T area, const Phys<T>& ph, T (&f)[NV], T& lam_area) {
-  const Side<T> L = side_terms(wl, nx, ny, nz, ph);
-  const Side<T> R = side_terms(wr, nx, ny, nz, ph);
-  T lam = L.sp > R.sp ? L.sp : R.sp;
+template <bool NZ = true>
+__device__ __forceinline__ void rusanov(const float (&wl)[NV], const float (&wr)[NV], float nx, float ny,
+                                        float nz, float area, const Phys<float>& ph, float (&f)[NV],
+                                        float& lam_area) {
+  const Side<float> L = side_terms<NZ>(wl, nx, ny, nz, ph);
+  const Side<float> R = side_terms<NZ>(wr, nx, ny, nz, ph);
+  float lam = L.sp > R.sp ? L.sp : R.sp;
   lam = lam > ph.ch ? lam : ph.ch;
-  const T h = (T)0.5 * area;
+  const float h = 0.5f * area;
   lam_area = lam * area;
-  const T d = (T)0.5 * lam_area;  // halving is exact: the same value as (lam / 2) area
+  const float d = 0.5f * lam_area;  // halving is exact: the same value as (lam / 2) area
+  const float n[3] = {nx, ny, nz};
   // mass
-  const T ml = wl[0] * L.un, mr = wr[0] * R.un;
+  const float ml = wl[0] * L.un, mr = wr[0] * R.un;
   f[0] = h * (ml + mr) - d * (wr[0] - wl[0]);
-  // momentum
-  f[1] = h * ((ml * wl[1] + L.pt * nx - wl[4] * L.bn) + (mr * wr[1] + R.pt * nx - wr[4] * R.bn))
-         - d * (wr[0] * wr[1] - wl[0] * wl[1]);
-  f[2] = h * ((ml * wl[2] + L.pt * ny - wl[5] * L.bn) + (mr * wr[2] + R.pt * ny - wr[5] * R.bn))
-         - d * (wr[0] * wr[2] - wl[0] * wl[2]);
-  f[3] = h * ((ml * wl[3] + L.pt * nz - wl[6] * L.bn) + (mr * wr[3] + R.pt * nz - wr[6] * R.bn))
-         - d * (wr[0] * wr[3] - wl[0] * wl[3]);
-  // induction with the GLM gradient term
-  f[4] = h * ((L.un * wl[4] - L.bn * wl[1] + wl[8] * nx) + (R.un * wr[4] - R.bn * wr[1] + wr[8] * nx))
-         - d * (wr[4] - wl[4]);
-  f[5] = h * ((L.un * wl[5] - L.bn * wl[2] + wl[8] * ny) + (R.un * wr[5] - R.bn * wr[2] + wr[8] * ny))
-         - d * (wr[5] - wl[5]);
-  f[6] = h * ((L.un * wl[6] - L.bn * wl[3] + wl[8] * nz) + (R.un * wr[6] - R.bn * wr[3] + wr[8] * nz))
-         - d * (wr[6] - wl[6]);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const bool on = NZ || c < 2;
+    // momentum
+    float a = ml * wl[1 + c], b = mr * wr[1 + c];
+    if (on) { a += L.pt * n[c]; b += R.pt * n[c]; }
+    a -= wl[4 + c] * L.bn;
+    b -= wr[4 + c] * R.bn;
+    f[1 + c] = h * (a + b) - d * (wr[0] * wr[1 + c] - wl[0] * wl[1 + c]);
+    // induction with the GLM gradient term
+    float p = L.un * wl[4 + c] - L.bn * wl[1 + c], q = R.un * wr[4 + c] - R.bn * wr[1 + c];
+    if (on) { p += wl[8] * n[c]; q += wr[8] * n[c]; }
+    f[4 + c] = h * (p + q) - d * (wr[4 + c] - wl[4 + c]);
+  }
   // energy
-  const T vbl = wl[1] * wl[4] + wl[2] * wl[5] + wl[3] * wl[6];
-  const T vbr = wr[1] * wr[4] + wr[2] * wr[5] + wr[3] * wr[6];
-  f[7] = h * (((L.en + L.pt) * L.un - L.bn * vbl) + ((R.en + R.pt) * R.un - R.bn * vbr))
+  f[7] = h * (((L.en + L.pt) * L.un - L.bn * L.vb) + ((R.en + R.pt) * R.un - R.bn * R.vb))
          - d * (R.en - L.en);
   // cleaning scalar
   f[8] = h * (ph.ch2 * (L.bn + R.bn)) - d * (wr[8] - wl[8]);
+}
+
+template <bool NZ = true>
+__device__ __forceinline__ void rusanov(const double (&wl)[NV], const double (&wr)[NV], double nx, double ny,
+                                        double nz, double area, const Phys<double>& ph, double (&f)[NV],
+                                        double& lam_area) {
+  const Side<double> L = side_terms<NZ>(wl, nx, ny, nz, ph);
+  const Side<double> R = side_terms<NZ>(wr, nx, ny, nz, ph);
+  double lam = greater(L.sp, R.sp) ? L.sp : R.sp;
+  lam = greater(lam, ph.ch) ? lam : ph.ch;
+  const double h = 0.5 * area;
+  lam_area = lam * area;
+  const double d = lam * h;
+  const double ul = h * L.un, ur = h * R.un, bl = h * L.bn, br = h * R.bn;
+  const double ml = wl[0] * ul, mr = wr[0] * ur;
+  const double pt = h * (L.pt + R.pt), ps = h * (wl[8] + wr[8]);
+  const double n[3] = {nx, ny, nz};
+  // mass
+  f[0] = fma(-d, wr[0] - wl[0], ml + mr);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const bool on = NZ || c < 2;
+    // momentum
+    double a = fma(mr, wr[1 + c], ml * wl[1 + c]);
+    if (on) a = fma(pt, n[c], a);
+    a = fma(-bl, wl[4 + c], a);
+    a = fma(-br, wr[4 + c], a);
+    f[1 + c] = fma(-d, fma(wr[0], wr[1 + c], -(wl[0] * wl[1 + c])), a);
+    // induction with the GLM gradient term
+    double e = fma(ur, wr[4 + c], ul * wl[4 + c]);
+    e = fma(-bl, wl[1 + c], e);
+    e = fma(-br, wr[1 + c], e);
+    if (on) e = fma(ps, n[c], e);
+    f[4 + c] = fma(-d, wr[4 + c] - wl[4 + c], e);
+  }
+  // energy
+  double e = fma(R.en + R.pt, ur, (L.en + L.pt) * ul);
+  e = fma(-bl, L.vb, e);
+  e = fma(-br, R.vb, e);
+  f[7] = fma(-d, R.en - L.en, e);
+  // cleaning scalar
+  f[8] = fma(-d, wr[8] - wl[8], ph.ch2 * (bl + br));
 }
 
 // across-pole / periodic mapping of a (possibly out-of-range) column (j, i):

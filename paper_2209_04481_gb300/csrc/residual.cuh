@@ -6,13 +6,13 @@
 //
 //  * residual_tiled   -- the production kernel.  A CTA owns a TT x TP block of
 //    (theta, phi) columns and marches outwards in r over a chunk of planes.
-//    Each plane (cells + a 2-cell theta/phi halo) is loaded once, its
-//    primitives recovered once and kept in a 4-plane shared-memory ring; every
-//    face flux of the tile is computed once per plane into shared memory and
-//    gathered by the two cells it separates (no atomics); the r-face flux is
-//    double-buffered across planes.  Residual norms and the step bound are
-//    reduced per thread, per warp (shuffles), per CTA, and across CTAs by the
-//    last CTA to finish (fixed order, bitwise reproducible).
+//    Each cell (and a 2-cell theta/phi halo) is loaded and its primitives
+//    recovered once per tile; a thread keeps its own column in registers, the
+//    neighbours see the plane in shared memory.  Every face flux of the tile is
+//    computed once and gathered by the two cells it separates (no atomics).
+//    Residual norms and the step bound are reduced per thread, per warp
+//    (shuffles), per CTA, and across CTAs by the last CTA to finish (fixed
+//    order, bitwise reproducible).
 //  * residual_cellwise -- a deliberately simple reference kernel: one thread
 //    per cell re-evaluates all six of its faces from global memory.
 #pragma once
@@ -68,39 +68,40 @@ __device__ __forceinline__ void flag_bad(const Reduce& red, long long cell) {
   atomicMin(red.err_cell, (unsigned long long)cell);
 }
 
-// Block + grid reduction of 9 sums of squares and one minimum.  Every thread
-// of every CTA calls it once at the end of the kernel.
-// WARP_DONE: the caller has already reduced within each warp (lane 0 holds
-// the warp's sums, every lane the warp's minimum).
-template <int NTHREADS, bool WARP_DONE = false>
-__device__ void reduce_and_finalize_at(const double (&sum)[NV], double dtmin, const Reduce& red,
+// the smaller of two positive doubles (or +inf), on the integer pipe
+__device__ __forceinline__ double min_positive(double a, double b) {
+  return __double_as_longlong(b) < __double_as_longlong(a) ? b : a;
+}
+
+// Block + grid reduction of 9 sums of squares and one minimum from the warps'
+// values (S = float or double; lane 0 of every warp holds its warp's).  Every
+// thread of every CTA calls it once at the end of the kernel.  The FP64 adds
+// of one warp take 16 clocks of the SM's FP64 pipe however few lanes are
+// active, and the last CTA's are the tail of the whole launch, so they are
+// packed: ten threads add and convert the block's warp sums, and the last CTA
+// reads the partials 16 lanes to a row of ten (320 rows: 160 warp adds, where
+// one row per thread with a shuffle tree per quantity took 540).
+template <int NTHREADS, class S>
+__device__ void reduce_and_finalize_at(const S (&sum)[NV], S dtmin, const Reduce& red,
                                        double* scratch /* >= (NTHREADS/32) * RED_STRIDE doubles */,
                                        int bid, int nblocks) {
   constexpr int NW = NTHREADS / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double v[NV + 1];
-#pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = sum[q];
-  v[NV] = dtmin;
-  if (!WARP_DONE) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-      for (int q = 0; q < NV; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-      v[NV] = fmin(v[NV], __shfl_xor_sync(0xffffffffu, v[NV], off));
-    }
-  }
+  S* sc = reinterpret_cast<S*>(scratch);
   __syncthreads();  // scratch may alias buffers still in use
   if (lane == 0) {
 #pragma unroll
-    for (int q = 0; q <= NV; ++q) scratch[warp * RED_STRIDE + q] = v[q];
+    for (int q = 0; q < NV; ++q) sc[warp * RED_STRIDE + q] = sum[q];
+    sc[warp * RED_STRIDE + NV] = dtmin;
   }
   __syncthreads();
   if (threadIdx.x <= NV) {
     const int q = threadIdx.x;
-    double a = scratch[q];
-    for (int w = 1; w < NW; ++w)
-      a = (q < NV) ? a + scratch[w * RED_STRIDE + q] : fmin(a, scratch[w * RED_STRIDE + q]);
+    double a = (double)sc[q];
+    for (int w = 1; w < NW; ++w) {
+      const double x = (double)sc[w * RED_STRIDE + q];
+      a = q < NV ? a + x : min_positive(a, x);
+    }
     red.partials[(size_t)bid * RED_STRIDE + q] = a;
   }
   __shared__ unsigned int s_last;
@@ -111,33 +112,28 @@ __device__ void reduce_and_finalize_at(const double (&sum)[NV], double dtmin, co
   if (!s_last) return;
   __threadfence();
   // last CTA: fixed-order reduction of all partials
-  double acc[NV + 1];
-#pragma unroll
-  for (int q = 0; q < NV; ++q) acc[q] = 0.0;
-  acc[NV] = INFINITY;
-  for (int b = threadIdx.x; b < nblocks; b += NTHREADS) {
-    const volatile double* p = red.partials + (size_t)b * RED_STRIDE;
-#pragma unroll
-    for (int q = 0; q < NV; ++q) acc[q] += p[q];
-    acc[NV] = fmin(acc[NV], p[NV]);
+  constexpr int NS = NTHREADS / RED_STRIDE;
+  const int q = threadIdx.x % RED_STRIDE;
+  double acc = q < NV ? 0.0 : INFINITY;
+  if (q <= NV) {
+#pragma unroll 4
+    for (int b = threadIdx.x / RED_STRIDE; b < nblocks; b += NS) {
+      const double x = __ldcg(red.partials + (size_t)b * RED_STRIDE + q);
+      acc = q < NV ? acc + x : min_positive(acc, x);
+    }
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], off);
-    acc[NV] = fmin(acc[NV], __shfl_xor_sync(0xffffffffu, acc[NV], off));
+  {
+    const double x = __shfl_xor_sync(0xffffffffu, acc, RED_STRIDE);
+    acc = q < NV ? acc + x : min_positive(acc, x);
   }
-  __syncthreads();
-  if (lane == 0) {
-#pragma unroll
-    for (int q = 0; q <= NV; ++q) scratch[warp * RED_STRIDE + q] = acc[q];
-  }
+  if (lane <= NV) scratch[warp * RED_STRIDE + lane] = acc;
   __syncthreads();
   if (threadIdx.x <= NV) {
-    const int q = threadIdx.x;
     double a = scratch[q];
-    for (int w = 1; w < NW; ++w)
-      a = (q < NV) ? a + scratch[w * RED_STRIDE + q] : fmin(a, scratch[w * RED_STRIDE + q]);
+    for (int w = 1; w < NW; ++w) {
+      const double x = scratch[w * RED_STRIDE + q];
+      a = q < NV ? a + x : min_positive(a, x);
+    }
     if (red.log_out) {
       if (q < NV) red.log_out[q] = log10(sqrt(a));
     } else if (q < NV) {
@@ -152,12 +148,18 @@ __device__ void reduce_and_finalize_at(const double (&sum)[NV], double dtmin, co
   if (threadIdx.x == 0) *red.counter = 0u;
 }
 
-// the same with the block id and count of the launch grid
-template <int NTHREADS, bool WARP_DONE = false>
-__device__ __forceinline__ void reduce_and_finalize(const double (&sum)[NV], double dtmin, const Reduce& red,
+// the same from per-thread values, for the block id and count of the launch grid
+template <int NTHREADS>
+__device__ __forceinline__ void reduce_and_finalize(double (&sum)[NV], double dtmin, const Reduce& red,
                                                     double* scratch) {
-  reduce_and_finalize_at<NTHREADS, WARP_DONE>(sum, dtmin, red, scratch, blockIdx.y * gridDim.x + blockIdx.x,
-                                              gridDim.x * gridDim.y);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) sum[v] += __shfl_xor_sync(0xffffffffu, sum[v], off);
+    dtmin = min_positive(dtmin, __shfl_xor_sync(0xffffffffu, dtmin, off));
+  }
+  reduce_and_finalize_at<NTHREADS>(sum, dtmin, red, scratch, blockIdx.y * gridDim.x + blockIdx.x,
+                                   gridDim.x * gridDim.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -370,43 +372,67 @@ cell_efield_kernel(int64_t ncell, const T* __restrict__ U, double* __restrict__ 
   }
 }
 
+// whether the squares of a cell's residuals and their sum are finite
+__device__ __forceinline__ bool squares_finite(const float (&r)[NV]) {
+  float s = 0.f;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) s = fmaf(r[v], r[v], s);
+  return fabsf(s) < INFINITY;
+}
+// FP64: on the integer pipe, |r| < 2^511 from the exponents
+__device__ __forceinline__ bool squares_finite(const double (&r)[NV]) {
+  int m = 0;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) m = max(m, __double2hiint(r[v]) & 0x7fffffff);
+  return m < 0x5fe00000;
+}
+
 // ---------------------------------------------------------------------------
 // production kernel: radial marching over a (theta, phi) tile
 // ---------------------------------------------------------------------------
-// Thread (jj, ii) owns column (j0 + jj, i0 + ii) of the tile.  Per plane k:
-//   A  the prefetched plane k + 2 (own cell + at most one halo cell per thread)
-//      is recovered to primitives and stored in a 3-plane ring (k, k+1, k+2)
-//   B  the loads of plane k + 3 are issued (they complete during B-E); every
-//      cell of plane k gets its theta and phi slopes once, stored as the lower
-//      and upper face values; the own column gets the r slope of plane k + 1
-//      (registers)
-//   C  every theta and phi face of plane k is evaluated once (Rusanov + GLM)
-//      into shared memory; the r face k + 1/2 stays in registers
-//   E  each cell gathers its six faces, adds gravity and writes R
-// The r face k - 1/2 and the upper r face value of plane k + 1 are carried in
-// registers from one plane to the next.
+// Thread (jj, ii) owns column (j0 + jj, i0 + ii) of the tile and keeps the
+// primitives of planes k and k + 1 of it in registers; shared memory holds the
+// halo'd plane k.  Two phases per plane, a barrier after each:
+//   1  gather the six faces of the cell of plane k - 1 into R; the theta and
+//      phi slopes of plane k: the cell's lower face values stay in registers,
+//      its upper ones go to the face above it; the halo cells' slopes are
+//      spread over all threads, three variables of one cell each
+//   2  the cell's lower theta and phi face (Rusanov + GLM) into shared
+//      memory; the faces past the tile's last row and column on its last
+//      warps; the r slope of plane k + 1 and the r face k + 1/2 in registers;
+//      plane k + 1 replaces plane k in shared memory; the loads of the own
+//      cell of plane k + 3 and the halo of plane k + 2 are issued
+//
+// FP32 is bound by instruction issue at 16 warps per SM (128 registers): 61 %
+// of the slots at 1575 instructions per cell, 920 of them on the FMA pipe.
+// 128 x 64 x 128: 77 us, against 87 us for three phases per plane with a ring
+// of three planes, both face values in shared memory and a global load per
+// radial factor (55 % of the slots, 1660 instructions).  FP64 is bound by the
+// FP64 pipe: about 1020 operations per cell, 2.10 ms (2.65 ms with 1208).
 template <int TT, int TP>
 struct TileDims {
   static constexpr int NT = TT * TP;                            // threads = own columns
   static constexpr int HT = TT + 4, HP = TP + 4, HC = HT * HP;  // halo'd plane
-  static constexpr int NHALO = HC - NT;                         // halo positions
+  static constexpr int NHALO = 4 * (TT + TP);                   // halo positions (a cross: no corners)
   static constexpr int NTV = (TT + 1) * TP;                     // theta faces (rows 0..TT)
   static constexpr int NPV = TT * (TP + 1);                     // phi faces (cols 0..TP)
+  static constexpr int NFA = NTV + NPV;                         // both, theta faces first
   static constexpr int NF = NV + 1;                             // 9 fluxes + lambda |S|
-  static constexpr int NEXTRA_V = 2 * TP + 2 * TT;              // halo cells needing face values
-  static constexpr int NEXTRA_F = TP + TT;                      // faces beyond the own lower faces
+  static constexpr int NEXTRA_V = 2 * (TT + TP);                // halo cells needing a face value
+  static constexpr int NEXTRA_F = TT + TP;                      // faces beyond the own lower faces
   // per-CTA geometry staged once: theta-face normals, phi-face normals, own
   // r-face normals, own radial unit vectors, theta factors of the areas/volumes
   static constexpr int NGEO = 3 * NTV + 2 * (TP + 1) + 6 * NT + (TT + 1) + 2 * TT;
+  static constexpr int NRAD = 8;                                // radial factors of a plane, three planes held
   template <class T>
   static constexpr size_t smem_bytes() {
-    return sizeof(T) * ((size_t)3 * NV * HC + (size_t)2 * NV * (NTV + NPV) + (size_t)NGEO);
+    return sizeof(T) * ((size_t)NV * HC + (size_t)NV * NFA + (size_t)NF * NFA + (size_t)NV * NEXTRA_F +
+                        (size_t)NV * NHALO + (size_t)3 * NRAD + (size_t)NGEO);
   }
   // halo position h in [0, NHALO) -> halo'd (row, col)
   __device__ static void halo_rc(int h, int& row, int& col) {
-    if (h < 2 * HP) { row = h / HP; col = h % HP; }
-    else if (h < 4 * HP) { h -= 2 * HP; row = TT + 2 + h / HP; col = h % HP; }
-    else { h -= 4 * HP; row = 2 + h / 4; const int c = h % 4; col = c < 2 ? c : TP + c; }
+    if (h < 4 * TP) { const int r = h / TP; row = r < 2 ? r : TT + r; col = 2 + h % TP; }
+    else { h -= 4 * TP; row = 2 + h / 4; const int c = h % 4; col = c < 2 ? c : TP + c; }
   }
 };
 
@@ -416,9 +442,23 @@ __device__ __forceinline__ void load_raw(const T* __restrict__ src, int64_t N, i
   for (int v = 0; v < NV; ++v) u[v] = __ldg(src + v * N + c);
 }
 
-// resident CTAs per SM the register allocation is sized for: two FP32 CTAs
-// (16 warps); FP64 CTAs are limited to one by their shared memory anyway
-template <class T> struct MinCtas { static constexpr int value = sizeof(T) == 4 ? 2 : 1; };
+// asynchronous copy of one element from global to shared memory, the wait for
+// all of the thread's copies
+template <class T>
+__device__ __forceinline__ void copy_async(T* dst, const T* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  if constexpr (sizeof(T) == 4)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// resident CTAs per SM the register allocation is sized for: 16 FP32 warps;
+// 8 FP64 warps (the FP64 pipe needs no more, and their state is twice as wide)
+template <class T, int NT> struct MinCtas { static constexpr int value = (sizeof(T) == 4 ? 512 : 256) / NT; };
 
 // One work item of the tiled residual: tile `tile` (row-major over the
 // (theta, phi) tiles) and radial chunk `chunk` of one grid; `bid` / `nblocks`
@@ -429,23 +469,18 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
                                            T* __restrict__ R, const Reduce& red, int kchunk, int tile,
                                            int chunk, int bid, int nblocks, unsigned char* smem_raw) {
   using D = TileDims<TT, TP>;
-  constexpr int NT = D::NT, HP = D::HP, HC = D::HC, NTV = D::NTV, NPV = D::NPV, NF = D::NF;
+  constexpr int NT = D::NT, HP = D::HP, HC = D::HC, NTV = D::NTV, NFA = D::NFA, NF = D::NF;
+  constexpr int NX = D::NEXTRA_V, NXF = D::NEXTRA_F;
+  static_assert(D::NRAD <= D::NHALO, "the halo threads wait for the radial factors too");
   static_assert(D::NHALO <= NT, "each thread stores at most one halo position");
-  static_assert(D::NEXTRA_F <= NT && NT % 32 == 0, "tile shape");
-  T* ring = reinterpret_cast<T*>(smem_raw);  // [3][NV][HC]   primitives of planes k..k+2
-  T* tvu = ring + 3 * NV * HC;               // [NV][NTV]     theta: upper value of the row below face f
-  T* tvl = tvu + NV * NTV;                   // [NV][NTV]     theta: lower value of the row above face f
-  T* pvu = tvl + NV * NTV;                   // [NV][NPV]     phi: upper value of the col left of face f
-  T* pvl = pvu + NV * NPV;                   // [NV][NPV]     phi: lower value of the col right of face f
-  // face fluxes x area overwrite the face values they were computed from (each
-  // face is read and written by one thread): flux v of theta face f in
-  // tvu[v][f], its lambda x area in tvl[0][f]; likewise phi faces in pvu / pvl
-  T* ftb = tvu;
-  T* fpb = pvu;
-  T* ftl = tvl;                              // lambda x area of theta faces
-  T* fpl = pvl;                              // lambda x area of phi faces
-  T* gs = pvl + NV * NPV;                    // per-CTA geometry
-  T* s_nth = gs;                             // [3][NTV]
+  static_assert(NXF <= NT && NT % 32 == 0, "tile shape");
+  T* sp = reinterpret_cast<T*>(smem_raw);    // [NV][HC]   primitives of plane k
+  T* uv = sp + NV * HC;                      // [NV][NFA]  L state of each face (upper value of the cell below)
+  T* fx = uv + NV * NFA;                     // [NF][NFA]  flux x area of each face, lambda x area last
+  T* xr = fx + NF * NFA;                     // [NV][NXF]  R states of the faces past the last row / column
+  T* hr = xr + NV * NXF;                     // [NV][NHALO] raw halo cells of plane k + 1
+  T* s_rad = hr + NV * D::NHALO;             // [3][NRAD] radial factors of planes k .. k + 2
+  T* s_nth = s_rad + 3 * D::NRAD;            // [3][NTV]
   T* s_nph = s_nth + 3 * NTV;                // [2][TP + 1]
   T* s_nr = s_nph + 2 * (TP + 1);            // [3][NT]
   T* s_rh = s_nr + 3 * NT;                   // [3][NT]
@@ -465,167 +500,141 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
   const bool own = jo < nt && io < np;
   const int hown = (jj + 2) * HP + (ii + 2);
   // global column of the own position and of this thread's halo position
-  int64_t c_own, c_halo = 0;
+  int c_own, c_halo = 0;
   int h_halo = -1;
   {
     int j = jo, i = io;
     map_column(j, i, nt, np);
-    c_own = (int64_t)j * np + i;
+    c_own = j * np + i;
     if (tid < D::NHALO) {
       int row, col;
       D::halo_rc(tid, row, col);
       h_halo = row * HP + col;
       int jh = j0 - 2 + row, ih = i0 - 2 + col;
       map_column(jh, ih, nt, np);
-      c_halo = (int64_t)jh * np + ih;
+      c_halo = jh * np + ih;
     }
   }
-  const int64_t ocol = own ? (int64_t)jo * np + io : 0;
+  const int ocol = own ? c_own : 0;
   const T one = (T)1, half = (T)0.5;
-  {
-    const int64_t ts = (int64_t)(nt + 1) * np;
-    for (int q = tid; q < NTV; q += NT) {
-      const int f = q / TP, col = q % TP;
-      const int jf = min(j0 + f, nt), ic = min(i0 + col, np - 1);
-      const int64_t fc = (int64_t)jf * np + ic;
-      s_nth[q] = g.nth[fc];
-      s_nth[NTV + q] = g.nth[ts + fc];
-      s_nth[2 * NTV + q] = g.nth[2 * ts + fc];
-    }
-    for (int q = tid; q <= TP; q += NT) {
-      int ic = i0 + q;
-      ic = ic >= np ? ic - np : ic;
-      s_nph[q] = g.nph[ic];
-      s_nph[TP + 1 + q] = g.nph[np + ic];
-    }
-    s_nr[tid] = g.nr[ocol];
-    s_nr[NT + tid] = g.nr[cs + ocol];
-    s_nr[2 * NT + tid] = g.nr[2 * cs + ocol];
-    s_rh[tid] = g.rhat[c_own];
-    s_rh[NT + tid] = g.rhat[cs + c_own];
-    s_rh[2 * NT + tid] = g.rhat[2 * cs + c_own];
-    if (tid <= TT) s_at[tid] = g.at[min(j0 + tid, nt)];
-    if (tid < TT) {
-      s_ar[tid] = g.ar[min(j0 + tid, nt - 1)];
-      s_av[tid] = g.av[min(j0 + tid, nt - 1)];
-    }
+
+  // ---------------- preamble: every load of the chunk's first planes at once
+  T wc[NV], w1[NV];   // primitives of planes k and k + 1 of the own column
+  T rL[NV];           // L state of r face k + 1/2 (upper r value of plane k)
+  T frl[NF];          // flux x area of r face k - 1/2, lambda x area last
+  T pf_own[NV];       // raw own cell of plane k + 2
+  // radial factor tid of plane p: r_b, r_v and gravity of p, face area factor of
+  // its upper face, slope and face distances of plane p + 1.  They come in with
+  // the halo cells, two planes ahead: a global load where they are used would
+  // stall every warp just after a barrier.
+  const T* rad_src = nullptr;
+  if (tid < D::NRAD) {
+    const T* const src[D::NRAD] = {g.rb, g.rv, g.grav, g.ra + 1, g.inv_dm, g.inv_dp, g.hm, g.hp};
+#pragma unroll
+    for (int q = 0; q < D::NRAD; ++q) rad_src = tid == q ? src[q] : rad_src;
   }
-
-  auto slot = [&](int p) -> T* { return ring + ((p + 3) % 3) * (NV * HC); };
-
-  // raw state of the prefetched plane (own position, halo position)
-  T pf_own[NV], pf_halo[NV];
-  auto prefetch = [&](int p) {
-    const T* src = U + (int64_t)p * cs;
-    load_raw(src, N, c_own, pf_own);
-    if (h_halo >= 0) load_raw(src, N, c_halo, pf_halo);
+  auto rad_at = [&](int p) -> const T* { return rad_src + (tid < 4 ? p : min(p + 1, nr - 1)); };
+  auto rad_slot = [&](int p) -> T* { return s_rad + (p % 3) * D::NRAD; };
+  // the halo cell of plane p into its slot of hr, read back by the same thread:
+  // held in registers its nine values would spill
+  auto fetch_halo = [&](int p) {
+    const T* src = U + (int64_t)p * cs + c_halo;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) copy_async(hr + v * D::NHALO + tid, src + v * N);
   };
-  auto store_prefetched = [&](int p) {
-    T* dst = slot(p);
-    T w[NV];
-    recover(pf_own, ph, w);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) dst[v * HC + hown] = w[v];
-    if (h_halo >= 0) {
-      recover(pf_halo, ph, w);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) dst[v * HC + h_halo] = w[v];
-    }
-  };
-  // outer ghost plane nr from plane nr - 1, own and halo positions
-  auto outer_plane = [&]() {
-    const T* src = slot(nr - 1);
-    T* dst = slot(nr);
-    for (int pass = 0; pass < 2; ++pass) {
-      const int h = pass == 0 ? hown : h_halo;
-      if (h < 0) continue;
-      const int64_t c = pass == 0 ? c_own : c_halo;
-      T wi[NV], wg[NV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) wi[v] = src[v * HC + h];
-      outer_ghost(wi, g.rhat[c], g.rhat[cs + c], g.rhat[2 * cs + c], ph, wg);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) dst[v * HC + h] = wg[v];
-    }
-  };
-  auto read_own = [&](const T* pl, T (&w)[NV]) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) w[v] = pl[v * HC + hown];
-  };
-  // r slope of plane p for the own column from planes p-1, p, p+1
-  auto r_values = [&](int p, const T (&wm)[NV], const T (&w0)[NV], const T (&wp)[NV], T (&lo)[NV],
-                      T (&up)[NV]) {
-    const T im = g.inv_dm[p], ip = g.inv_dp[p], hm = g.hm[p], hp = g.hp[p];
-    constexpr int VSTEP = sizeof(T) == 8 ? 2 : 1;  // FP64: slopes in pairs
-#pragma unroll
-    for (int v = 0; v < NV; v += VSTEP) {
-      if (VSTEP == 2 && v + 1 < NV) {
-        T s, s1;
-        limited_slope2<LIM>((w0[v] - wm[v]) * im, (wp[v] - w0[v]) * ip, (w0[v + 1] - wm[v + 1]) * im,
-                            (wp[v + 1] - w0[v + 1]) * ip, ph.eps, s, s1);
-        lo[v] = fmat(-s, hm, w0[v]);
-        up[v] = fmat(s, hp, w0[v]);
-        lo[v + 1] = fmat(-s1, hm, w0[v + 1]);
-        up[v + 1] = fmat(s1, hp, w0[v + 1]);
-      } else {
-        const T s = limited_slope<LIM>((w0[v] - wm[v]) * im, (wp[v] - w0[v]) * ip, ph.eps);
-        lo[v] = fmat(-s, hm, w0[v]);
-        up[v] = fmat(s, hp, w0[v]);
+  {
+    T um1[NV], um2[NV], u0[NV], u1[NV], uh[NV];
+    load_raw(U + (int64_t)k0 * cs, N, c_own, u0);
+    if (h_halo >= 0) load_raw(U + (int64_t)k0 * cs, N, c_halo, uh);
+    if (h_halo >= 0 && k0 + 1 < k1) fetch_halo(k0 + 1);
+    if (k0 + 1 < nr) load_raw(U + (int64_t)(k0 + 1) * cs, N, c_own, u1);
+    if (k0 >= 1) load_raw(U + (int64_t)(k0 - 1) * cs, N, c_own, um1);
+    if (k0 >= 2) load_raw(U + (int64_t)(k0 - 2) * cs, N, c_own, um2);
+    if (k0 + 2 < nr) load_raw(U + (int64_t)(k0 + 2) * cs, N, c_own, pf_own);
+    {
+      const int64_t ts = (int64_t)(nt + 1) * np;
+      for (int q = tid; q < NTV; q += NT) {
+        const int f = q / TP, col = q % TP;
+        const int jf = min(j0 + f, nt), ic = min(i0 + col, np - 1);
+        const int64_t fc = (int64_t)jf * np + ic;
+        s_nth[q] = g.nth[fc];
+        s_nth[NTV + q] = g.nth[ts + fc];
+        s_nth[2 * NTV + q] = g.nth[2 * ts + fc];
+      }
+      for (int q = tid; q <= TP; q += NT) {
+        int ic = i0 + q;
+        ic = ic >= np ? ic - np : ic;
+        s_nph[q] = g.nph[ic];
+        s_nph[TP + 1 + q] = g.nph[np + ic];
+      }
+      s_nr[tid] = g.nr[ocol];
+      s_nr[NT + tid] = g.nr[cs + ocol];
+      s_nr[2 * NT + tid] = g.nr[2 * cs + ocol];
+      s_rh[tid] = g.rhat[c_own];
+      s_rh[NT + tid] = g.rhat[cs + c_own];
+      s_rh[2 * NT + tid] = g.rhat[2 * cs + c_own];
+      if (tid < D::NRAD) {
+        rad_slot(k0)[tid] = *rad_at(k0);
+        if (k0 + 1 < k1) rad_slot(k0 + 1)[tid] = *rad_at(k0 + 1);
+      }
+      if (tid <= TT) s_at[tid] = g.at[min(j0 + tid, nt)];
+      if (tid < TT) {
+        s_ar[tid] = g.ar[min(j0 + tid, nt - 1)];
+        s_av[tid] = g.av[min(j0 + tid, nt - 1)];
       }
     }
-  };
-
-  // ---------------- preamble
-  T rL[NV];          // L state of r face k + 1/2 (upper r value of plane k)
-  T frl[NF];         // flux x area of r face k - 1/2, lambda x area last
-  {
-    // own column of planes k0 - 1 and k0 - 2 (loads issued first so that they
-    // overlap with those of planes k0 and k0 + 1)
-    const int64_t ccol = c_own;
-    T um1[NV], um2[NV];
-    if (k0 >= 1) load_raw(U + (int64_t)(k0 - 1) * cs, N, ccol, um1);
-    if (k0 >= 2) load_raw(U + (int64_t)(k0 - 2) * cs, N, ccol, um2);
-    // planes k0 and k0 + 1 into the ring
-    for (int p = k0; p <= min(k0 + 1, nr - 1); ++p) {
-      prefetch(p);
-      store_prefetched(p);
+    recover(u0, ph, wc);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) sp[v * HC + hown] = wc[v];
+    if (h_halo >= 0) {
+      T w[NV];
+      recover(uh, ph, w);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) sp[v * HC + h_halo] = w[v];
     }
     __syncthreads();
-    if (k0 + 1 >= nr) outer_plane();
-    __syncthreads();
-    T w0[NV], w1[NV], wm1[NV], wm2[NV];
-    read_own(slot(k0), w0);
-    read_own(slot(k0 + 1), w1);
-    // inner ghost for plane -1
+    if (k0 + 1 < nr)
+      recover(u1, ph, w1);
+    else
+      outer_ghost(wc, s_rh[tid], s_rh[NT + tid], s_rh[2 * NT + tid], ph, w1);
+    T wm1[NV], wm2[NV];
     if (k0 >= 1) {
       recover(um1, ph, wm1);
-    } else {
-      inner_ghost_at(w0, Br, ccol, cs, (double)g.rhat[ccol], (double)g.rhat[cs + ccol],
-                     (double)g.rhat[2 * cs + ccol], ph, wm1);
+    } else {  // inner ghost for plane -1
+      inner_ghost_at(wc, Br, c_own, cs, (double)g.rhat[c_own], (double)g.rhat[cs + c_own],
+                     (double)g.rhat[2 * cs + c_own], ph, wm1);
     }
     if (k0 >= 2) {
       recover(um2, ph, wm2);
     } else if (k0 == 1) {
-      T wz[NV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) wz[v] = wm1[v];  // plane 0
-      inner_ghost_at(wz, Br, ccol, cs, (double)g.rhat[ccol], (double)g.rhat[cs + ccol],
-                     (double)g.rhat[2 * cs + ccol], ph, wm2);
+      inner_ghost_at(wm1, Br, c_own, cs, (double)g.rhat[c_own], (double)g.rhat[cs + c_own],
+                     (double)g.rhat[2 * cs + c_own], ph, wm2);
     }
     // r face k0 - 1/2
-    T wl[NV], wr[NV], up0[NV];
-    r_values(k0, wm1, w0, w1, wr, up0);  // lower / upper r values of plane k0
+    T wl[NV], wr[NV];
+    {
+      const T im = g.inv_dm[k0], ip = g.inv_dp[k0], hm = g.hm[k0], hp = g.hp[k0];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const T s = limited_slope<LIM>((wc[v] - wm1[v]) * im, (w1[v] - wc[v]) * ip, ph.eps);
+        wr[v] = fmat(-s, hm, wc[v]);
+        rL[v] = fmat(s, hp, wc[v]);
+      }
+    }
     if (k0 == 0) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) { wl[v] = wm1[v]; wr[v] = w0[v]; }  // boundary: first order
+      for (int v = 0; v < NV; ++v) { wl[v] = wm1[v]; wr[v] = wc[v]; }  // boundary: first order
     } else {
-      T lo[NV];
-      r_values(k0 - 1, wm2, wm1, w0, lo, wl);
+      const T im = g.inv_dm[k0 - 1], ip = g.inv_dp[k0 - 1], hp = g.hp[k0 - 1];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const T s = limited_slope<LIM>((wm1[v] - wm2[v]) * im, (wc[v] - wm1[v]) * ip, ph.eps);
+        wl[v] = fmat(s, hp, wm1[v]);
+      }
     }
     if (own) {
       T f[NV], la;
-      const T area = g.ra[k0] * s_ar[jj];
-      rusanov(wl, wr, s_nr[tid], s_nr[NT + tid], s_nr[2 * NT + tid], area, ph, f, la);
+      rusanov<true>(wl, wr, s_nr[tid], s_nr[NT + tid], s_nr[2 * NT + tid], g.ra[k0] * s_ar[jj], ph, f, la);
 #pragma unroll
       for (int v = 0; v < NV; ++v) frl[v] = f[v];
       frl[NV] = la;
@@ -633,207 +642,229 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
 #pragma unroll
       for (int v = 0; v < NF; ++v) frl[v] = (T)0;
     }
-#pragma unroll
-    for (int v = 0; v < NV; ++v) rL[v] = up0[v];
-    if (k0 + 2 < nr) prefetch(k0 + 2);
   }
 
   T sq[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) sq[v] = (T)0;
-  T dtm = (T)INFINITY;
+  T rate = (T)0;      // largest lambda |S| / V of the thread's cells
+  T dr[NF];           // r faces' contribution to the cell being gathered
+  bool bad = false;   // rho <= 0 or p <= 0 in that cell
 
-  for (int k = k0; k < k1; ++k) {
-    // ---- A: plane k + 2 enters the ring
-    if (k + 2 < nr) store_prefetched(k + 2);
-    __syncthreads();
-    if (k + 2 == nr) {
-      outer_plane();
-      __syncthreads();
-    }
-    // ---- B: prefetch plane k + 3; face values of plane k; r values of plane k + 1
-    if (k + 3 < nr) prefetch(k + 3);
-    const T* Pk = slot(k);
-    T wc[NV];
-    read_own(Pk, wc);
-    {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        const T* q = Pk + v * HC + hown;
-        T st, sp;
-        if constexpr (sizeof(T) == 8) {
-          limited_slope2<LIM>(wc[v] - q[-HP], q[HP] - wc[v], wc[v] - q[-1], q[1] - wc[v], ph.eps, st, sp);
-        } else {
-          st = limited_slope<LIM>(wc[v] - q[-HP], q[HP] - wc[v], ph.eps);
-          sp = limited_slope<LIM>(wc[v] - q[-1], q[1] - wc[v], ph.eps);
-        }
-        // explicit FMAs: the same rounding in every kernel inlining this
-        tvl[v * NTV + jj * TP + ii] = fmat(-half, st, wc[v]);
-        tvu[v * NTV + (jj + 1) * TP + ii] = fmat(half, st, wc[v]);
-        pvl[v * NPV + jj * (TP + 1) + ii] = fmat(-half, sp, wc[v]);
-        pvu[v * NPV + jj * (TP + 1) + ii + 1] = fmat(half, sp, wc[v]);
-      }
-      // halo cells whose face values the tile's boundary faces need
-      for (int e = tid; e < D::NEXTRA_V; e += NT) {
-        int hrow, hcol, dstep, idx;
-        T* dst;
-        if (e < TP) {                 // theta row -1: upper value -> face 0
-          hrow = 1; hcol = e + 2; dstep = HP; dst = tvu; idx = e;
-        } else if (e < 2 * TP) {      // theta row TT: lower value -> face TT
-          hrow = TT + 2; hcol = e - TP + 2; dstep = HP; dst = tvl; idx = TT * TP + (e - TP);
-        } else if (e < 2 * TP + TT) { // phi col -1 of row r: upper value -> face 0
-          const int r = e - 2 * TP;
-          hrow = r + 2; hcol = 1; dstep = 1; dst = pvu; idx = r * (TP + 1);
-        } else {                      // phi col TP of row r: lower value -> face TP
-          const int r = e - 2 * TP - TT;
-          hrow = r + 2; hcol = TP + 2; dstep = 1; dst = pvl; idx = r * (TP + 1) + TP;
-        }
-        const bool upper = (dst == tvu) || (dst == pvu);
-        const int nstride = (dst == tvu || dst == tvl) ? NTV : NPV;
-        constexpr int VSTEP = sizeof(T) == 8 ? 2 : 1;  // FP64: slopes in pairs
-#pragma unroll
-        for (int v = 0; v < NV; v += VSTEP) {
-          const T* q = Pk + v * HC + hrow * HP + hcol;
-          const T w = q[0];
-          if (VSTEP == 2 && v + 1 < NV) {
-            const T* q1 = q + HC;
-            const T w1 = q1[0];
-            T s, s1;
-            limited_slope2<LIM>(w - q[-dstep], q[dstep] - w, w1 - q1[-dstep], q1[dstep] - w1, ph.eps, s, s1);
-            dst[v * nstride + idx] = fmat(upper ? half : -half, s, w);
-            dst[(v + 1) * nstride + idx] = fmat(upper ? half : -half, s1, w1);
-          } else {
-            const T s = limited_slope<LIM>(w - q[-dstep], q[dstep] - w, ph.eps);
-            dst[v * nstride + idx] = fmat(upper ? half : -half, s, w);
-          }
-        }
-      }
-    }
-    T rR[NV], rLn[NV];
-    if (k + 1 < nr) {
-      T w1[NV], w2[NV];
-      read_own(slot(k + 1), w1);
-      read_own(slot(k + 2), w2);
-      r_values(k + 1, wc, w1, w2, rR, rLn);
-    }
-    __syncthreads();
-    // ---- C: faces of plane k
-    {
-      const T rbk = g.rb[k];
-      auto theta_face = [&](int q) {
-        const int f = q / TP, col = q % TP;
-        const int jf = j0 + f, ic = i0 + col;
-        if (jf <= 0 || jf >= nt || ic >= np) {  // poles, ragged rows / columns
-#pragma unroll
-          for (int v = 0; v < NV; ++v) ftb[v * NTV + q] = (T)0;
-          ftl[q] = (T)0;
-          return;
-        }
-        T wl[NV], wr[NV], fl[NV], la;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) { wl[v] = tvu[v * NTV + q]; wr[v] = tvl[v * NTV + q]; }
-        rusanov(wl, wr, s_nth[q], s_nth[NTV + q], s_nth[2 * NTV + q], rbk * s_at[f], ph, fl, la);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) ftb[v * NTV + q] = fl[v];
-        ftl[q] = la;
-      };
-      auto phi_face = [&](int row, int f) {
-        const int qq = row * (TP + 1) + f;
-        const int jr = j0 + row, ifc = i0 + f;
-        if (jr >= nt || ifc > np || (f == TP && ifc - 1 >= np)) {
-#pragma unroll
-          for (int v = 0; v < NV; ++v) fpb[v * NPV + qq] = (T)0;
-          fpl[qq] = (T)0;
-          return;
-        }
-        T wl[NV], wr[NV], fl[NV], la;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) { wl[v] = pvu[v * NPV + qq]; wr[v] = pvl[v * NPV + qq]; }
-        rusanov(wl, wr, s_nph[f], s_nph[TP + 1 + f], (T)0, rbk * g.dtheta, ph, fl, la);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) fpb[v * NPV + qq] = fl[v];
-        fpl[qq] = la;
-      };
-      theta_face(tid);                      // own lower theta face (row jj)
-      phi_face(jj, ii);                     // own lower phi face (col ii)
-      if (tid < TP) theta_face(NT + tid);   // faces of row TT: warp 0
-      if (tid >= 32 && tid < 32 + TT) phi_face(tid - 32, TP);  // faces of col TP: warp 1
-    }
-    // r face k + 1/2 (own column, registers)
-    T fru[NF];
-    if (own) {
-      T wl[NV], wr[NV], fl[NV], la;
-      if (k + 1 < nr) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) { wl[v] = rL[v]; wr[v] = rR[v]; }
-      } else {  // outer boundary face: first order, interior | ghost
-        const T* pg = slot(nr);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) { wl[v] = wc[v]; wr[v] = pg[v * HC + hown]; }
-      }
-      rusanov(wl, wr, s_nr[tid], s_nr[NT + tid], s_nr[2 * NT + tid], g.ra[k + 1] * s_ar[jj], ph,
-              fl, la);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) fru[v] = fl[v];
-      fru[NV] = la;
-    }
-    __syncthreads();
-    // ---- E: gather the six faces of cell (k, jo, io)
-    if (own) {
-      const int tl = jj * TP + ii, tu = tl + TP;
-      const int pl = jj * (TP + 1) + ii, pu = pl + 1;
+  for (int k = k0;; ++k) {
+    // ======== phase 1
+    if (k > k0 && own) {  // the six faces and the sources of cell (k - 1, jo, io)
+      const int kg = k - 1;
+      const int tl = tid, tu = tid + TP;
+      const int pl = NTV + jj * (TP + 1) + ii, pu = pl + 1;
       T r[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v)
-        r[v] = (frl[v] - fru[v]) + (ftb[v * NTV + tl] - ftb[v * NTV + tu]) +
-               (fpb[v * NPV + pl] - fpb[v * NPV + pu]);
-      const T lam = (frl[NV] + fru[NV]) + (ftl[tl] + ftl[tu]) + (fpl[pl] + fpl[pu]);
-      const T vol = g.rv[k] * s_av[jj];
-      const T ivol = one / vol;
-#pragma unroll
-      for (int v = 0; v < NV; ++v) r[v] *= ivol;
-      const T gk = -g.grav[k];
-      const T gx = gk * s_rh[tid], gy = gk * s_rh[NT + tid], gz = gk * s_rh[2 * NT + tid];
-      r[1] += wc[0] * gx;
-      r[2] += wc[0] * gy;
-      r[3] += wc[0] * gz;
-      r[7] += wc[0] * (wc[1] * gx + wc[2] * gy + wc[3] * gz);
-      r[8] -= ph.psi_damp * wc[8];
-      const int64_t cell = (int64_t)k * cs + ocol;
-      T chk = (T)0;
+        r[v] = dr[v] + (fx[v * NFA + tl] - fx[v * NFA + tu]) + (fx[v * NFA + pl] - fx[v * NFA + pu]);
+      const T lam = dr[NV] + (fx[NV * NFA + tl] + fx[NV * NFA + tu]) + (fx[NV * NFA + pl] + fx[NV * NFA + pu]);
+      const T ivol = frcp(rad_slot(kg)[1] * s_av[jj]);
+      const T x = lam * ivol;
+      rate = greater(x, rate) ? x : rate;
+      T* dst = R + (int64_t)kg * cs + ocol;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        R[v * N + cell] = r[v];
+        r[v] *= ivol;
+        dst[v * N] = r[v];
         sq[v] = fmat(r[v], r[v], sq[v]);
-        chk = fmat(r[v], r[v], chk);
       }
-      const T dtc = vol / lam;
-      dtm = dtc < dtm ? dtc : dtm;
-      if (!(wc[0] > (T)0) || !(wc[7] > (T)0) || !(fabs(chk) < (T)INFINITY)) flag_bad(red, cell);
-#pragma unroll
-      for (int v = 0; v < NF; ++v) frl[v] = fru[v];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) rL[v] = rLn[v];
+      if (bad || !squares_finite(r)) flag_bad(red, (int64_t)kg * cs + ocol);
     }
+    if (k >= k1) break;
+    T tlo[NV], plo[NV];  // the cell's lower theta and phi face values
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const T* q = sp + v * HC + hown;
+      const T w = wc[v];
+      const T st = limited_slope<LIM>(w - q[-HP], q[HP] - w, ph.eps);
+      const T sf = limited_slope<LIM>(w - q[-1], q[1] - w, ph.eps);
+      // explicit FMAs: the same rounding in every kernel inlining this
+      tlo[v] = fmat(-half, st, w);
+      uv[v * NFA + tid + TP] = fmat(half, st, w);
+      plo[v] = fmat(-half, sf, w);
+      uv[v * NFA + NTV + jj * (TP + 1) + ii + 1] = fmat(half, sf, w);
+    }
+    // halo cells whose face values the tile's boundary faces need: three
+    // variables of one cell per item
+    for (int x = tid; x < 3 * NX; x += NT) {
+      const int e = x % NX, v0 = 3 * (x / NX);
+      int h, step, dst, stride;
+      T sgn;
+      T* base;
+      if (e < TP) {                  // theta row -1: upper value -> face row 0
+        h = HP + e + 2; step = HP; base = uv; dst = e; stride = NFA; sgn = half;
+      } else if (e < TP + TT) {      // phi col -1 of row r: upper value -> face col 0
+        const int r = e - TP;
+        h = (r + 2) * HP + 1; step = 1; base = uv; dst = NTV + r * (TP + 1); stride = NFA; sgn = half;
+      } else if (e < 2 * TP + TT) {  // theta row TT: lower value, R state of face row TT
+        const int c = e - TP - TT;
+        h = (TT + 2) * HP + c + 2; step = HP; base = xr; dst = c; stride = NXF; sgn = -half;
+      } else {                       // phi col TP of row r: lower value, R state of face col TP
+        const int r = e - 2 * TP - TT;
+        h = (r + 2) * HP + TP + 2; step = 1; base = xr; dst = TP + r; stride = NXF; sgn = -half;
+      }
+      const T* q = sp + v0 * HC + h;
+      T* o = base + v0 * stride + dst;
+#pragma unroll
+      for (int v = 0; v < 3; ++v) {
+        const T w = q[v * HC];
+        const T s = limited_slope<LIM>(w - q[v * HC - step], q[v * HC + step] - w, ph.eps);
+        o[v * stride] = fmat(sgn, s, w);
+      }
+    }
+    __syncthreads();
+    // ======== phase 2
+    const T* rad = rad_slot(k);
+    const T rbk = rad[0];
+    {  // lower theta face of the own cell; poles and ragged rows / columns carry nothing
+      T fl[NV], la = (T)0;
+      if (jo > 0 && jo < nt && io < np) {
+        T wl[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) wl[v] = uv[v * NFA + tid];
+        rusanov<true>(wl, tlo, s_nth[tid], s_nth[NTV + tid], s_nth[2 * NTV + tid], rbk * s_at[jj], ph, fl, la);
+      } else {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) fl[v] = (T)0;
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) fx[v * NFA + tid] = fl[v];
+      fx[NV * NFA + tid] = la;
+    }
+    {  // lower phi face of the own cell
+      const int f = NTV + jj * (TP + 1) + ii;
+      T fl[NV], la = (T)0;
+      if (jo < nt && io <= np) {
+        T wl[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) wl[v] = uv[v * NFA + f];
+        rusanov<false>(wl, plo, s_nph[ii], s_nph[TP + 1 + ii], (T)0, rbk * g.dtheta, ph, fl, la);
+      } else {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) fl[v] = (T)0;
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) fx[v * NFA + f] = fl[v];
+      fx[NV * NFA + f] = la;
+    }
+    if (tid >= NT - ((NXF + 31) / 32) * 32) {  // the faces past the last row and column: the last warps
+      const int e = tid - (NT - ((NXF + 31) / 32) * 32);
+      if (e < NXF) {
+        int f;
+        T nx, ny, nz, area;
+        bool live;
+        if (e < TP) {
+          f = TT * TP + e;
+          live = j0 + TT < nt && i0 + e < np;
+          nx = s_nth[f]; ny = s_nth[NTV + f]; nz = s_nth[2 * NTV + f];
+          area = rbk * s_at[TT];
+        } else {
+          const int r = e - TP;
+          f = NTV + r * (TP + 1) + TP;
+          live = j0 + r < nt && i0 + TP <= np;
+          nx = s_nph[TP]; ny = s_nph[2 * TP + 1]; nz = (T)0;
+          area = rbk * g.dtheta;
+        }
+        T fl[NV], la = (T)0;
+        if (live) {
+          T wl[NV], wr[NV];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) { wl[v] = uv[v * NFA + f]; wr[v] = xr[v * NXF + e]; }
+          rusanov<true>(wl, wr, nx, ny, nz, area, ph, fl, la);
+        } else {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) fl[v] = (T)0;
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v) fx[v * NFA + f] = fl[v];
+        fx[NV * NFA + f] = la;
+      }
+    }
+    // r face k + 1/2 and the plane k + 1 that follows
+    T w2[NV], rLn[NV];
+    if (k + 2 < nr)
+      recover(pf_own, ph, w2);
+    else if (k + 2 == nr)
+      outer_ghost(w1, s_rh[tid], s_rh[NT + tid], s_rh[2 * NT + tid], ph, w2);
+    if (k + 3 < nr && k + 2 < k1 + 1) load_raw(U + (int64_t)(k + 3) * cs, N, c_own, pf_own);
+    {
+      T rR[NV];
+      if (k + 1 < nr) {
+        const T im = rad[4], ip = rad[5], hm = rad[6], hp = rad[7];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          const T s = limited_slope<LIM>((w1[v] - wc[v]) * im, (w2[v] - w1[v]) * ip, ph.eps);
+          rR[v] = fmat(-s, hm, w1[v]);
+          rLn[v] = fmat(s, hp, w1[v]);
+        }
+      } else {  // outer boundary face: first order, interior | ghost
+#pragma unroll
+        for (int v = 0; v < NV; ++v) { rL[v] = wc[v]; rR[v] = w1[v]; }
+      }
+      if (own) {
+        T f[NV], la;
+        rusanov<true>(rL, rR, s_nr[tid], s_nr[NT + tid], s_nr[2 * NT + tid], rad[3] * s_ar[jj], ph, f, la);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) { dr[v] = frl[v] - f[v]; frl[v] = f[v]; }
+        dr[NV] = frl[NV] + la;
+        frl[NV] = la;
+        // the sources in flux units (x V): gravity [Sect. 2.2] and GLM damping
+        const T vol = rad[1] * s_av[jj];
+        const T a = -(rad[2] * vol) * wc[0];
+        const T ex = s_rh[tid], ey = s_rh[NT + tid], ez = s_rh[2 * NT + tid];
+        dr[1] = fmat(a, ex, dr[1]);
+        dr[2] = fmat(a, ey, dr[2]);
+        dr[3] = fmat(a, ez, dr[3]);
+        dr[7] = fmat(a, fmat(wc[1], ex, fmat(wc[2], ey, wc[3] * ez)), dr[7]);
+        dr[8] = fmat(-(ph.psi_damp * vol), wc[8], dr[8]);
+        bad = !positive(wc[0]) || !positive(wc[7]);
+      }
+    }
+    if (k + 1 < k1) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) sp[v * HC + hown] = w1[v];
+      if (h_halo >= 0) {
+        T u[NV], w[NV];
+        copy_async_wait();
+#pragma unroll
+        for (int v = 0; v < NV; ++v) u[v] = hr[v * D::NHALO + tid];
+        recover(u, ph, w);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) sp[v * HC + h_halo] = w[v];
+        if (k + 2 < k1) {
+          fetch_halo(k + 2);
+          if (tid < D::NRAD) copy_async(rad_slot(k + 2) + tid, rad_at(k + 2));
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      wc[v] = w1[v];
+      w1[v] = w2[v];
+      rL[v] = rLn[v];
+    }
+    __syncthreads();
   }
   // ---------------- reductions: warp tree in T, then FP64 across warps and CTAs
+  T dtm = (T)INFINITY;
+  if (rate > (T)0) dtm = sizeof(T) == 4 ? (T)__frcp_rn((float)rate) : one / rate;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) sq[v] += __shfl_xor_sync(0xffffffffu, sq[v], off);
     const T o = __shfl_xor_sync(0xffffffffu, dtm, off);
-    dtm = o < dtm ? o : dtm;
+    dtm = greater(dtm, o) ? o : dtm;
   }
-  double tot[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) tot[v] = (threadIdx.x & 31) == 0 ? (double)sq[v] : 0.0;
-  double* scratch = reinterpret_cast<double*>(smem_raw);
-  reduce_and_finalize_at<NT, true>(tot, (double)dtm, red, scratch, bid, nblocks);
+  reduce_and_finalize_at<NT>(sq, dtm, red, reinterpret_cast<double*>(smem_raw), bid, nblocks);
 }
 
 // one grid: block (x, y) = (tile, radial chunk)
 template <class T, int LIM, int TT, int TP>
-__global__ void __launch_bounds__(TT * TP, MinCtas<T>::value)
+__global__ void __launch_bounds__(TT * TP, (MinCtas<T, TT * TP>::value))
 residual_tiled(Shape sh, Geo<T> g, Phys<T> ph, const double* __restrict__ Br,
                const T* __restrict__ U, T* __restrict__ R, Reduce red, int kchunk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -865,10 +896,13 @@ struct EnsMember {
 
 
 template <class T, int LIM, int TT, int TP>
-__global__ void __launch_bounds__(TT * TP, MinCtas<T>::value)
+__global__ void __launch_bounds__(TT * TP, (MinCtas<T, TT * TP>::value))
 residual_ensemble(const EnsMember<T>* __restrict__ mem, int nmem, int nitems, unsigned int* __restrict__ next) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_item;
+  __shared__ EnsMember<T> M;  // the item's member: its fields are read where they are used, not held in registers
+  __shared__ int s_item, s_mem;
+  static_assert(sizeof(EnsMember<T>) % 8 == 0, "copied as 64-bit words");
+  if (threadIdx.x == 0) s_mem = -1;
   for (;;) {
     if (threadIdx.x == 0) s_item = (int)atomicAdd(next, 1u);
     __syncthreads();
@@ -876,7 +910,13 @@ residual_ensemble(const EnsMember<T>* __restrict__ mem, int nmem, int nitems, un
     if (item >= nitems) break;
     int m = 0;
     while (m + 1 < nmem && mem[m + 1].item0 <= item) ++m;
-    const EnsMember<T>& M = mem[m];
+    if (m != s_mem) {
+      const unsigned long long* src = reinterpret_cast<const unsigned long long*>(mem + m);
+      unsigned long long* dst = reinterpret_cast<unsigned long long*>(&M);
+      for (int q = threadIdx.x; q < (int)(sizeof(EnsMember<T>) / 8); q += TT * TP) dst[q] = src[q];
+      __syncthreads();
+      if (threadIdx.x == 0) s_mem = m;
+    }
     const int local = item - M.item0;
     tiled_item<T, LIM, TT, TP>(M.sh, M.g, M.ph, M.Br, M.U, M.R, M.red, M.kchunk, local % M.ntiles,
                                local / M.ntiles, local, M.nitems, smem_raw);

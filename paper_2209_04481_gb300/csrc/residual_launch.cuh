@@ -8,9 +8,10 @@
 
 namespace crn {
 
-template <class T> struct TileFor;
-template <> struct TileFor<double> { static constexpr int TT = 8, TP = 32; };
-template <> struct TileFor<float> { static constexpr int TT = 8, TP = 32; };
+template <class T>
+struct TileFor {
+  static constexpr int TT = ens_tt(own_tile(sizeof(T) == 8)), TP = ens_tp(own_tile(sizeof(T) == 8));
+};
 
 template <class T> const Geo<T>& geo_of(const crn_grid* g);
 template <> inline const Geo<double>& geo_of<double>(const crn_grid* g) { return g->g64.geo; }
@@ -147,6 +148,9 @@ cudaError_t launch_ensemble_shape(const EnsMember<T>* dev, int nmem, int nitems,
 template <class T>
 cudaError_t launch_ensemble_t(const EnsMember<T>* dev, int nmem, int nitems, unsigned int* next, int limiter,
                               int tile, int nctas, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8) {
+    if (tile == 2) return launch_ensemble_shape<T, ens_tt(2), ens_tp(2)>(dev, nmem, nitems, next, limiter, nctas, st);
+  }
   if (tile == 0) return launch_ensemble_shape<T, ens_tt(0), ens_tp(0)>(dev, nmem, nitems, next, limiter, nctas, st);
   return launch_ensemble_shape<T, ens_tt(1), ens_tp(1)>(dev, nmem, nitems, next, limiter, nctas, st);
 }
@@ -168,6 +172,9 @@ int ensemble_ctas_shape(int limiter) {
 // shared-memory opt-in and resident CTAs per SM of one tile shape's kernel
 template <class T>
 int ensemble_ctas_t(int limiter, int tile) {
+  if constexpr (sizeof(T) == 8) {
+    if (tile == 2) return ensemble_ctas_shape<T, ens_tt(2), ens_tp(2)>(limiter);
+  }
   return tile == 0 ? ensemble_ctas_shape<T, ens_tt(0), ens_tp(0)>(limiter)
                    : ensemble_ctas_shape<T, ens_tt(1), ens_tp(1)>(limiter);
 }

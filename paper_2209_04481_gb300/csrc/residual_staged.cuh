@@ -524,11 +524,7 @@ __device__ __forceinline__ void staged_item(const Shape& sh, const Geo<float>& g
     const float o = __shfl_xor_sync(0xffffffffu, dtm, off);
     dtm = o < dtm ? o : dtm;
   }
-  double tot[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) tot[v] = lane == 0 ? (double)sq[v] : 0.0;
-  double* scratch = reinterpret_cast<double*>(ft);
-  reduce_and_finalize_at<D::NTH, true>(tot, (double)dtm, red, scratch, bid, nblocks);
+  reduce_and_finalize_at<D::NTH>(sq, dtm, red, reinterpret_cast<double*>(ft), bid, nblocks);
 }
 
 // the 1024-byte aligned base of the dynamic shared memory

@@ -70,6 +70,8 @@ struct DeviceSlot {
   bool geo_valid = false;
   crn_grid_desc geo_desc{};
   bool captured = false;  // a call on this device was recorded in a graph
+  crn_grid_desc plan_desc{};  // sizes, precision and limiter the radial chunk was chosen for
+  int kchunk = 0;             // (0: none yet)
 };
 
 std::mutex g_mu;
@@ -237,9 +239,11 @@ crn::Phys<T> phys_static(const crn_grid_desc& d) {
   return ph;
 }
 
-template <class T> struct StaticTile;
-template <> struct StaticTile<double> { static constexpr int TT = 8, TP = 32; };
-template <> struct StaticTile<float> { static constexpr int TT = 8, TP = 32; };
+// the tile of a grid's own launch
+template <class T>
+struct StaticTile {
+  static constexpr int TT = crn::ens_tt(crn::own_tile(sizeof(T) == 8)), TP = crn::ens_tp(crn::own_tile(sizeof(T) == 8));
+};
 
 template <class T>
 cudaError_t opt_in_smem() {
@@ -261,9 +265,36 @@ bool same_geometry(const crn_grid_desc& a, const crn_grid_desc& b) {
          a.precision == b.precision && a.r_in == b.r_in && a.r_out == b.r_out && a.g0 == b.g0;
 }
 
+// the radial chunk of a launch, as crn_grid_create chooses it
 template <class T>
-int run(const crn_grid_desc& d, unsigned char* base, const double* Br, const void* U, void* R,
+int plan(const crn_grid_desc& d, DeviceSlot& slot) {
+  const crn_grid_desc& p = slot.plan_desc;
+  if (slot.kchunk > 0 && p.n_r == d.n_r && p.n_theta == d.n_theta && p.n_phi == d.n_phi &&
+      p.precision == d.precision && p.limiter == d.limiter)
+    return slot.kchunk;
+  constexpr int TT = StaticTile<T>::TT, TP = StaticTile<T>::TP;
+  const int64_t ntiles = (int64_t)((d.n_theta + TT - 1) / TT) * ((d.n_phi + TP - 1) / TP);
+  int nsm = 0, per_sm = 0, dev = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const size_t smem = crn::TileDims<TT, TP>::template smem_bytes<T>();
+  if (d.limiter == CRN_LIM_NONE)
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 0, TT, TP>, TT * TP, smem);
+  else if (d.limiter == CRN_LIM_MINMOD)
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 1, TT, TP>, TT * TP, smem);
+  else
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 2, TT, TP>, TT * TP, smem);
+  int kc = crn::choose_radial_chunk(d.n_r, ntiles, std::max(nsm, 1), per_sm, sizeof(T) == 8);
+  while (ntiles * ((d.n_r + kc - 1) / kc) > kMaxBlocks) kc *= 2;
+  slot.plan_desc = d;
+  slot.kchunk = kc;
+  return kc;
+}
+
+template <class T>
+int run(const crn_grid_desc& d, DeviceSlot& slot, const double* Br, const void* U, void* R,
         double* norms, double* dtmin, cudaStream_t st) {
+  unsigned char* const base = slot.base;
   constexpr int TT = StaticTile<T>::TT, TP = StaticTile<T>::TP;
   crn::Shape sh;
   sh.nr = d.n_r;
@@ -271,14 +302,7 @@ int run(const crn_grid_desc& d, unsigned char* base, const double* Br, const voi
   sh.np = d.n_phi;
   sh.ncell = (int64_t)d.n_r * d.n_theta * d.n_phi;
   const int ntiles = ((sh.nt + TT - 1) / TT) * ((sh.np + TP - 1) / TP);
-  int nsm = 0, per_sm = 0;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 2, TT, TP>, TT * TP,
-                                                crn::TileDims<TT, TP>::template smem_bytes<T>());
-  int kc = crn::choose_kchunk(sh.nr, ntiles, (long long)std::max(nsm, 1) * std::max(per_sm, 1));
-  while ((int64_t)ntiles * ((sh.nr + kc - 1) / kc) > kMaxBlocks) kc *= 2;
+  const int kc = plan<T>(d, slot);
   const int nch = (sh.nr + kc - 1) / kc;
   crn::Reduce red;
   red.partials = reinterpret_cast<double*>(base + kPartialOff);
@@ -368,6 +392,6 @@ extern "C" int crn_residual_static(const crn_grid_desc* d, const double* Br_dev,
     slot.geo_valid = !slot.captured;
   }
   if (d->precision == CRN_FP64)
-    return run<double>(*d, slot.base, Br_dev, U_dev, R_dev, norms9_dev, dtmin_dev, st);
-  return run<float>(*d, slot.base, Br_dev, U_dev, R_dev, norms9_dev, dtmin_dev, st);
+    return run<double>(*d, slot, Br_dev, U_dev, R_dev, norms9_dev, dtmin_dev, st);
+  return run<float>(*d, slot, Br_dev, U_dev, R_dev, norms9_dev, dtmin_dev, st);
 }

@@ -59,8 +59,7 @@ __device__ __forceinline__ void pair_add(float& s, float& c, float s2, float c2)
 // Block sum of the per-thread compensated FP32 sums (256 threads): FP32
 // pairs across each warp by shuffles, then across the eight warps by warp 0;
 // tot[] of thread 0 receives the block's totals, every other thread's tot[]
-// is zero (the form reduce_and_finalize_at<256, true> takes, which adds the
-// warps' lane-0 values).  `scratch` holds at least 8 * 2 * NV floats.
+// is zero (reduce_and_finalize_at adds the warps' lane-0 values).  `scratch` holds at least 8 * 2 * NV floats.
 __device__ __forceinline__ void block_sum_pairs(Acc<float>& acc, double (&tot)[NV], double* scratch) {
   float* sp = reinterpret_cast<float*>(scratch);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -162,12 +161,16 @@ __device__ __forceinline__ void update_block(int64_t N, double* __restrict__ U, 
   double tot[NV];
   if constexpr (std::is_same<TR, float>::value) {
     block_sum_pairs(acc, tot, scratch);
-    reduce_and_finalize_at<256, true>(tot, INFINITY, red, scratch, bid, nblocks);
   } else {
 #pragma unroll
     for (int v = 0; v < NV; ++v) tot[v] = acc.total(v);
-    reduce_and_finalize_at<256>(tot, INFINITY, red, scratch, bid, nblocks);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) tot[v] += __shfl_xor_sync(0xffffffffu, tot[v], off);
+    }
   }
+  reduce_and_finalize_at<256>(tot, (double)INFINITY, red, scratch, bid, nblocks);
 }
 
 template <class TR>
