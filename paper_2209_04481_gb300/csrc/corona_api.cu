@@ -349,9 +349,11 @@ int crn_grid_create(const crn_grid_desc* d, crn_grid** out) {
     const int per_sm = d->precision == CRN_FP64 ? crn::tiled_ctas_per_sm_fp64(d->limiter)
                                                  : crn::tiled_ctas_per_sm_fp32(d->limiter);
     int kc = crn::choose_radial_chunk(d->n_r, ntiles, std::max(nsm, 1), per_sm, d->precision == CRN_FP64);
+    g->cfg.kchunk_pair =
+        crn::choose_radial_chunk(d->n_r, 2 * ntiles, std::max(nsm, 1), per_sm, d->precision == CRN_FP64);
     if (const char* env = std::getenv("CRN_KCHUNK")) {  // tuning override
       const int v = std::atoi(env);
-      if (v >= 1) kc = v;
+      if (v >= 1) kc = g->cfg.kchunk_pair = v;
     }
     g->cfg.kchunk_tiled = kc;
     g->cfg.num_sms = std::max(nsm, 1);

@@ -29,6 +29,7 @@ struct GeoBuf {
 
 struct LaunchCfg {
   int kchunk_tiled = 16;  // radial planes per CTA of the tiled kernel
+  int kchunk_pair = 16;   // the same for two residuals in one launch
   int num_sms = 152;      // streaming multiprocessors of the grid's device
   int update_per_sm = 2;  // resident blocks per SM of the pseudo-time update
   bool staged = false;    // FP32 residuals use the TMA-staged kernel (on request)
@@ -71,6 +72,12 @@ cudaError_t launch_residual_fp64(crn_grid* g, const double* U, double* R, double
                                  double* dt_user, cudaStream_t st, int* nlaunch);
 cudaError_t launch_residual_fp32(crn_grid* g, const float* U, float* R, double* norms_user,
                                  double* dt_user, cudaStream_t st, int* nlaunch);
+// two residuals in one launch, without norms or dtmin (cellwise and TMA-staged
+// grids: two launches)
+cudaError_t launch_residual_pair_fp64(crn_grid* g, const double* Ua, double* Ra, const double* Ub, double* Rb,
+                                      cudaStream_t st, int* nlaunch);
+cudaError_t launch_residual_pair_fp32(crn_grid* g, const float* Ua, float* Ra, const float* Ub, float* Rb,
+                                      cudaStream_t st, int* nlaunch);
 cudaError_t launch_update(crn_grid* g, double* U64, double cfl, double* res_out,
                           cudaStream_t st, int* nlaunch);
 cudaError_t launch_shadow(crn_grid* g, const double* U64, cudaStream_t st, int* nlaunch);

@@ -44,14 +44,36 @@ namespace crn {
 
 namespace {
 
-constexpr int NKB = 256;  // threads per block of the vector kernels
+constexpr int NKB = 256;  // threads per block of the elementwise kernels
+constexpr int NKD = 512;  // threads per block of the Gram-Schmidt kernels
 // a Newton step keeps at least this fraction of every cell's density and pressure
 constexpr double kKeepFrac = 0.1;
-constexpr int MD = 8;     // vectors per multi-dot launch
+constexpr int MD = 8;     // vectors a Gram-Schmidt pass takes at a time
 
 // ---------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------
+// whether this block is the last of the grid to get here; its threads then see
+// everything the others wrote before (*counter is zero before and after)
+__device__ __forceinline__ bool last_block(unsigned int* counter) {
+  __shared__ unsigned int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s_last = atomicAdd(counter, 1u) == gridDim.x * gridDim.y - 1 ? 1u : 0u;
+    if (s_last) *counter = 0u;
+  }
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  return true;
+}
+
+// an FP32 Krylov vector widens on the integer pipe (exact): the FP64 pipe also
+// runs the conversion instruction
+__device__ __forceinline__ double as_double(float x) { return widen_f32(x); }
+__device__ __forceinline__ double as_double(double x) { return x; }
+
 // block sum of K values per thread into part[(row + k) * nblk + blockIdx.x]
 template <int K>
 __device__ __forceinline__ void block_sum_rows(double (&a)[K], double* part, int nblk, int row,
@@ -70,36 +92,6 @@ __device__ __forceinline__ void block_sum_rows(double (&a)[K], double* part, int
     double s = 0.0;
     for (int q = 0; q < NKB / 32; ++q) s += sm[q * K + threadIdx.x];
     part[(size_t)(row + threadIdx.x) * nblk + blockIdx.x] = s;
-  }
-}
-
-// partial dots <V_(i0+t), w>, t < cnt, into rows row_v + t; with ww also
-// <w, w> into row row_ww
-__global__ void __launch_bounds__(NKB)
-mdot_kernel(const double* __restrict__ V, int64_t n, int i0, int cnt, const double* __restrict__ w,
-            double* __restrict__ part, int nblk, int row_v, int ww, int row_ww) {
-  double a[MD + 1];
-#pragma unroll
-  for (int t = 0; t <= MD; ++t) a[t] = 0.0;
-  const int64_t stride = (int64_t)nblk * NKB;
-  // two elements per trip: their loads are in flight together, so that the
-  // FMAs (bound by the FP64 pipe) overlap the memory latency
-#pragma unroll 2
-  for (int64_t e = (int64_t)blockIdx.x * NKB + threadIdx.x; e < n; e += stride) {
-    const double we = w[e];
-#pragma unroll
-    for (int t = 0; t < MD; ++t)
-      if (t < cnt) a[t] += V[(int64_t)(i0 + t) * n + e] * we;
-    a[MD] += we * we;
-  }
-  double b[MD];
-#pragma unroll
-  for (int t = 0; t < MD; ++t) b[t] = a[t];
-  block_sum_rows<MD>(b, part, nblk, row_v, cnt);
-  if (ww) {
-    double c[1] = {a[MD]};
-    __syncthreads();
-    block_sum_rows<1>(c, part, nblk, row_ww, 1);
   }
 }
 
@@ -125,6 +117,210 @@ finish_kernel(const double* __restrict__ part, int nblk, int row0, double* __res
   if (threadIdx.x == 0) out[row] = sm[0];
 }
 
+// ---- Gram-Schmidt on the device -------------------------------------------
+// Classical Gram-Schmidt of w against V_0 .. V_(cnt-1), repeated once if the
+// norm dropped to below 0.7: dots, update (which also takes the new norm and
+// decides), and the same two kernels again, which return at once if the repeat
+// is not needed.  The host reads the column of the Hessenberg matrix once per
+// Krylov step.  An FP32 basis keeps the products on the FP32 pipe (GB300 runs
+// FP64 FMAs at 1/64 of the FP32 rate): sums over a thread's elements in FP32,
+// across threads in FP64.  What bounds these kernels is the traffic of V for
+// large shells and, for small ones, the FP64 adds of the reductions, which a
+// warp issues at one per 16 clocks: eight sums of 32 lanes take 9 adds by
+// recursive halving (40 with a shuffle tree each), the grid is one block per SM
+// so that few partials remain, and the last block adds those.  A Krylov step's
+// products with V on 32 x 16 x 32: five launches of 20 us and five of 5 us over
+// their partials before, four of 13 us (cold) now; the step 33 -> 6.4 ms in all.
+struct GsOut {
+  double* h;             // [m + 1] the column: h_t
+  double* ww;            // [1] |w|^2 before the first pass
+  double* after;         // [1] |w|^2 after the last pass
+  double* inv;           // [1] 1 / |w| then (0 for w = 0)
+  double* coef;          // [m + 1] -h_t of the pass
+  double* redo;          // [1] 1: the second pass is needed
+  unsigned int* counter;
+};
+
+template <class T> struct Vec;
+template <> struct Vec<float> { using type = float4; static constexpr int N = 4; };
+template <> struct Vec<double> { using type = double2; static constexpr int N = 2; };
+__device__ __forceinline__ void vdot(float& s, const float4& a, const float4& b) {
+  s = fmaf(a.x, b.x, s); s = fmaf(a.y, b.y, s); s = fmaf(a.z, b.z, s); s = fmaf(a.w, b.w, s);
+}
+__device__ __forceinline__ void vdot(double& s, const double2& a, const double2& b) {
+  s = fma(a.x, b.x, s); s = fma(a.y, b.y, s);
+}
+__device__ __forceinline__ void vaxpy(float4& w, float c, const float4& v) {
+  w.x = fmaf(c, v.x, w.x); w.y = fmaf(c, v.y, w.y); w.z = fmaf(c, v.z, w.z); w.w = fmaf(c, v.w, w.w);
+}
+__device__ __forceinline__ void vaxpy(double2& w, double c, const double2& v) {
+  w.x = fma(c, v.x, w.x); w.y = fma(c, v.y, w.y);
+}
+
+// eight sums over a warp by recursive halving: lane l returns the sum of
+// a[l >> 2] (the same in its group of four lanes)
+__device__ __forceinline__ double warp_sum8(double (&a)[MD], int lane) {
+#pragma unroll
+  for (int w = 4, bit = 16; w > 0; w >>= 1, bit >>= 1) {
+    const bool hi = (lane & bit) != 0;
+#pragma unroll
+    for (int t = 0; t < w; ++t) {
+      const double give = hi ? a[t] : a[t + w], keep = hi ? a[t + w] : a[t];
+      a[t] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+    }
+  }
+  double s = a[0];
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  return s;
+}
+
+// the block's sums of eight values per thread into part[(row + t) * nblk + block], t < cnt
+__device__ __forceinline__ void block_sum8(double (&a)[MD], double* part, int nblk, int row, int cnt) {
+  __shared__ double sm[(NKD / 32) * MD];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const double s = warp_sum8(a, lane);
+  __syncthreads();  // sm may still be read for the previous eight
+  if ((lane & 3) == 0) sm[wid * MD + (lane >> 2)] = s;
+  __syncthreads();
+  if ((int)threadIdx.x < cnt) {
+    double x = 0.0;
+#pragma unroll
+    for (int q = 0; q < NKD / 32; ++q) x += sm[q * MD + threadIdx.x];
+    part[(size_t)(row + threadIdx.x) * nblk + blockIdx.x] = x;
+  }
+}
+
+// the last block's sums over the partials of `rows` rows: one warp takes eight
+// rows at a time; put(row, sum) runs on one lane per row
+template <class F>
+__device__ __forceinline__ void sum_partials(const double* part, int nblk, int rows, F put) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int r0 = wid * MD; r0 < rows; r0 += (NKD / 32) * MD) {
+    double a[MD];
+#pragma unroll
+    for (int t = 0; t < MD; ++t) {
+      a[t] = 0.0;
+      if (r0 + t < rows)
+        for (int q = lane; q < nblk; q += 32) a[t] += __ldcg(part + (size_t)(r0 + t) * nblk + q);
+    }
+    const double s = warp_sum8(a, lane);
+    const int r = r0 + (lane >> 2);
+    if ((lane & 3) == 0 && r < rows) put(r, s);
+  }
+}
+
+// h_t = <V_t, w> for t < cnt; pass 0 also |w|^2, pass 1 only if the repeat is
+// needed, its h_t added to the first's
+template <class TV>
+__global__ void __launch_bounds__(NKD)
+gs_dots_kernel(const TV* __restrict__ V, int64_t n, int cnt, const TV* __restrict__ w, double* __restrict__ part,
+               GsOut o, int pass) {
+  if (pass == 1 && *o.redo == 0.0) return;
+  using V4 = typename Vec<TV>::type;
+  const int64_t nv = n / Vec<TV>::N;
+  const int64_t stride = (int64_t)gridDim.x * NKD, first = (int64_t)blockIdx.x * NKD + threadIdx.x;
+  const V4* w4 = reinterpret_cast<const V4*>(w);
+  const int nblk = gridDim.x;
+  // rows: the cnt dots, then |w|^2; block y takes eight vectors (their dots side
+  // by side: one after the other, a small shell's took 20 us for 16)
+  if (pass == 0 && blockIdx.y == 0) {
+    TV s = (TV)0;
+    for (int64_t e = first; e < nv; e += stride) { const V4 x = w4[e]; vdot(s, x, x); }
+    double b[MD] = {(double)s};
+    block_sum8(b, part, nblk, cnt, 1);
+  }
+  const int i0 = blockIdx.y * MD, c = min(MD, cnt - i0);
+  if (c > 0) {
+    const V4* v4 = reinterpret_cast<const V4*>(V + (int64_t)i0 * n);
+    TV a[MD];
+#pragma unroll
+    for (int t = 0; t < MD; ++t) a[t] = (TV)0;
+    if (c == MD) {
+      for (int64_t e = first; e < nv; e += stride) {
+        const V4 x = w4[e];
+#pragma unroll
+        for (int t = 0; t < MD; ++t) vdot(a[t], v4[(int64_t)t * nv + e], x);
+      }
+    } else {
+      for (int64_t e = first; e < nv; e += stride) {
+        const V4 x = w4[e];
+#pragma unroll
+        for (int t = 0; t < MD; ++t)
+          if (t < c) vdot(a[t], v4[(int64_t)t * nv + e], x);
+      }
+    }
+    double b[MD];
+#pragma unroll
+    for (int t = 0; t < MD; ++t) b[t] = (double)a[t];
+    block_sum8(b, part, nblk, i0, c);
+  }
+  if (!last_block(o.counter)) return;
+  sum_partials(part, nblk, cnt + (pass == 0 ? 1 : 0), [&](int r, double s) {
+    if (r == cnt) {
+      *o.ww = s;
+    } else {
+      o.coef[r] = -s;
+      o.h[r] = pass == 0 ? s : o.h[r] + s;
+    }
+  });
+}
+
+// w += sum_t coef_t V_t, then |w|^2; pass 0 decides whether the norm dropped
+// enough for a second pass, pass 1 runs only then
+template <class TV>
+__global__ void __launch_bounds__(NKD)
+gs_update_kernel(TV* __restrict__ w, const TV* __restrict__ V, int64_t n, int cnt, double* __restrict__ part,
+                 GsOut o, int pass) {
+  if (pass == 1 && *o.redo == 0.0) return;
+  using V4 = typename Vec<TV>::type;
+  __shared__ TV sc[512];
+  for (int t = threadIdx.x; t < cnt; t += NKD) sc[t] = (TV)o.coef[t];
+  __syncthreads();
+  const int64_t nv = n / Vec<TV>::N;
+  const int64_t stride = (int64_t)gridDim.x * NKD;
+  const V4* v4 = reinterpret_cast<const V4*>(V);
+  V4* w4 = reinterpret_cast<V4*>(w);
+  TV s = (TV)0;
+  for (int64_t e = (int64_t)blockIdx.x * NKD + threadIdx.x; e < nv; e += stride) {
+    V4 x = w4[e];
+#pragma unroll 16
+    for (int t = 0; t < cnt; ++t) vaxpy(x, sc[t], v4[(int64_t)t * nv + e]);
+    w4[e] = x;
+    vdot(s, x, x);
+  }
+  double b[MD] = {(double)s};
+  block_sum8(b, part, gridDim.x, 0, 1);
+  if (!last_block(o.counter)) return;
+  sum_partials(part, gridDim.x, 1, [&](int, double a) {
+    *o.after = a;
+    *o.inv = a > 0.0 ? 1.0 / sqrt(a) : 0.0;
+    if (pass == 0) *o.redo = sqrt(fmax(a, 0.0)) < 0.7 * sqrt(fmax(*o.ww, 0.0)) ? 1.0 : 0.0;
+  });
+}
+
+// V_j = w / |w| (w may be V_j); nothing if |w| is 0.  1 / |w| comes from the
+// update's last block: a square root and a division in every thread are 40 slots
+// of the FP64 pipe, 7 us on a small shell.
+template <class TV>
+__global__ void __launch_bounds__(NKB)
+gs_scale_kernel(TV* y, const TV* x, int64_t n, const double* __restrict__ inv) {
+  using V4 = typename Vec<TV>::type;
+  const TV f = (TV)*inv;
+  if (!(f > (TV)0)) return;
+  const int64_t nv = n / Vec<TV>::N, stride = (int64_t)gridDim.x * NKB;
+  for (int64_t e = (int64_t)blockIdx.x * NKB + threadIdx.x; e < nv; e += stride) {
+    V4 v = reinterpret_cast<const V4*>(x)[e];
+    v.x *= f;
+    v.y *= f;
+    if constexpr (sizeof(TV) == 4) {
+      v.z *= f;
+      v.w *= f;
+    }
+    reinterpret_cast<V4*>(y)[e] = v;
+  }
+}
+
 // w += sum_t coef[t] V_t (V FP64, or the FP32 basis into an FP64 w)
 template <class TV>
 __global__ void __launch_bounds__(NKB)
@@ -134,49 +330,6 @@ maxpy_kernel(double* __restrict__ w, const TV* __restrict__ V, int64_t n,
   for (int64_t e = (int64_t)blockIdx.x * NKB + threadIdx.x; e < n; e += stride) {
     double s = w[e];
     for (int t = 0; t < cnt; ++t) s += coef[t] * (double)V[(int64_t)t * n + e];
-    w[e] = s;
-  }
-}
-
-// ---- FP32 Krylov basis: the orthogonalisation on the FP32 pipe (GB300 runs
-// FP64 FMAs at 1/64 of the FP32 rate, which bounds the FP64 multi-dot and
-// update); sums over a thread's elements in FP32, across threads in FP64
-
-// partial dots <Vf_(i0+t), wf>, t < cnt, into rows row_v + t; with ww <wf, wf>
-__global__ void __launch_bounds__(NKB)
-mdot32_kernel(const float* __restrict__ V, int64_t n, int i0, int cnt, const float* __restrict__ w,
-              double* __restrict__ part, int nblk, int row_v, int ww, int row_ww) {
-  float a[MD + 1];
-#pragma unroll
-  for (int t = 0; t <= MD; ++t) a[t] = 0.f;
-  const int64_t stride = (int64_t)nblk * NKB;
-#pragma unroll 2
-  for (int64_t e = (int64_t)blockIdx.x * NKB + threadIdx.x; e < n; e += stride) {
-    const float we = w[e];
-#pragma unroll
-    for (int t = 0; t < MD; ++t)
-      if (t < cnt) a[t] = fmaf(V[(int64_t)(i0 + t) * n + e], we, a[t]);
-    a[MD] = fmaf(we, we, a[MD]);
-  }
-  double b[MD];
-#pragma unroll
-  for (int t = 0; t < MD; ++t) b[t] = (double)a[t];
-  block_sum_rows<MD>(b, part, nblk, row_v, cnt);
-  if (ww) {
-    double c[1] = {(double)a[MD]};
-    __syncthreads();
-    block_sum_rows<1>(c, part, nblk, row_ww, 1);
-  }
-}
-
-// wf += sum_t coef[t] Vf_t in FP32
-__global__ void __launch_bounds__(NKB)
-maxpy32_kernel(float* __restrict__ w, const float* __restrict__ V, int64_t n,
-               const float* __restrict__ coef, int cnt) {
-  const int64_t stride = (int64_t)gridDim.x * NKB;
-  for (int64_t e = (int64_t)blockIdx.x * NKB + threadIdx.x; e < n; e += stride) {
-    float s = w[e];
-    for (int t = 0; t < cnt; ++t) s = fmaf(coef[t], V[(int64_t)t * n + e], s);
     w[e] = s;
   }
 }
@@ -215,26 +368,48 @@ add_kernel(double* y, const double* x, int64_t n) {
 }
 
 // w = z / dtau - w: the shifted adjoint operator (D - J^T) z from w = J^T z
-// (D = diag(1 / dtau), one dtau per cell shared by its nine variables)
+// (D = diag(1 / dtau), one dtau per cell shared by its nine variables).  The
+// kernels that pair a cell with its variables take the variable from block y:
+// no index division.
 __global__ void __launch_bounds__(NKB)
 shift_combine_kernel(double* __restrict__ w, const double* __restrict__ z, const double* __restrict__ dtau,
-                     int64_t N, int64_t n) {
-  const int64_t stride = (int64_t)gridDim.x * NKB;
-  for (int64_t e = (int64_t)blockIdx.x * NKB + threadIdx.x; e < n; e += stride) w[e] = z[e] / dtau[e % N] - w[e];
+                     int64_t N) {
+  const int64_t stride = (int64_t)gridDim.x * NKB, q0 = blockIdx.y * N;
+  for (int64_t c = (int64_t)blockIdx.x * NKB + threadIdx.x; c < N; c += stride)
+    w[q0 + c] = fma(z[q0 + c], frcp(dtau[c]), -w[q0 + c]);
 }
 
-// per-variable partial sums of |u| (rows 0..8)
+// floors of the finite-difference step, s_v = 1e-3 (mean |u_v| + mean |u| over
+// the nine variables): never zero, also for a variable that vanishes everywhere
+// (psi of a start state); in out[row .. row + 8]
 __global__ void __launch_bounds__(NKB)
-absmean_kernel(const double* __restrict__ U, int64_t N, double* __restrict__ part, int nblk, int row) {
+floors_kernel(const double* __restrict__ U, int64_t N, double* __restrict__ part, double* __restrict__ out,
+              int row, unsigned int* counter) {
   double a[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) a[v] = 0.0;
-  const int64_t stride = (int64_t)nblk * NKB;
+  const int64_t stride = (int64_t)gridDim.x * NKB;
   for (int64_t c = (int64_t)blockIdx.x * NKB + threadIdx.x; c < N; c += stride) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) a[v] += fabs(U[v * N + c]);
   }
-  block_sum_rows<NV>(a, part, nblk, row, NV);
+  block_sum_rows<NV>(a, part, gridDim.x, row, NV);
+  if (!last_block(counter)) return;
+  __shared__ double sum[NV];
+  const int lane = threadIdx.x & 31;
+  for (int v = threadIdx.x >> 5; v < NV; v += NKB / 32) {
+    double s = 0.0;
+    for (int q = lane; q < (int)gridDim.x; q += 32) s += __ldcg(part + (size_t)(row + v) * gridDim.x + q);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) sum[v] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < NV) {
+    double tot = 0.0;
+    for (int v = 0; v < NV; ++v) tot += sum[v];
+    out[row + threadIdx.x] = 1e-3 * (sum[threadIdx.x] + tot / NV) / (double)N;
+  }
 }
 
 // reciprocal good to about 20 bits (PTX rcp.approx.ftz.f64), for the ratios
@@ -246,109 +421,158 @@ __device__ __forceinline__ double rcp_coarse(double x) {
   return r;
 }
 
-// z = dtau . v (dtau per cell, shared by its nine variables).  With want_min,
-// two partial minima for the finite-difference step: over entries of
-// (|u| + s_v) / |z| into row `row`, and over cells of p / |dp_lin(z)| into
-// row `row` + 1 (dp_lin the linearised pressure change along z)
+// z = dtau . v (dtau per cell, shared by its nine variables)
 template <class TV>
 __global__ void __launch_bounds__(NKB)
-precond_kernel(const TV* __restrict__ v, const double* __restrict__ dtau, int64_t N,
-               double* __restrict__ z, const double* __restrict__ U, const double* __restrict__ sumabs,
-               double gm1, double* __restrict__ part, int nblk, int row, int want_min) {
-  double m = INFINITY, mp = INFINITY;
-  const int64_t stride = (int64_t)nblk * NKB;
-  // floors s_v = 1e-3 (mean |u_v| + mean |u| over the nine variables): never
-  // zero, also for a variable that vanishes everywhere (psi of a start state)
-  double s[NV];
-  if (want_min) {
-    double tot = 0.0;
+scale_cells_kernel(const TV* __restrict__ v, const double* __restrict__ dtau, int64_t N, double* __restrict__ z) {
+  const int64_t stride = (int64_t)gridDim.x * NKB, q0 = blockIdx.y * N;
+  for (int64_t c = (int64_t)blockIdx.x * NKB + threadIdx.x; c < N; c += stride)
+    z[q0 + c] = dtau[c] * as_double(v[q0 + c]);
+}
+
+// z = dtau . v (dtau null: v is the direction z already) and the
+// finite-difference step along it: eps = min(b min_entries (|u| + s_v) / |z|,
+// min_cells p / (4 |dp_lin(z)|)) with dp_lin the linearised pressure change, and
+// for the second order p(U + e z) = p + e dp - e^2 (gamma - 1) Q, Q = |z_B|^2 / 2
+// + |z_m - V z_rho|^2 / (2 rho): e <= sqrt(p / ((gamma - 1) Q)) / 2 keeps the
+// last term within p / 4.  eps and 1 / eps go to eps_out[0] and [1] (1 if z = 0).
+// The step needs the ratios' magnitude only: they are formed in FP32 wherever
+// the entries fit (a conversion on the integer pipe and an FP32 reciprocal in
+// place of two slots of the FP64 pipe), the pressures in FP64.  The minima are
+// combined by integer minima of their bit patterns, and the last block forms
+// eps: 38 us on 96 x 48 x 96, where FP64 ratios, nine divisions per thread for
+// the floors and two more kernels for the minima and eps took 134 + 8 us.
+struct StepMin {
+  unsigned int* bits;      // [2] minima as FP32 bit patterns (0x7f800000 between launches)
+  unsigned int* counter;
+};
+constexpr int NKE = 128;  // threads per block: long threads, and a small shell has few cells
+template <class TV>
+__global__ void __launch_bounds__(NKE)
+direction_kernel(const TV* __restrict__ v, const double* __restrict__ dtau, int64_t N, double* __restrict__ z,
+                 const double* __restrict__ U, const double* __restrict__ floors, double gm1, double b,
+                 StepMin sm, double* __restrict__ eps_out) {
+  float m = INFINITY, mp = INFINITY;
+  float fl[NV];
 #pragma unroll
-    for (int q = 0; q < NV; ++q) tot += sumabs[q];
-#pragma unroll
-    for (int q = 0; q < NV; ++q) s[q] = 1e-3 * (sumabs[q] + tot / NV) / (double)N;
-  }
-  for (int64_t c = (int64_t)blockIdx.x * NKB + threadIdx.x; c < N; c += stride) {
-    // dtau null: v already is the direction z (statistics only)
-    const double d = dtau ? dtau[c] : 1.0;
-    double zz[NV];
+  for (int q = 0; q < NV; ++q) fl[q] = narrow_f64(floors[q]);
+  const int64_t stride = (int64_t)gridDim.x * NKE;
+  for (int64_t c = (int64_t)blockIdx.x * NKE + threadIdx.x; c < N; c += stride) {
+    double zz[NV], u[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
-      zz[q] = d * (double)v[q * N + c];
-      if (dtau) z[q * N + c] = zz[q];
-    }
-    if (!want_min) continue;
-    double u[NV];
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
+      zz[q] = as_double(v[q * N + c]);
       u[q] = U[q * N + c];
-      if (zz[q] != 0.0) m = fmin(m, (fabs(u[q]) + s[q]) * rcp_coarse(fabs(zz[q])));
+    }
+    if (dtau) {
+      const double d = dtau[c];
+#pragma unroll
+      for (int q = 0; q < NV; ++q) {
+        zz[q] *= d;
+        z[q * N + c] = zz[q];
+      }
+    }
+    float zf[NV], uf[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      zf[q] = narrow_f64(zz[q]);
+      uf[q] = narrow_f64(u[q]);
+      const float az = fabsf(zf[q]), au = fabsf(uf[q]) + fl[q];
+      float r;
+      if (az > 1e-30f && az < 1e30f && au > 1e-30f && au < 1e30f)
+        r = __fdividef(au, az);
+      else  // zero, or beyond the range of FP32 arithmetic
+        r = zz[q] != 0.0 ? narrow_f64((fabs(u[q]) + floors[q]) * rcp_coarse(fabs(zz[q]))) : INFINITY;
+      m = fminf(m, r);
     }
     const double ir = rcp_coarse(u[0]);
     const double vx = u[1] * ir, vy = u[2] * ir, vz = u[3] * ir;
-    const double p = gm1 * (u[7] - 0.5 * (u[1] * vx + u[2] * vy + u[3] * vz) -
-                            0.5 * (u[4] * u[4] + u[5] * u[5] + u[6] * u[6]));
-    const double dp = gm1 * (zz[7] - (vx * zz[1] + vy * zz[2] + vz * zz[3]) +
-                             0.5 * (vx * vx + vy * vy + vz * vz) * zz[0] -
-                             (u[4] * zz[4] + u[5] * zz[5] + u[6] * zz[6]));
-    if (dp != 0.0) mp = fmin(mp, p * rcp_coarse(fabs(dp)));
-    // second order: p(U + e z) = p + e dp - e^2 gm1 Q + ..., Q = |z_B|^2 / 2 +
-    // |z_m - V z_rho|^2 / (2 rho); with e <= mp / 4 this keeps e^2 gm1 Q <= p / 4
-    const double wx = zz[1] - vx * zz[0], wy = zz[2] - vy * zz[0], wz = zz[3] - vz * zz[0];
-    const double Q = 0.5 * (zz[4] * zz[4] + zz[5] * zz[5] + zz[6] * zz[6]) +
-                     0.5 * (wx * wx + wy * wy + wz * wz) * ir;
-    if (Q > 0.0 && p > 0.0) mp = fmin(mp, 2.0 * sqrt(p * rcp_coarse(gm1 * Q)));
-  }
-  if (!want_min) return;
-  __shared__ double sm[2][NKB];
-  sm[0][threadIdx.x] = m;
-  sm[1][threadIdx.x] = mp;
-  __syncthreads();
-  for (int h = NKB / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) {
-      sm[0][threadIdx.x] = fmin(sm[0][threadIdx.x], sm[0][threadIdx.x + h]);
-      sm[1][threadIdx.x] = fmin(sm[1][threadIdx.x], sm[1][threadIdx.x + h]);
+    // p / (gamma - 1) and dp / (gamma - 1)
+    const double t = fma(u[1], vx, fma(u[2], vy, fma(u[3], vz, fma(u[4], u[4], fma(u[5], u[5], u[6] * u[6])))));
+    const double pe = fma(-0.5, t, u[7]);
+    const double v2 = fma(vx, vx, fma(vy, vy, vz * vz));
+    const double dpe = fma(0.5 * v2, zz[0], zz[7]) -
+                       fma(vx, zz[1], fma(vy, zz[2], fma(vz, zz[3],
+                           fma(u[4], zz[4], fma(u[5], zz[5], u[6] * zz[6])))));
+    const float pf = narrow_f64(pe), df = fabsf(narrow_f64(dpe));
+    if (df > 1e-30f && df < 1e30f && fabsf(pf) > 1e-30f && fabsf(pf) < 1e30f)
+      mp = fminf(mp, __fdividef(pf, df));
+    else if (dpe != 0.0)
+      mp = fminf(mp, narrow_f64(pe * rcp_coarse(fabs(dpe))));
+    const float rf = uf[0], fx = narrow_f64(vx), fy = narrow_f64(vy), fz = narrow_f64(vz);
+    const float wx = zf[1] - fx * zf[0], wy = zf[2] - fy * zf[0], wz = zf[3] - fz * zf[0];
+    const float Q = 0.5f * (zf[4] * zf[4] + zf[5] * zf[5] + zf[6] * zf[6]) +
+                    0.5f * (wx * wx + wy * wy + wz * wz) / rf;
+    if (Q > 1e-30f && Q < 1e30f && pf > 1e-30f && pf < 1e30f) {
+      mp = fminf(mp, 2.f * sqrtf(pf / Q));
+    } else if (pe > 0.0) {
+      const double dx = zz[1] - vx * zz[0], dy = zz[2] - vy * zz[0], dz = zz[3] - vz * zz[0];
+      const double Qd = 0.5 * (zz[4] * zz[4] + zz[5] * zz[5] + zz[6] * zz[6]) +
+                        0.5 * (dx * dx + dy * dy + dz * dz) * ir;
+      if (Qd > 0.0) mp = fminf(mp, narrow_f64(2.0 * sqrt(pe * rcp_coarse(Qd))));
     }
-    __syncthreads();
   }
+  // a negative pressure gives a negative ratio: it orders below every other
+  // minimum and, like a zero, leaves the entry ratio to set the step
+  m = fmaxf(m, 0.f);
+  mp = fmaxf(mp, 0.f);
+  const unsigned bm = __reduce_min_sync(0xffffffffu, __float_as_uint(m));
+  const unsigned bp = __reduce_min_sync(0xffffffffu, __float_as_uint(mp));
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(sm.bits, bm);
+    atomicMin(sm.bits + 1, bp);
+  }
+  if (!last_block(sm.counter)) return;
   if (threadIdx.x == 0) {
-    part[(size_t)row * nblk + blockIdx.x] = sm[0][0];
-    part[(size_t)(row + 1) * nblk + blockIdx.x] = sm[1][0];
+    const double me = b * (double)__uint_as_float(__ldcg(sm.bits));
+    const double e = fmin(me, 0.25 * (double)__uint_as_float(__ldcg(sm.bits + 1)));
+    const double eps = isfinite(e) && e > 0.0 ? e : (isfinite(me) && me > 0.0 ? me : 1.0);
+    eps_out[0] = eps;
+    eps_out[1] = 1.0 / eps;
+    sm.bits[0] = sm.bits[1] = 0x7f800000u;
   }
 }
 
-// eps = min(b * entry ratio, p ratio / 4) (1 if z = 0), written to out[dst]
-__global__ void eps_kernel(double* out, int src, int dst, double b) {
-  const double m = b * out[src];
-  const double mp = 0.25 * out[src + 1];
-  const double e = fmin(m, mp);
-  out[dst] = isfinite(e) && e > 0.0 ? e : (isfinite(m) ? m : 1.0);
-}
-
-// ut = (T)(U + sign eps z) (eps = 0 without z)
+// ut = (T)U
 template <class T>
 __global__ void __launch_bounds__(NKB)
-perturb_kernel(const double* __restrict__ U, const double* __restrict__ z,
-               const double* __restrict__ eps, double sign, int64_t n, T* __restrict__ ut) {
-  const double ee = z ? sign * *eps : 0.0;
+cast_kernel(const double* __restrict__ U, int64_t n, T* __restrict__ ut) {
   const int64_t stride = (int64_t)gridDim.x * NKB;
-  for (int64_t e = (int64_t)blockIdx.x * NKB + threadIdx.x; e < n; e += stride)
-    ut[e] = (T)(z ? U[e] + ee * z[e] : U[e]);
+  for (int64_t e = (int64_t)blockIdx.x * NKB + threadIdx.x; e < n; e += stride) ut[e] = (T)U[e];
 }
 
-// w = v - (R(U + eps z) - R(U)) / eps (forward difference, div = 1) or
-// w = v - (R(U + eps z) - R(U - eps z)) / (2 eps) (central difference, div = 2)
-template <class T, class TV = double>
+__device__ __forceinline__ void store_as(double* p, double x) { *p = x; }
+__device__ __forceinline__ void store_as(float* p, double x) { *p = narrow_f64(x); }
+
+// up = (T)(U + eps z) and, if um is set, um = (T)(U - eps z)
+template <class T>
 __global__ void __launch_bounds__(NKB)
-jvp_combine_kernel(const TV* __restrict__ v, const T* __restrict__ rp, const T* __restrict__ rb,
-                   const double* __restrict__ eps, double div, int64_t n, double* __restrict__ w,
-                   const double* __restrict__ dinv = nullptr, const double* __restrict__ z = nullptr,
-                   int64_t N = 1) {
-  const double ie = 1.0 / (div * *eps);
+perturb_kernel(const double* __restrict__ U, const double* __restrict__ z, const double* __restrict__ eps,
+               int64_t n, T* __restrict__ up, T* __restrict__ um) {
+  const double ee = *eps;
   const int64_t stride = (int64_t)gridDim.x * NKB;
   for (int64_t e = (int64_t)blockIdx.x * NKB + threadIdx.x; e < n; e += stride) {
-    // with dinv: the D z term of (D - J) z for a general right preconditioner
-    const double first = dinv ? dinv[e % N] * z[e] : (v ? (double)v[e] : 0.0);
-    w[e] = first - ((double)rp[e] - (double)rb[e]) * ie;
+    const double u = U[e], x = z[e];
+    store_as(up + e, fma(ee, x, u));
+    if (um) store_as(um + e, fma(-ee, x, u));
+  }
+}
+
+// w = v - (R(U + eps z) - R(U)) / eps (forward difference, half = 1) or
+// w = v - (R(U + eps z) - R(U - eps z)) / (2 eps) (central difference, half =
+// 0.5), ieps = 1 / eps; with dinv the D z term of (D - J) z in place of v.  TW:
+// FP64, or the FP32 of an FP32 basis.
+template <class T, class TV, class TW>
+__global__ void __launch_bounds__(NKB)
+jvp_combine_kernel(const TV* __restrict__ v, const T* __restrict__ rp, const T* __restrict__ rb,
+                   const double* __restrict__ ieps, double half, int64_t N, TW* __restrict__ w,
+                   const double* __restrict__ dinv, const double* __restrict__ z) {
+  const double ie = half * *ieps;
+  const int64_t stride = (int64_t)gridDim.x * NKB, q0 = blockIdx.y * N;
+  for (int64_t c = (int64_t)blockIdx.x * NKB + threadIdx.x; c < N; c += stride) {
+    const int64_t e = q0 + c;
+    const double first = dinv ? dinv[c] * z[e] : as_double(v[e]);
+    store_as(w + e, fma(-(as_double(rp[e]) - as_double(rb[e])), ie, first));
   }
 }
 
@@ -569,12 +793,9 @@ line_factor_kernel(Shape sh, const double* __restrict__ lo, const double* __rest
 // y_k = (v_k - l_k y_(k-1)) / m_k, backward z_k = y_k - c_k z_(k+1).  One
 // thread per (variable, column): the nine right-hand sides share the factors,
 // and 9 n_theta n_phi threads keep every SM busy; the loads along r do not
-// depend on the recurrence and are issued ahead of it.
-// an FP32 Krylov vector widens on the integer pipe (exact): the FP64 pipe,
-// which also runs the conversion instruction, carries the recurrence
-__device__ __forceinline__ double as_double(float x) { return widen_f32(x); }
-__device__ __forceinline__ double as_double(double x) { return x; }
-
+// depend on the recurrence and are issued ahead of it.  96 x 48 x 96 with an FP32
+// vector: 48 us; 32 x 16 x 32: 11 us (89 and 25 us with the loads left to the
+// compiler's unrolling).
 template <class TV>
 __global__ void __launch_bounds__(NKB)
 line_solve_kernel(Shape sh, const double* __restrict__ lo, const double* __restrict__ cp,
@@ -585,19 +806,61 @@ line_solve_kernel(Shape sh, const double* __restrict__ lo, const double* __restr
   const int64_t q = t / cs, col = t - q * cs;
   const TV* __restrict__ vq = v + q * N;
   double* __restrict__ zq = z + q * N;
-  double y = as_double(vq[col]) * im[col];
-  zq[col] = y;
-#pragma unroll 4
-  for (int k = 1; k < sh.nr; ++k) {
-    const int64_t c = (int64_t)k * cs + col;
-    y = fma(-lo[c], y, as_double(vq[c])) * im[c];
-    zq[c] = y;
+  // eight planes at a time, the next eight's loads in flight: the backward sweep
+  // reads z where the forward one wrote it, so the compiler keeps every load
+  // behind the stores before it
+  constexpr int B = 8;
+  const int nr = sh.nr;
+  double y = 0.0;
+  {
+    double l[B], m[B], l2[B], m2[B];
+    TV x[B], x2[B];
+    auto fetch = [&](int k, double (&a)[B], double (&b)[B], TV (&c)[B]) {
+#pragma unroll
+      for (int u = 0; u < B; ++u)
+        if (k + u < nr) {
+          const int64_t e = (int64_t)(k + u) * cs + col;
+          a[u] = lo[e];  // 0 in plane 0
+          b[u] = im[e];
+          c[u] = vq[e];
+        }
+    };
+    fetch(0, l, m, x);
+    for (int k = 0; k < nr; k += B) {
+      fetch(k + B, l2, m2, x2);
+#pragma unroll
+      for (int u = 0; u < B; ++u)
+        if (k + u < nr) {
+          y = fma(-l[u], y, as_double(x[u])) * m[u];
+          zq[(int64_t)(k + u) * cs + col] = y;
+        }
+#pragma unroll
+      for (int u = 0; u < B; ++u) { l[u] = l2[u]; m[u] = m2[u]; x[u] = x2[u]; }
+    }
   }
-#pragma unroll 4
-  for (int k = sh.nr - 2; k >= 0; --k) {
-    const int64_t c = (int64_t)k * cs + col;
-    y = fma(-cp[c], y, zq[c]);
-    zq[c] = y;
+  {
+    double f[B], x[B], f2[B], x2[B];
+    auto fetch = [&](int k, double (&a)[B], double (&b)[B]) {
+#pragma unroll
+      for (int u = 0; u < B; ++u)
+        if (k - u >= 0) {
+          const int64_t e = (int64_t)(k - u) * cs + col;
+          a[u] = cp[e];
+          b[u] = zq[e];
+        }
+    };
+    fetch(nr - 2, f, x);
+    for (int k = nr - 2; k >= 0; k -= B) {
+      fetch(k - B, f2, x2);
+#pragma unroll
+      for (int u = 0; u < B; ++u)
+        if (k - u >= 0) {
+          y = fma(-f[u], y, x[u]);
+          zq[(int64_t)(k - u) * cs + col] = y;
+        }
+#pragma unroll
+      for (int u = 0; u < B; ++u) { f[u] = f2[u]; x[u] = x2[u]; }
+    }
   }
 }
 
@@ -616,7 +879,8 @@ struct NkWork {
   double* x = nullptr;     // n: GMRES solution y
   double* b = nullptr;     // n: R(U) in FP64
   double* w = nullptr;     // n: Arnoldi vector
-  void* ut = nullptr;      // n of T: cast / perturbed state
+  void* ut = nullptr;      // n of T: cast state / U + eps z
+  void* um = nullptr;      // n of T: U - eps z (allocated by the first central difference)
   void* rt = nullptr;      // n of T: perturbed residual
   void* rb = nullptr;      // n of T: base residual (FP32 grids) / R(U - eps z) (FP64 grids)
   void* rm = nullptr;      // n of T: R(U - eps z) (FP32 grids)
@@ -625,12 +889,11 @@ struct NkWork {
                            //     factors c_k, upper of the transposed lines for the adjoint,
                            //     the inverse pivots 1/m_k)
   float* Vf = nullptr;     // (m + 1) n: the FP32 Krylov basis (allocated on first use)
-  float* wf = nullptr;     // n: the FP32 Arnoldi vector
-  float* coef32 = nullptr; // m + 2 FP32 coefficients
   double* part = nullptr;  // rows x nblk partials
   double* out = nullptr;   // rows reduced values
   double* coef = nullptr;  // m + 2 coefficients
   double* host = nullptr;  // pinned mirror of out
+  unsigned int* sync = nullptr;  // arrival counter, then the two minima of direction_kernel
   double* adj = nullptr;   // 2n: the pseudo-time adjoint's lambda and residual (first use)
   double* fv = nullptr;    // (mf + 1) n: outer FGMRES basis of the pseudo-time adjoint
   double* fz = nullptr;    // mf n: its preconditioned directions
@@ -642,7 +905,7 @@ void nk_free(NkWork* w) {
   cudaFree(w->V); cudaFree(w->z); cudaFree(w->x); cudaFree(w->b); cudaFree(w->w);
   cudaFree(w->ut); cudaFree(w->rt); cudaFree(w->rb); cudaFree(w->rm); cudaFree(w->dtau);
   cudaFree(w->line);
-  cudaFree(w->Vf); cudaFree(w->wf); cudaFree(w->coef32);
+  cudaFree(w->Vf); cudaFree(w->um); cudaFree(w->sync);
   cudaFree(w->part); cudaFree(w->out); cudaFree(w->coef);
   cudaFree(w->adj);
   cudaFree(w->fv); cudaFree(w->fz);
@@ -652,15 +915,17 @@ void nk_free(NkWork* w) {
 
 namespace {
 
-// rows of the out array beyond the m + 2 dot rows
+// rows of the out array: the column h_0 .. h_m, then
 struct Rows {
-  int ww, sumabs, minr, eps, relmax, bad, total;
+  int ww, after, redo, inv, floors, eps, relmax, bad, total;
   explicit Rows(int m) {
     ww = m + 1;
-    sumabs = m + 2;
-    minr = sumabs + NV;  // two rows: entry ratio, pressure ratio
-    eps = minr + 2;
-    relmax = eps + 1;
+    after = ww + 1;
+    redo = after + 1;
+    inv = redo + 1;
+    floors = inv + 1;
+    eps = floors + NV;  // eps, 1 / eps
+    relmax = eps + 2;
     bad = relmax + 1;
     total = bad + 1;
   }
@@ -671,14 +936,14 @@ int report(int code, const std::string& msg) { return report_error(code, msg.c_s
 // the FP32 Krylov basis of a workspace (allocated on first use)
 cudaError_t ensure_basis32(NkWork* w) {
   if (w->Vf) return cudaSuccess;
-  cudaError_t e = cudaMalloc(&w->Vf, sizeof(float) * (size_t)(w->m + 1) * w->n);
-  if (e == cudaSuccess) e = cudaMalloc(&w->wf, sizeof(float) * w->n);
-  if (e == cudaSuccess) e = cudaMalloc(&w->coef32, sizeof(float) * (w->m + 2));
-  if (e != cudaSuccess) {
-    cudaFree(w->Vf); cudaFree(w->wf); cudaFree(w->coef32);
-    w->Vf = nullptr; w->wf = nullptr; w->coef32 = nullptr;
-  }
-  return e;
+  return cudaMalloc(&w->Vf, sizeof(float) * (size_t)(w->m + 1) * w->n);
+}
+
+// the second perturbed state of a central difference (allocated on first use)
+cudaError_t ensure_central(crn_grid* g) {
+  NkWork* w = g->nk;
+  if (w->um) return cudaSuccess;
+  return cudaMalloc(&w->um, (size_t)(g->d.precision == CRN_FP64 ? 8 : 4) * w->n);
 }
 
 bool use_basis32(const crn_nk_options& o) {
@@ -712,6 +977,11 @@ cudaError_t ensure_work(crn_grid* g, int m) {
   if (e == cudaSuccess) e = cudaMalloc(&w->out, sizeof(double) * w->rows);
   if (e == cudaSuccess) e = cudaMalloc(&w->coef, sizeof(double) * (m + 2));
   if (e == cudaSuccess) e = cudaMallocHost(&w->host, sizeof(double) * w->rows);
+  if (e == cudaSuccess) e = cudaMalloc(&w->sync, 3 * sizeof(unsigned int));
+  if (e == cudaSuccess) {
+    const unsigned int init[3] = {0u, 0x7f800000u, 0x7f800000u};
+    e = cudaMemcpy(w->sync, init, sizeof(init), cudaMemcpyHostToDevice);
+  }
   if (e != cudaSuccess) { nk_free(w); g->nk = nullptr; }
   return e;
 }
@@ -731,6 +1001,8 @@ struct Ctx {
                                       n(9 * gg->shape.ncell) {
     grid = (unsigned)std::min<int64_t>((n + NKB - 1) / NKB, (int64_t)g->cfg.num_sms * 16);
   }
+  // grid of the kernels over (cell, variable)
+  dim3 cells() const { return dim3((unsigned)std::min<int64_t>((N + NKB - 1) / NKB, (int64_t)g->cfg.num_sms * 2), NV); }
   bool ok() { if (err == cudaSuccess) err = cudaGetLastError(); return err == cudaSuccess; }
 
   void finish(int row0, int nrows, int op) {
@@ -743,68 +1015,44 @@ struct Ctx {
     err = cudaMemcpyAsync(w->host + row0, w->out + row0, sizeof(double) * cnt, cudaMemcpyDeviceToHost, st);
     if (err == cudaSuccess) err = cudaStreamSynchronize(st);
   }
-  // h[t] = <V_t, v> for t < cnt (into out rows 0..cnt-1); with ww also <v, v>
-  void dots(int cnt, const double* v, bool ww) { dots_on(w->V, cnt, v, ww); }
-  void dots_on(const double* base, int cnt, const double* v, bool ww) {
-    for (int i0 = 0; i0 < cnt || (i0 == 0 && ww); i0 += MD) {
-      const int c = std::min(MD, cnt - i0);
-      mdot_kernel<<<w->nblk, NKB, 0, st>>>(base, n, i0, std::max(c, 0), v, w->part, w->nblk, i0,
-                                           (ww && i0 == 0) ? 1 : 0, rows.ww);
-      ++launches;
-      if (i0 + MD >= cnt) break;
+  GsOut gs() const {
+    return GsOut{w->out, w->out + rows.ww, w->out + rows.after, w->out + rows.inv, w->coef, w->out + rows.redo, w->sync};
+  }
+  // blocks of the Gram-Schmidt kernels: one per SM, fewer for a short vector
+  unsigned gs_blocks(int per) const {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n / per + NKD - 1) / NKD, g->cfg.num_sms));
+  }
+  // x orthogonalised against base_0 .. base_(cnt-1), its column of the Hessenberg
+  // matrix h_0 .. h_(cnt-1) and its remaining norm in host memory, x scaled to one
+  template <class TV>
+  double orthonormalise(const TV* base, int cnt, TV* x, double* h) {
+    const unsigned nb = gs_blocks(Vec<TV>::N);
+    for (int pass = 0; pass < 2; ++pass) {
+      gs_dots_kernel<TV><<<dim3(nb, (unsigned)((cnt + MD - 1) / MD)), NKD, 0, st>>>(base, n, cnt, x, w->part, gs(), pass);
+      gs_update_kernel<TV><<<nb, NKD, 0, st>>>(x, base, n, cnt, w->part, gs(), pass);
     }
-    if (cnt > 0) finish(0, cnt, 0);
-    if (ww) finish(rows.ww, 1, 0);
+    gs_scale_kernel<TV><<<grid, NKB, 0, st>>>(x, x, n, w->out + rows.inv);
+    launches += 5;
+    fetch(0, rows.redo);
+    for (int t = 0; t < cnt; ++t) h[t] = w->host[t];
+    return std::sqrt(std::max(w->host[rows.after], 0.0));
   }
   double norm(const double* v) {
-    dots(0, v, true);
+    gs_dots_kernel<double><<<gs_blocks(2), NKD, 0, st>>>(v, n, 0, v, w->part, gs(), 0);
+    ++launches;
     fetch(rows.ww, 1);
     return std::sqrt(std::max(w->host[rows.ww], 0.0));
   }
   // y += sum_t c[t] V_t
   void combine(double* y, const double* c, int cnt) { combine_on(y, w->V, c, cnt); }
-  void combine_on(double* y, const double* base, const double* c, int cnt) {
+  template <class TV>
+  void combine_on(double* y, const TV* base, const double* c, int cnt) {
     if (!ok() || cnt <= 0) return;
     // a copy from pageable memory returns once the source has been staged, so
     // c may be reused at once; stream order keeps coef intact for maxpy
     err = cudaMemcpyAsync(w->coef, c, sizeof(double) * cnt, cudaMemcpyHostToDevice, st);
     if (err != cudaSuccess) return;
-    maxpy_kernel<double><<<grid, NKB, 0, st>>>(y, base, n, w->coef, cnt);
-    ++launches;
-  }
-  // FP32 basis: h[t] = <Vf_t, vf> (rows 0..cnt-1), with ww also <vf, vf>
-  void dots32(int cnt, const float* v, bool ww) {
-    for (int i0 = 0; i0 < cnt || (i0 == 0 && ww); i0 += MD) {
-      const int c = std::min(MD, cnt - i0);
-      mdot32_kernel<<<w->nblk, NKB, 0, st>>>(w->Vf, n, i0, std::max(c, 0), v, w->part, w->nblk, i0,
-                                             (ww && i0 == 0) ? 1 : 0, rows.ww);
-      ++launches;
-      if (i0 + MD >= cnt) break;
-    }
-    if (cnt > 0) finish(0, cnt, 0);
-    if (ww) finish(rows.ww, 1, 0);
-  }
-  double norm32(const float* v) {
-    dots32(0, v, true);
-    fetch(rows.ww, 1);
-    return std::sqrt(std::max(w->host[rows.ww], 0.0));
-  }
-  // vf += sum_t c[t] Vf_t in FP32
-  void combine32(float* y, const double* c, int cnt) {
-    if (!ok() || cnt <= 0) return;
-    std::vector<float> cf(c, c + cnt);
-    // from pageable memory the copy returns once cf has been staged
-    err = cudaMemcpyAsync(w->coef32, cf.data(), sizeof(float) * cnt, cudaMemcpyHostToDevice, st);
-    if (err != cudaSuccess) return;
-    maxpy32_kernel<<<grid, NKB, 0, st>>>(y, w->Vf, n, w->coef32, cnt);
-    ++launches;
-  }
-  // x += sum_t c[t] Vf_t in FP64 (the solution update of a cycle)
-  void combine_x32(double* y, const double* c, int cnt) {
-    if (!ok() || cnt <= 0) return;
-    err = cudaMemcpyAsync(w->coef, c, sizeof(double) * cnt, cudaMemcpyHostToDevice, st);
-    if (err != cudaSuccess) return;
-    maxpy_kernel<float><<<grid, NKB, 0, st>>>(y, w->Vf, n, w->coef, cnt);
+    maxpy_kernel<TV><<<grid, NKB, 0, st>>>(y, base, n, w->coef, cnt);
     ++launches;
   }
   template <class TX>
@@ -819,6 +1067,18 @@ struct Ctx {
                         : launch_residual_fp32(g, (const float*)u, (float*)r, nullptr, nullptr, st, &nl);
     launches += nl;
     ++evals;
+    if (err == cudaSuccess) err = e;
+  }
+  // the two residuals of a central difference in one launch
+  void residual_pair(const void* ua, void* ra, const void* ub, void* rb) {
+    int nl = 0;
+    cudaError_t e = g->d.precision == CRN_FP64
+                        ? launch_residual_pair_fp64(g, (const double*)ua, (double*)ra, (const double*)ub,
+                                                    (double*)rb, st, &nl)
+                        : launch_residual_pair_fp32(g, (const float*)ua, (float*)ra, (const float*)ub,
+                                                    (float*)rb, st, &nl);
+    launches += nl;
+    evals += 2;
     if (err == cudaSuccess) err = e;
   }
   int mode = 0;  // 0: y - J(dtau . y) (pseudo-time step), 1: J^T (dtau . y) (adjoint)
@@ -846,9 +1106,10 @@ struct Ctx {
     ++launches;
   }
 
-  // v: a Krylov vector (FP64, or FP32 with the FP32 basis, forward mode only)
+  // v: a Krylov vector, wout the operator's product with it, both FP64 or both
+  // FP32 (the FP32 basis, forward mode only)
   template <class TV>
-  void apply(const TV* v, double* wout, const double* U, double b_rel, bool central) {
+  void apply(const TV* v, TV* wout, const double* U, double b_rel, bool central) {
     if constexpr (sizeof(TV) == 8) {
       if (mode == 1) {
         adjoint_op(v, wout);
@@ -858,20 +1119,23 @@ struct Ctx {
     apply_op(v, wout, U, b_rel, central);
   }
 
+  // z = P^-1 v for the adjoint and for the solution: dtau . v or the radial lines
+  void precondition(const double* v, double* z) {
+    if (precond == 1) {
+      line_solve(v, z);
+    } else {
+      scale_cells_kernel<double><<<cells(), NKB, 0, st>>>(v, w->dtau, N, z);
+      ++launches;
+    }
+  }
   // w_out = J^T (dtau . v) by the hand-written VJP of the residual; on FP32-bulk
   // grids ut holds the FP32 copy of U and the cotangent goes through rm / rt.
   // With ashift: w_out = (D - J^T) P^-1 v.
   void adjoint_op(const double* v, double* wout) {
-    if (precond == 1) {
-      line_solve(v, w->z);
-    } else {
-      precond_kernel<double><<<w->nblk, NKB, 0, st>>>(v, w->dtau, N, w->z, nullptr, nullptr, 0.0, w->part,
-                                                      w->nblk, rows.minr, 0);
-      ++launches;
-    }
+    precondition(v, w->z);
     vjp(w->z, wout);
     if (ashift) {
-      shift_combine_kernel<<<grid, NKB, 0, st>>>(wout, w->z, w->dtau, N, n);
+      shift_combine_kernel<<<cells(), NKB, 0, st>>>(wout, w->z, w->dtau, N);
       ++launches;
     }
   }
@@ -882,7 +1146,7 @@ struct Ctx {
     if (g->d.precision == CRN_FP64) {
       e = launch_vjp_fp64(g, (const double*)w->ut, v, wout, nullptr, st, &nl);
     } else {
-      perturb_kernel<float><<<grid, NKB, 0, st>>>(v, nullptr, nullptr, 0.0, n, (float*)w->rm);
+      cast_kernel<float><<<grid, NKB, 0, st>>>(v, n, (float*)w->rm);
       ++launches;
       e = launch_vjp_fp32(g, (const float*)w->ut, (const float*)w->rm, (float*)w->rt, nullptr, st, &nl);
       widen_kernel<<<grid, NKB, 0, st>>>((const float*)w->rt, n, wout);
@@ -895,49 +1159,37 @@ struct Ctx {
 
   // w_out = v - J (dtau . v), J by a forward or central difference
   template <class TV>
-  void apply_op(const TV* v, double* wout, const double* U, double b_rel, bool central) {
+  void apply_op(const TV* v, TV* wout, const double* U, double b_rel, bool central) {
+    const StepMin sm{w->sync + 1, w->sync};
+    double* e = w->out + rows.eps;
+    const double gm1 = g->d.gamma - 1.0;
+    const unsigned nb = (unsigned)std::min<int64_t>((N + NKE - 1) / NKE, 8 * (int64_t)g->cfg.num_sms);
     if (precond == 1) {
       line_solve(v, w->z);
-      precond_kernel<double><<<w->nblk, NKB, 0, st>>>(w->z, nullptr, N, w->z, U, w->out + rows.sumabs,
-                                                      g->d.gamma - 1.0, w->part, w->nblk, rows.minr, 1);
+      direction_kernel<double><<<nb, NKE, 0, st>>>(w->z, nullptr, N, w->z, U, w->out + rows.floors, gm1, b_rel, sm, e);
     } else {
-      precond_kernel<TV><<<w->nblk, NKB, 0, st>>>(v, w->dtau, N, w->z, U, w->out + rows.sumabs,
-                                                  g->d.gamma - 1.0, w->part, w->nblk, rows.minr, 1);
+      direction_kernel<TV><<<nb, NKE, 0, st>>>(v, w->dtau, N, w->z, U, w->out + rows.floors, gm1, b_rel, sm, e);
     }
     ++launches;
-    const double* dinv = precond == 1 ? w->line : nullptr;
-    finish(rows.minr, 2, 2);
-    eps_kernel<<<1, 1, 0, st>>>(w->out, rows.minr, rows.eps, b_rel);
-    ++launches;
+    if (g->d.precision == CRN_FP64)
+      difference<double>(v, wout, U, central, w->b, w->rb);
+    else
+      difference<float>(v, wout, U, central, w->rb, w->rm);
+  }
+  // the finite difference along z: base R(U) for the forward one, the second
+  // residual in `other` for the central one
+  template <class T, class TV>
+  void difference(const TV* v, TV* wout, const double* U, bool central, const void* base, void* other) {
     const double* e = w->out + rows.eps;
-    if (g->d.precision == CRN_FP64) {
-      perturb_kernel<double><<<grid, NKB, 0, st>>>(U, w->z, e, 1.0, n, (double*)w->ut);
-      ++launches;
+    perturb_kernel<T><<<grid, NKB, 0, st>>>(U, w->z, e, n, (T*)w->ut, central ? (T*)w->um : nullptr);
+    if (central)
+      residual_pair(w->ut, w->rt, w->um, other);
+    else
       residual(w->ut, w->rt);
-      const double* base = w->b;
-      if (central) {
-        perturb_kernel<double><<<grid, NKB, 0, st>>>(U, w->z, e, -1.0, n, (double*)w->ut);
-        ++launches;
-        residual(w->ut, w->rb);
-        base = (const double*)w->rb;
-      }
-      jvp_combine_kernel<double, TV><<<grid, NKB, 0, st>>>(v, (const double*)w->rt, base, e,
-                                                           central ? 2.0 : 1.0, n, wout, dinv, w->z, N);
-    } else {
-      perturb_kernel<float><<<grid, NKB, 0, st>>>(U, w->z, e, 1.0, n, (float*)w->ut);
-      ++launches;
-      residual(w->ut, w->rt);
-      const float* base = (const float*)w->rb;
-      if (central) {
-        perturb_kernel<float><<<grid, NKB, 0, st>>>(U, w->z, e, -1.0, n, (float*)w->ut);
-        ++launches;
-        residual(w->ut, w->rm);
-        base = (const float*)w->rm;
-      }
-      jvp_combine_kernel<float, TV><<<grid, NKB, 0, st>>>(v, (const float*)w->rt, base, e,
-                                                          central ? 2.0 : 1.0, n, wout, dinv, w->z, N);
-    }
-    ++launches;
+    jvp_combine_kernel<T, TV, TV><<<cells(), NKB, 0, st>>>(v, (const T*)w->rt, (const T*)(central ? other : base), e + 1,
+                                                        central ? 0.5 : 1.0, N, wout,
+                                                        precond == 1 ? w->line : nullptr, w->z);
+    launches += 2;
   }
 };
 
@@ -948,7 +1200,7 @@ void base_residual(Ctx& c, const double* U, bool outer64) {
   if (c.g->d.precision == CRN_FP64) {
     c.residual(U, c.w->b);
   } else {
-    perturb_kernel<float><<<c.grid, NKB, 0, c.st>>>(U, nullptr, nullptr, 0.0, c.n, (float*)c.w->ut);
+    cast_kernel<float><<<c.grid, NKB, 0, c.st>>>(U, c.n, (float*)c.w->ut);
     ++c.launches;
     c.residual(c.w->ut, c.w->rb);
     if (outer64) {
@@ -970,10 +1222,10 @@ double gmres(Ctx& c, const double* U, const crn_nk_options& o, double b_rel, dou
   const bool central = o.fd_central != 0;
   NkWork* w = c.w;
   const int m = o.krylov_dim;
-  // FP32 basis (forward mode): V_j in Vf, the new Arnoldi vector in wf after
-  // its FP64 product; FP64 basis: V_j and the new vector in V
+  // FP32 basis (forward mode): V_j in Vf, the new Arnoldi vector rounded there
+  // after its FP64 product; FP64 basis: V_j and the new vector in V
   const bool f32 = c.mode == 0 && use_basis32(o) && w->Vf;
-  std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), gv(m + 1), y(m), h(m + 1), h2(m + 1);
+  std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), gv(m + 1), y(m), h(m + 1);
   auto Hat = [&](int i, int j) -> double& { return H[(size_t)i * m + j]; };
   // V_0 = r / beta from an FP64 vector r
   auto first = [&](const double* r, double beta) {
@@ -1008,49 +1260,22 @@ double gmres(Ctx& c, const double* U, const crn_nk_options& o, double b_rel, dou
     gv[0] = beta;
     int jdone = 0;
     for (int j = 0; j < m; ++j) {
-      double* vn = w->V + (size_t)(j + 1) * c.n;  // FP64 basis: the new vector in place
-      float* vf = w->wf;                          // FP32 basis: the new vector
+      // the new vector in place of V_(j+1); classical Gram-Schmidt, repeated
+      // once if the norm dropped by > 0.7
+      double after;
       if (f32) {
-        c.apply(w->Vf + (size_t)j * c.n, w->w, U, b_rel, central);
-        c.to32(vf, w->w, 1.0);
+        float* vn = w->Vf + (size_t)(j + 1) * c.n;
+        c.apply(w->Vf + (size_t)j * c.n, vn, U, b_rel, central);
+        after = c.orthonormalise(w->Vf, j + 1, vn, h.data());
       } else {
+        double* vn = w->V + (size_t)(j + 1) * c.n;
         c.apply(w->V + (size_t)j * c.n, vn, U, b_rel, central);
+        after = c.orthonormalise(w->V, j + 1, vn, h.data());
       }
       ++iters;
-      auto dots = [&](bool ww) { if (f32) c.dots32(j + 1, vf, ww); else c.dots(j + 1, vn, ww); };
-      auto combine = [&](const double* coef) {
-        if (f32) c.combine32(vf, coef, j + 1); else c.combine(vn, coef, j + 1);
-      };
-      auto norm = [&]() { return f32 ? c.norm32(vf) : c.norm(vn); };
-      // classical Gram-Schmidt, repeated once if the norm dropped by > 0.7
-      dots(true);
-      c.fetch(0, j + 1);
-      c.fetch(c.rows.ww, 1);
-      if (!c.ok()) return rel;
-      const double before = std::sqrt(std::max(w->host[c.rows.ww], 0.0));
-      for (int t = 0; t <= j; ++t) h[t] = w->host[t];
-      for (int t = 0; t <= j; ++t) h2[t] = -h[t];
-      combine(h2.data());
-      double after = norm();
-      if (after < 0.7 * before) {
-        dots(false);
-        c.fetch(0, j + 1);
-        if (!c.ok()) return rel;
-        for (int t = 0; t <= j; ++t) { h2[t] = -w->host[t]; h[t] += w->host[t]; }
-        combine(h2.data());
-        after = norm();
-      }
       if (!c.ok()) return rel;
       for (int t = 0; t <= j; ++t) Hat(t, j) = h[t];
       Hat(j + 1, j) = after;
-      if (after > 0.0) {
-        if (f32) {
-          c.to32(w->Vf + (size_t)(j + 1) * c.n, vf, 1.0 / after);
-        } else {
-          scale_kernel<<<c.grid, NKB, 0, c.st>>>(vn, vn, 1.0 / after, c.n);
-          ++c.launches;
-        }
-      }
       // Givens rotations on column j
       for (int t = 0; t < j; ++t) {
         const double a = Hat(t, j), bb = Hat(t + 1, j);
@@ -1075,7 +1300,7 @@ double gmres(Ctx& c, const double* U, const crn_nk_options& o, double b_rel, dou
       for (int q = t + 1; q < jdone; ++q) s -= Hat(t, q) * y[q];
       y[t] = Hat(t, t) != 0.0 ? s / Hat(t, t) : 0.0;
     }
-    if (f32) c.combine_x32(w->x, y.data(), jdone);
+    if (f32) c.combine_on(w->x, w->Vf, y.data(), jdone);
     else c.combine(w->x, y.data(), jdone);
     if (rel <= o.lin_rtol) break;
   }
@@ -1109,6 +1334,7 @@ int nk_step(crn_grid* g, double* U, double cfl, const crn_nk_options& o, crn_nk_
   stopped = false;
   cudaError_t e = ensure_work(g, o.krylov_dim);
   if (e == cudaSuccess && use_basis32(o)) e = ensure_basis32(g->nk);
+  if (e == cudaSuccess && o.fd_central != 0) e = ensure_central(g);
   if (e != cudaSuccess) return report(CRN_E_CUDA, std::string("Newton-Krylov workspace: ") + cudaGetErrorString(e));
   Ctx c(g, st);
   c.precond = o.precond;
@@ -1137,9 +1363,9 @@ int nk_step(crn_grid* g, double* U, double cfl, const crn_nk_options& o, crn_nk_
     ++c.launches;
     c.line_factor();
   }
-  absmean_kernel<<<w->nblk, NKB, 0, st>>>(U, c.N, w->part, w->nblk, c.rows.sumabs);
+  floors_kernel<<<(unsigned)std::min<int64_t>((c.N + NKB - 1) / NKB, w->nblk), NKB, 0, st>>>(
+      U, c.N, w->part, w->out, c.rows.floors, w->sync);
   ++c.launches;
-  c.finish(c.rows.sumabs, NV, 0);
   const bool outer64 = g->d.precision == CRN_FP32_BULK && o.outer_fp64 != 0;
   if (outer64) {  // the FP64 tiled kernels' shared-memory opt-in (an FP32-bulk grid skips it)
     e = prepare_fp64();
@@ -1171,13 +1397,7 @@ int nk_step(crn_grid* g, double* U, double cfl, const crn_nk_options& o, crn_nk_
   int iters = 0;
   const double rel = gmres(c, U, o, b_rel, bnorm, iters);
   // dU = P^-1 y (dtau . y, or the radial line solve)
-  if (o.precond == 1) {
-    c.line_solve(w->x, w->z);
-  } else {
-    precond_kernel<double><<<w->nblk, NKB, 0, st>>>(w->x, w->dtau, c.N, w->z, U, w->out + c.rows.sumabs, gm1,
-                                            w->part, w->nblk, c.rows.minr, 0);
-    ++c.launches;
-  }
+  c.precondition(w->x, w->z);
   // step length: relative-change limiter, then positivity
   double alpha = 1.0;
   if (o.max_rel_change > 0.0) {
@@ -1269,7 +1489,7 @@ void sensitivity(Ctx& c, double* sens) {
   if (g->d.precision == CRN_FP64) {
     e = launch_vjp_fp64(g, (const double*)w->ut, w->z, w->w, sens, c.st, &nl);
   } else {
-    perturb_kernel<float><<<c.grid, NKB, 0, c.st>>>(w->z, nullptr, nullptr, 0.0, c.n, (float*)w->rm);
+    cast_kernel<float><<<c.grid, NKB, 0, c.st>>>(w->z, c.n, (float*)w->rm);
     ++c.launches;
     e = launch_vjp_fp32(g, (const float*)w->ut, (const float*)w->rm, (float*)w->rt, sens, c.st, &nl);
   }
@@ -1324,7 +1544,7 @@ int adjoint_fgmres(Ctx& c, const double* U, const double* gbar, double* lam, dou
     }
     w->mf = mf;
   }
-  std::vector<double> H((size_t)(mf + 1) * mf), cs(mf), sn(mf), gv(mf + 1), y(mf), h(mf + 1), h2(mf + 1);
+  std::vector<double> H((size_t)(mf + 1) * mf), cs(mf), sn(mf), gv(mf + 1), y(mf), h(mf + 1);
   auto Hat = [&](int i, int j) -> double& { return H[(size_t)i * mf + j]; };
   for (;;) {
     // the true residual of the current lambda
@@ -1353,39 +1573,14 @@ int adjoint_fgmres(Ctx& c, const double* U, const double* gbar, double* lam, dou
       int it = 0;
       gmres(c, U, inner, 0.0, 1.0, it);
       kry += it;
-      if (o.precond == 1) {
-        c.line_solve(w->x, zj);
-      } else {
-        precond_kernel<double><<<w->nblk, NKB, 0, c.st>>>(w->x, w->dtau, c.N, zj, nullptr, nullptr, 0.0, w->part,
-                                                          w->nblk, c.rows.minr, 0);
-        ++c.launches;
-      }
+      c.precondition(w->x, zj);
       ++pass;
       outer_vjp(zj, vn);  // J^T z_j
       // classical Gram-Schmidt against v_0 .. v_j, repeated once if the norm dropped by > 0.7
-      c.dots_on(w->fv, j + 1, vn, true);
-      c.fetch(0, j + 1);
-      c.fetch(c.rows.ww, 1);
-      if (!c.ok()) return report(CRN_E_CUDA, std::string("adjoint solve: ") + cudaGetErrorString(c.err));
-      const double before = std::sqrt(std::max(w->host[c.rows.ww], 0.0));
-      for (int t = 0; t <= j; ++t) { h[t] = w->host[t]; h2[t] = -h[t]; }
-      c.combine_on(vn, w->fv, h2.data(), j + 1);
-      double after = c.norm(vn);
-      if (after < 0.7 * before) {
-        c.dots_on(w->fv, j + 1, vn, false);
-        c.fetch(0, j + 1);
-        if (!c.ok()) return report(CRN_E_CUDA, std::string("adjoint solve: ") + cudaGetErrorString(c.err));
-        for (int t = 0; t <= j; ++t) { h2[t] = -w->host[t]; h[t] += w->host[t]; }
-        c.combine_on(vn, w->fv, h2.data(), j + 1);
-        after = c.norm(vn);
-      }
+      const double after = c.orthonormalise(w->fv, j + 1, vn, h.data());
       if (!c.ok()) return report(CRN_E_CUDA, std::string("adjoint solve: ") + cudaGetErrorString(c.err));
       for (int t = 0; t <= j; ++t) Hat(t, j) = h[t];
       Hat(j + 1, j) = after;
-      if (after > 0.0) {
-        scale_kernel<<<c.grid, NKB, 0, c.st>>>(vn, vn, 1.0 / after, c.n);
-        ++c.launches;
-      }
       for (int t = 0; t < j; ++t) {
         const double a = Hat(t, j), bb = Hat(t + 1, j);
         Hat(t, j) = cs[t] * a + sn[t] * bb;
@@ -1442,7 +1637,7 @@ int adjoint_pseudo_time(crn_grid* g, const double* U, const double* gbar, double
   } else {
     local_dt_kernel<float><<<c.grid, NKB, 0, st>>>(g->shape, g->g32.geo, g->d.gamma, g->d.c_h, U,
                                                    o.adjoint_cfl, w->dtau);
-    perturb_kernel<float><<<c.grid, NKB, 0, st>>>(U, nullptr, nullptr, 0.0, c.n, (float*)w->ut);
+    cast_kernel<float><<<c.grid, NKB, 0, st>>>(U, c.n, (float*)w->ut);
     ++c.launches;
   }
   ++c.launches;
@@ -1491,13 +1686,7 @@ int adjoint_pseudo_time(crn_grid* g, const double* U, const double* gbar, double
     int it = 0;
     gmres(c, U, inner, 0.0, rel * gnorm, it);
     kry += it;
-    if (o.precond == 1) {
-      c.line_solve(w->x, w->z);
-    } else {
-      precond_kernel<double><<<w->nblk, NKB, 0, st>>>(w->x, w->dtau, c.N, w->z, nullptr, nullptr, 0.0, w->part,
-                                                      w->nblk, c.rows.minr, 0);
-      ++c.launches;
-    }
+    c.precondition(w->x, w->z);
     add_kernel<<<c.grid, NKB, 0, st>>>(lam, w->z, c.n);
     ++c.launches;
   }
@@ -1558,7 +1747,7 @@ int adjoint_solve(crn_grid* g, const double* U, const double* gbar, double* lamb
     cudaMemcpyAsync(w->ut, U, sizeof(double) * c.n, cudaMemcpyDeviceToDevice, st);
   } else {
     local_dt_kernel<float><<<c.grid, NKB, 0, st>>>(g->shape, g->g32.geo, g->d.gamma, g->d.c_h, U, 1.0, w->dtau);
-    perturb_kernel<float><<<c.grid, NKB, 0, st>>>(U, nullptr, nullptr, 0.0, c.n, (float*)w->ut);
+    cast_kernel<float><<<c.grid, NKB, 0, st>>>(U, c.n, (float*)w->ut);
     ++c.launches;
   }
   ++c.launches;
@@ -1568,13 +1757,7 @@ int adjoint_solve(crn_grid* g, const double* U, const double* gbar, double* lamb
   int iters = 0;
   const double rel = gmres(c, U, o, 0.0, bnorm, iters);
   // lambda = P_a^-1 y (dt . y, or the transposed line solve)
-  if (o.precond == 1) {
-    c.line_solve(w->x, w->z);
-  } else {
-    precond_kernel<double><<<w->nblk, NKB, 0, st>>>(w->x, w->dtau, c.N, w->z, nullptr, nullptr, 0.0, w->part, w->nblk,
-                                            c.rows.minr, 0);
-    ++c.launches;
-  }
+  c.precondition(w->x, w->z);
   if (lambda) cudaMemcpyAsync(lambda, w->z, sizeof(double) * c.n, cudaMemcpyDeviceToDevice, st);
   if (sens) sensitivity(c, sens);  // (dR/dB_b)^T lambda from one more VJP, negated
   if (!c.ok()) return report(CRN_E_CUDA, std::string("adjoint solve: ") + cudaGetErrorString(c.err));

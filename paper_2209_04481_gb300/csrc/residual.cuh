@@ -24,7 +24,7 @@ namespace crn {
 // where the reductions and error reports go
 struct Reduce {
   double* partials;          // [gridDim.x * gridDim.y][16]
-  unsigned int* counter;     // CTA arrival counter, reset by the last CTA
+  unsigned int* counter;     // CTA arrival counter, reset by the last CTA; null: no reductions (tiled kernel)
   double* norms_out;         // [9] L2 norms (always written)
   double* dt_out;            // [1] min V / sum lambda |S| (always written)
   double* norms_user;        // optional copy for the caller
@@ -850,6 +850,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
     __syncthreads();
   }
   // ---------------- reductions: warp tree in T, then FP64 across warps and CTAs
+  if (red.counter == nullptr) return;  // the caller wants R alone
   T dtm = (T)INFINITY;
   if (rate > (T)0) dtm = sizeof(T) == 4 ? (T)__frcp_rn((float)rate) : one / rate;
 #pragma unroll
@@ -862,14 +863,17 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
   reduce_and_finalize_at<NT>(sq, dtm, red, reinterpret_cast<double*>(smem_raw), bid, nblocks);
 }
 
-// one grid: block (x, y) = (tile, radial chunk)
+// one grid: block (x, y) = (tile, radial chunk); with a second state, block z
+// picks the state
 template <class T, int LIM, int TT, int TP>
 __global__ void __launch_bounds__(TT * TP, (MinCtas<T, TT * TP>::value))
 residual_tiled(Shape sh, Geo<T> g, Phys<T> ph, const double* __restrict__ Br,
-               const T* __restrict__ U, T* __restrict__ R, Reduce red, int kchunk) {
+               const T* __restrict__ U, T* __restrict__ R, Reduce red, int kchunk, const T* __restrict__ U2,
+               T* __restrict__ R2) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  tiled_item<T, LIM, TT, TP>(sh, g, ph, Br, U, R, red, kchunk, blockIdx.x, blockIdx.y,
-                             blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y, smem_raw);
+  tiled_item<T, LIM, TT, TP>(sh, g, ph, Br, blockIdx.z == 0 ? U : U2, blockIdx.z == 0 ? R : R2, red, kchunk,
+                             blockIdx.x, blockIdx.y, blockIdx.y * gridDim.x + blockIdx.x,
+                             gridDim.x * gridDim.y, smem_raw);
 }
 
 // ---------------------------------------------------------------------------

@@ -116,6 +116,16 @@ cudaError_t launch_residual_fp32(crn_grid* g, const float* U, float* R, double* 
   g->last_kernel = g->d.kernel == CRN_KERNEL_CELLWISE ? CRN_KERNEL_CELLWISE : CRN_KERNEL_TILED_REGS;
   return launch_residual_t<float>(g, U, R, norms_user, dt_user, st, nlaunch);
 }
+cudaError_t launch_residual_pair_fp32(crn_grid* g, const float* Ua, float* Ra, const float* Ub, float* Rb,
+                                      cudaStream_t st, int* nlaunch) {
+  if (g->d.kernel != CRN_KERNEL_CELLWISE && !g->cfg.staged)
+    return launch_pair_t<float>(g, Ua, Ra, Ub, Rb, st, nlaunch);
+  int nl = 0;
+  cudaError_t e = launch_residual_fp32(g, Ua, Ra, nullptr, nullptr, st, nlaunch);
+  if (e == cudaSuccess) e = launch_residual_fp32(g, Ub, Rb, nullptr, nullptr, st, &nl);
+  *nlaunch += nl;
+  return e;
+}
 size_t tiled_smem_fp32() { return tiled_smem_t<float>(); }
 cudaError_t prepare_fp32() {
   cudaError_t e = prepare_t<float>();

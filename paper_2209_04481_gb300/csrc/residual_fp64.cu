@@ -7,6 +7,15 @@ cudaError_t launch_residual_fp64(crn_grid* g, const double* U, double* R, double
   g->last_kernel = g->d.kernel == CRN_KERNEL_CELLWISE ? CRN_KERNEL_CELLWISE : CRN_KERNEL_TILED_REGS;
   return launch_residual_t<double>(g, U, R, norms_user, dt_user, st, nlaunch);
 }
+cudaError_t launch_residual_pair_fp64(crn_grid* g, const double* Ua, double* Ra, const double* Ub, double* Rb,
+                                      cudaStream_t st, int* nlaunch) {
+  if (g->d.kernel != CRN_KERNEL_CELLWISE) return launch_pair_t<double>(g, Ua, Ra, Ub, Rb, st, nlaunch);
+  int nl = 0;
+  cudaError_t e = launch_residual_fp64(g, Ua, Ra, nullptr, nullptr, st, nlaunch);
+  if (e == cudaSuccess) e = launch_residual_fp64(g, Ub, Rb, nullptr, nullptr, st, &nl);
+  *nlaunch += nl;
+  return e;
+}
 size_t tiled_smem_fp64() { return tiled_smem_t<double>(); }
 cudaError_t prepare_fp64() { return prepare_t<double>(); }
 int tiled_ctas_per_sm_fp64(int limiter) { return tiled_ctas_t<double>(limiter); }

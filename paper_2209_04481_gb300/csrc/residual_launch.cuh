@@ -52,8 +52,36 @@ cudaError_t launch_lim(crn_grid* g, const T* U, T* R, double* nu, double* du, cu
   const int kc = g->cfg.kchunk_tiled;
   const int nch = (sh.nr + kc - 1) / kc;
   dim3 grid((unsigned)ntiles, (unsigned)nch);
-  residual_tiled<T, LIM, TT, TP><<<grid, D::NT, smem, st>>>(sh, geo, ph, g->br, U, R, red, kc);
+  residual_tiled<T, LIM, TT, TP><<<grid, D::NT, smem, st>>>(sh, geo, ph, g->br, U, R, red, kc, nullptr, nullptr);
   return cudaGetLastError();
+}
+
+// R = R(U) and R2 = R(U2) in one launch (grid z = state): the two together fill
+// an SM that one small state leaves half empty, and share one tail
+template <class T, int LIM>
+cudaError_t launch_pair_lim(crn_grid* g, const T* U, T* R, const T* U2, T* R2, cudaStream_t st) {
+  const Shape sh = g->shape;
+  Reduce red = make_reduce(g, nullptr, nullptr);
+  red.counter = nullptr;  // no norms, no dtmin
+  constexpr int TT = TileFor<T>::TT, TP = TileFor<T>::TP;
+  using D = TileDims<TT, TP>;
+  const int ntiles = ((sh.nt + TT - 1) / TT) * ((sh.np + TP - 1) / TP);
+  const int kc = g->cfg.kchunk_pair;
+  const dim3 grid((unsigned)ntiles, (unsigned)((sh.nr + kc - 1) / kc), 2);
+  residual_tiled<T, LIM, TT, TP><<<grid, D::NT, D::template smem_bytes<T>(), st>>>(
+      sh, geo_of<T>(g), phys_of<T>(g), g->br, U, R, red, kc, U2, R2);
+  return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_pair_t(crn_grid* g, const T* U, T* R, const T* U2, T* R2, cudaStream_t st, int* nlaunch) {
+  *nlaunch = 1;
+  g->last_kernel = CRN_KERNEL_TILED_REGS;
+  switch (g->d.limiter) {
+    case CRN_LIM_NONE: return launch_pair_lim<T, 0>(g, U, R, U2, R2, st);
+    case CRN_LIM_MINMOD: return launch_pair_lim<T, 1>(g, U, R, U2, R2, st);
+    default: return launch_pair_lim<T, 2>(g, U, R, U2, R2, st);
+  }
 }
 
 template <class T>

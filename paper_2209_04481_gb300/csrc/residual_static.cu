@@ -326,13 +326,16 @@ int run(const crn_grid_desc& d, DeviceSlot& slot, const double* Br, const void* 
   T* r = static_cast<T*>(R);
   switch (d.limiter) {
     case CRN_LIM_NONE:
-      crn::residual_tiled<T, 0, TT, TP><<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc);
+      crn::residual_tiled<T, 0, TT, TP><<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc, nullptr,
+                                                                          nullptr);
       break;
     case CRN_LIM_MINMOD:
-      crn::residual_tiled<T, 1, TT, TP><<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc);
+      crn::residual_tiled<T, 1, TT, TP><<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc, nullptr,
+                                                                          nullptr);
       break;
     default:
-      crn::residual_tiled<T, 2, TT, TP><<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc);
+      crn::residual_tiled<T, 2, TT, TP><<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc, nullptr,
+                                                                          nullptr);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(CRN_E_CUDA, std::string("residual launch: ") + cudaGetErrorString(e));
