@@ -177,10 +177,11 @@ int crn_residual(crn_grid* g, const void* U_dev, void* R_dev, double* norms9_dev
  * CRN_FP32_BULK grids run the tiled VJP: a radial pass over blocks of 16
  * columns x 13 planes and a lateral pass over 8 x 32 (theta, phi) tiles of
  * one plane, every intermediate in shared memory; no scratch, 2 launches.
- * CRN_FP64 grids (and grids created with CRN_KERNEL_CELLWISE) run the
- * face/cell pair: one thread per face, then one per cell, 3 launches (2 with
- * FP32), with a scratch of 36 values of the grid's type per face (about 108
- * per cell) allocated by the grid's first VJP call: make that call before
+ * CRN_FP64 grids (and grids created with CRN_KERNEL_CELLWISE) run three
+ * passes, one thread per cell, per face and per cell again, 3 launches (2 with
+ * FP32, which forms its slopes where they are used), with a scratch of about 144
+ * values of the grid's type per cell (54 with FP32) allocated by the grid's
+ * first VJP call: make that call before
  * any stream capture.  The environment variable CRN_VJP_KERNEL ("tiled" or
  * "faces"), read at each call, overrides the choice.  Ubar_dev must not
  * overlap U_dev or Rbar_dev (CRN_E_ARG).  Asynchronous. */

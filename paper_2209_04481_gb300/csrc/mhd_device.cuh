@@ -85,9 +85,13 @@ template <> __device__ __forceinline__ float fmat<float>(float a, float b, float
 //   1/x: y0 (1 + e + e^2) with e = 1 - x y0 (Newton's series cut after e^2:
 //        error e^3 ~ 2^-60), 3 operations, within one unit in the last place;
 //        x finite and nonzero.
-//   sqrt x: g (1 + e/2 + 3 e^2/8) with g = x y0, e = 1 - g y0 (the binomial
-//        series of (1 - e)^(-1/2)), 5 operations, within one unit in the last
-//        place; 0 below the normal range, NaN for x < 0.
+//   sqrt x: Goldschmidt's step on g = x y0 and h = y0 / 2 (y0 ~ 1 / sqrt x), then
+//        Newton's with the exact remainder x - g^2: 6 operations (h halves an
+//        exponent), correctly rounded but for values next to a rounding
+//        boundary.  In particular the square root of a rounded square is its
+//        base: with it a face state of negative pressure and B_n = 0 keeps c_f = 0
+//        where a last place less would make q + sqrt(q^2) negative.  0 below
+//        the normal range, NaN for x < 0.
 template <class T> __device__ __forceinline__ T frcp(T x);
 template <> __device__ __forceinline__ double frcp<double>(double x) {
   double y;
@@ -100,9 +104,11 @@ template <class T> __device__ __forceinline__ T fsqrt(T x);
 template <> __device__ __forceinline__ double fsqrt<double>(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));
   const double g = x * y;
-  const double e = fma(-g, y, 1.0);
-  const double r = fma(g * e, fma(e, 0.375, 0.5), g);
+  const double e = fma(-h, g, 0.5);
+  const double g1 = fma(g, e, g);
+  const double r = fma(fma(-g1, g1, x), fma(h, e, h), g1);
   return (__double2hiint(x) & 0x7ff00000) == 0 ? 0.0 : r;
 }
 template <> __device__ __forceinline__ float fsqrt<float>(float x) { return sqrtf(x); }
@@ -304,7 +310,7 @@ __device__ __forceinline__ T limited_slope(T a, T b, T eps) {
 // slowest pipe, so its operations are counted: h = |S|/2 is multiplied into
 // u_n, B_n and rho u_n once per side instead of into each of the nine sums, and
 // the pressure and GLM gradient terms of both sides are added before they meet
-// the normal (159 operations against about 200; every FMA explicit).  FP32
+// the normal (159 operations and 4 for the square roots against about 200; every FMA explicit).  FP32
 // keeps the sums by side: there the regrouping saved 3 % and moved the momentum
 // of the polar cells, whose opposite faces nearly cancel, by 1e-7 per step.
 // ---------------------------------------------------------------------------

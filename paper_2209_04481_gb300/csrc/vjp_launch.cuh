@@ -20,10 +20,10 @@ template <> inline const Phys<float>& vphys<float>(const crn_grid* g) { return g
 // Which VJP a grid runs.  FP32-bulk grids: the tiled two-pass VJP of
 // vjp_tiled.cuh (issue-bound; its on-chip intermediates replace 864 B/cell of
 // face scratch that would not fit in L2 at production sizes).  FP64 grids:
-// the face/cell pair of vjp.cuh, which evaluates each face exactly once; on
-// the FP64 pipe (1/64 of the FP32 rate) the tiled pass's redundant halo faces
-// cost more than its scratch traffic saves.  Grids created with the
-// cell-wise reference kernel take the face/cell pair too.  CRN_VJP_KERNEL
+// the slope/face/cell passes of vjp.cuh, which evaluate each slope and face
+// exactly once; on the FP64 pipe (1/64 of the FP32 rate) the tiled pass's
+// redundant halo faces cost more than its scratch traffic saves.  Grids created
+// with the cell-wise reference kernel take those passes too.  CRN_VJP_KERNEL
 // ("tiled" or "faces") overrides the choice.
 inline bool vjp_uses_scratch(const crn_grid* g) {
   if (const char* e = std::getenv("CRN_VJP_KERNEL")) {
@@ -33,10 +33,10 @@ inline bool vjp_uses_scratch(const crn_grid* g) {
   return g->d.kernel == CRN_KERNEL_CELLWISE || g->d.precision == CRN_FP64;
 }
 
-inline size_t vjp_scratch_elems(const Shape& s) {
+inline size_t vjp_scratch_elems(const Shape& s, bool fp64) {
   const size_t cs = (size_t)s.nt * s.np;
-  return (size_t)4 * NV * ((size_t)(s.nr + 1) * cs + (size_t)s.nr * (s.nt + 1) * s.np + (size_t)s.nr * cs) +
-         (size_t)NV * s.ncell;
+  return (size_t)2 * NV * ((size_t)(s.nr + 1) * cs + (size_t)s.nr * (s.nt + 1) * s.np + (size_t)s.nr * cs) +
+         (fp64 ? (size_t)10 * NV * s.ncell : 0);
 }
 
 template <class T, int LIM>
@@ -44,21 +44,23 @@ cudaError_t vjp_lim(crn_grid* g, const T* U, const T* Rb, T* Ub, double* Brb, cu
                     int* nl) {
   const Shape sh = g->shape;
   const size_t cs = (size_t)sh.nt * sh.np;
-  T* base = static_cast<T*>(g->vjp_buf);
+  // FP64 keeps the slopes of the first pass; FP32 (the reference variant there)
+  // forms them again where they are used
+  constexpr bool STORED = sizeof(T) == 8;
   VjpBufs<T> b;
-  b.cr = base;
-  b.ct = b.cr + (size_t)4 * NV * (sh.nr + 1) * cs;
-  b.cp = b.ct + (size_t)4 * NV * sh.nr * (sh.nt + 1) * sh.np;
-  // FP64: recover the primitives once (each FP64 division is costly); FP32:
-  // recovery inside the face pass is cheaper than one more pass over memory
-  b.W = sizeof(T) == 8 ? b.cp + (size_t)4 * NV * sh.nr * cs : nullptr;
-  if (b.W) vjp_prims<T><<<(unsigned)((sh.ncell + 255) / 256), 256, 0, st>>>(sh, vphys<T>(g), U, b.W);
+  b.fr = static_cast<T*>(g->vjp_buf);
+  b.ft = b.fr + (size_t)2 * NV * (sh.nr + 1) * cs;
+  b.fp = b.ft + (size_t)2 * NV * sh.nr * (sh.nt + 1) * sh.np;
+  b.W = b.fp + (size_t)2 * NV * sh.nr * cs;
+  b.S = b.W + (size_t)NV * sh.ncell;
+  const unsigned nbc = (unsigned)((sh.ncell + 127) / 128);
+  if constexpr (STORED)
+    vjp_slopes<T, LIM><<<dim3(nbc, 3), 128, 0, st>>>(sh, vgeo<T>(g), vphys<T>(g), g->br, U, b);
   const int64_t nf = (int64_t)(sh.nr + 1) * (int64_t)cs + (int64_t)sh.nr * (sh.nt + 1) * sh.np +
                      (int64_t)sh.nr * (int64_t)cs;
-  vjp_faces<T, LIM><<<(unsigned)((nf + 127) / 128), 128, 0, st>>>(sh, vgeo<T>(g), vphys<T>(g), g->br, U, Rb, b);
-  const unsigned nbc = (unsigned)((sh.ncell + 127) / 128);
-  vjp_cells<T><<<nbc, 128, 0, st>>>(sh, vgeo<T>(g), vphys<T>(g), g->br, U, Rb, b, Ub, Brb);
-  *nl = b.W ? 3 : 2;
+  vjp_faces<T, LIM, STORED><<<(unsigned)((nf + 127) / 128), 128, 0, st>>>(sh, vgeo<T>(g), vphys<T>(g), g->br, U, Rb, b);
+  vjp_cells<T, LIM, STORED><<<nbc, 128, 0, st>>>(sh, vgeo<T>(g), vphys<T>(g), g->br, U, Rb, b, Ub, Brb);
+  *nl = STORED ? 3 : 2;
   return cudaGetLastError();
 }
 

@@ -43,6 +43,12 @@ def test_within_one_ulp(ops):
     assert np.all(np.abs(rcp + 1.0 / x) <= np.spacing(1.0 / x))
 
 
+def test_root_of_a_rounded_square_is_its_base(ops):
+    m = np.random.default_rng(2).uniform(1.0, 2.0, 300000) * 2.0 ** np.random.default_rng(3).integers(-100, 100, 300000)
+    _, root = ops(m * m)
+    assert np.array_equal(root, m)
+
+
 def test_edge_values(ops):
     _, root = ops(np.array([0.0, -0.0, 5e-324, -1.0, np.nan]))
     assert root[0] == 0.0 and root[1] == 0.0 and root[2] == 0.0
