@@ -115,16 +115,24 @@ template <> __device__ __forceinline__ float fsqrt<float>(float x) { return sqrt
 
 // Comparisons of FP64 values on the integer pipe (an FP64 compare takes a slot
 // of the FP64 pipe): positive doubles order as their bit patterns.
-// positive(x): x > 0; greater(x, y): x > y for y >= 0; both false for a NaN x.
+// positive(x): x > 0; greater(x, y): x > y for y >= +0.  Both false for a NaN of
+// either sign: as unsigned numbers NaNs and negative values lie above +inf.
 __device__ __forceinline__ bool positive(float x) { return x > 0.f; }
 __device__ __forceinline__ bool positive(double x) {
-  const long long b = __double_as_longlong(x);
-  return b > 0 && b <= 0x7ff0000000000000ll;
+  return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7ff0000000000000ull;
 }
 __device__ __forceinline__ bool greater(float x, float y) { return x > y; }
 __device__ __forceinline__ bool greater(double x, double y) {
-  const long long b = __double_as_longlong(x);
-  return b > __double_as_longlong(y) && b <= 0x7ff0000000000000ll;
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return b > (unsigned long long)__double_as_longlong(y) && b <= 0x7ff0000000000000ull;
+}
+
+// |x| to FP32, cut off (not rounded), by integer instructions: 0 below the FP32
+// normal range, +inf above it and for NaN
+__device__ __forceinline__ float magnitude_f32(double x) {
+  const int e = (__double2hiint(x) & 0x7fffffff) - 0x38000000;
+  const unsigned b = __funnelshift_l((unsigned)__double2loint(x), (unsigned)e, 3);
+  return __uint_as_float(e < 0x00100000 ? 0u : (e < 0x0ff00000 ? b : 0x7f800000u));
 }
 
 // ---------------------------------------------------------------------------
@@ -345,6 +353,38 @@ __device__ __forceinline__ Side<float> side_terms(const float (&w)[NV], float nx
   return s;
 }
 
+// Whether a face state's signal speed is certainly below c_h, from an FP32 bound:
+// for rho, p > 0, |u_n| + c_f <= |u_n| + sqrt(a^2 + B^2 / rho).  Then lambda = c_h
+// and the FP64 fast speed (24 operations a side) need not be formed: both sides
+// of three faces in four of a solar-wind shell.  The bound costs about 25
+// integer and FP32 instructions, less than one FP64 operation; its margins
+// (1e-5 of the squares, 1e-6 c_h) cover every rounding in it.
+__device__ __forceinline__ bool speed_below_ch(double rho, double p, double un, double b2, const Phys<double>& ph) {
+  const float r = magnitude_f32(rho), c = magnitude_f32(ph.ch);
+  const float t = fmaf(-1e-6f, c, c) - magnitude_f32(un);
+  const float q = fmaf(magnitude_f32(ph.gamma), magnitude_f32(p), magnitude_f32(b2));
+  return (__double2hiint(rho) | __double2hiint(p)) >= 0 && r > 1e-20f && t > 0.f &&
+         t * t * r > fmaf(1.00001f, q, 1e-18f * r);
+}
+
+// An FP32 estimate of |u_n| + c_f and a bound of its error, to tell which side of
+// a face has the larger speed: only that side's is then formed in FP64.  Where
+// the discriminant (a^2 - B^2/rho)^2 + 4 a^2 (B^2 - B_n^2)/rho nears zero its
+// rounding, 1e-7 of q^2, moves the root by 1e-7 q^2 / root.  The error is
+// infinite (either side may be larger) for rho, p <= 0 and out of FP32's range.
+__device__ __forceinline__ float speed_estimate(double rho, double p, double un, double bn, double b2,
+                                                const Phys<double>& ph, float& err) {
+  const float r = magnitude_f32(rho), ir = __fdividef(1.f, r), u = magnitude_f32(un), b = magnitude_f32(bn);
+  const float a2 = magnitude_f32(ph.gamma) * magnitude_f32(p) * ir, br = magnitude_f32(b2) * ir;
+  const float q = a2 + br, d = a2 - br;
+  const float root = sqrtf(fmaxf(fmaf(d, d, 4.f * a2 * fmaf(-b * ir, b, br)), 0.f));
+  const float cf = sqrtf(0.5f * (q + root));
+  err = fmaf(cf, fmaf(2e-6f, __fdividef(q, root), 2e-6f), 1e-6f * u);
+  if (!((__double2hiint(rho) | __double2hiint(p)) >= 0 && r > 1e-20f && q > 1e-15f && q < 1e15f && err < 1e15f))
+    err = INFINITY;
+  return u + cf;
+}
+
 template <bool NZ>
 __device__ __forceinline__ double dot_n(const double* w, double nx, double ny, double nz) {
   return NZ ? fma(w[0], nx, fma(w[1], ny, w[2] * nz)) : fma(w[0], nx, w[1] * ny);
@@ -353,6 +393,17 @@ __device__ __forceinline__ double dot3(const double* a, const double* b) {
   return fma(a[0], b[0], fma(a[1], b[1], a[2] * b[2]));
 }
 
+// |u_n| + c_f: c_f^2 = (q + sqrt(q^2 - 4 a^2 B_n^2 / rho)) / 2, q = a^2 + B^2 / rho
+__device__ __forceinline__ double signal_speed(double rho, double p, double un, double bn, double b2,
+                                               const Phys<double>& ph) {
+  const double ir = frcp(rho);
+  const double a2 = (ph.gamma * p) * ir;
+  const double q = fma(b2, ir, a2);
+  const double disc = fma(-4.0 * (a2 * ir), bn * bn, q * q);
+  return fabs(un) + fsqrt(0.5 * (q + fsqrt(positive(disc) ? disc : 0.0)));
+}
+
+// sp holds B^2
 template <bool NZ>
 __device__ __forceinline__ Side<double> side_terms(const double (&w)[NV], double nx, double ny, double nz,
                                                    const Phys<double>& ph) {
@@ -360,17 +411,10 @@ __device__ __forceinline__ Side<double> side_terms(const double (&w)[NV], double
   s.un = dot_n<NZ>(w + 1, nx, ny, nz);
   s.bn = dot_n<NZ>(w + 4, nx, ny, nz);
   s.vb = dot3(w + 1, w + 4);
-  const double b2 = dot3(w + 4, w + 4);
+  s.sp = dot3(w + 4, w + 4);
   const double v2 = dot3(w + 1, w + 1);
-  s.pt = fma(0.5, b2, w[7]);
-  s.en = fma(0.5, fma(w[0], v2, b2), w[7] * ph.igm1);
-  // fast speed: c_f^2 = (q + sqrt(q^2 - 4 a^2 B_n^2 / rho)) / 2, q = a^2 + B^2 / rho
-  const double ir = frcp(w[0]);
-  const double a2 = (ph.gamma * w[7]) * ir;
-  const double q = fma(b2, ir, a2);
-  const double disc = fma(-4.0 * (a2 * ir), s.bn * s.bn, q * q);
-  const double cf = fsqrt(0.5 * (q + fsqrt(positive(disc) ? disc : 0.0)));
-  s.sp = fabs(s.un) + cf;
+  s.pt = fma(0.5, s.sp, w[7]);
+  s.en = fma(0.5, fma(w[0], v2, s.sp), w[7] * ph.igm1);
   return s;
 }
 
@@ -416,8 +460,23 @@ __device__ __forceinline__ void rusanov(const double (&wl)[NV], const double (&w
                                         double& lam_area) {
   const Side<double> L = side_terms<NZ>(wl, nx, ny, nz, ph);
   const Side<double> R = side_terms<NZ>(wr, nx, ny, nz, ph);
-  double lam = greater(L.sp, R.sp) ? L.sp : R.sp;
-  lam = greater(lam, ph.ch) ? lam : ph.ch;
+  double lam = ph.ch;
+  if (!(speed_below_ch(wl[0], wl[7], L.un, L.sp, ph) && speed_below_ch(wr[0], wr[7], R.un, R.sp, ph))) {
+    float el, er;
+    const float fl = speed_estimate(wl[0], wl[7], L.un, L.bn, L.sp, ph, el);
+    const float fr = speed_estimate(wr[0], wr[7], R.un, R.bn, R.sp, ph, er);
+    const bool left = fl > fr;
+    lam = signal_speed(left ? wl[0] : wr[0], left ? wl[7] : wr[7], left ? L.un : R.un, left ? L.bn : R.bn,
+                       left ? L.sp : R.sp, ph);
+    if (!(fabsf(fl - fr) > el + er)) {  // too close to tell: the other side too
+      const double o = signal_speed(left ? wr[0] : wl[0], left ? wr[7] : wl[7], left ? R.un : L.un,
+                                    left ? R.bn : L.bn, left ? R.sp : L.sp, ph);
+      // the larger, and the right one of a pair with a NaN left one
+      const double sl = left ? lam : o, sr = left ? o : lam;
+      lam = greater(sl, sr) ? sl : sr;
+    }
+    lam = greater(lam, ph.ch) ? lam : ph.ch;
+  }
   const double h = 0.5 * area;
   lam_area = lam * area;
   const double d = lam * h;

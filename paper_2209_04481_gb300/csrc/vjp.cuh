@@ -224,7 +224,6 @@ __device__ void rusanov_adjoint(const float (&wl)[NV], const float (&wr)[NV], fl
 template <bool NZ>
 __device__ __forceinline__ SideFwd<double> side_fwd(const double (&w)[NV], double nx, double ny, double nz, const Phys<double>& ph) {
   SideFwd<double> s;
-  s.ir = frcp(w[0]);
   s.un = fma(w[1], nx, w[2] * ny);
   s.bn = fma(w[4], nx, w[5] * ny);
   if (NZ) {
@@ -236,14 +235,19 @@ __device__ __forceinline__ SideFwd<double> side_fwd(const double (&w)[NV], doubl
   s.vb = fma(w[1], w[4], fma(w[2], w[5], w[3] * w[6]));
   s.pt = fma(0.5, s.b2, w[7]);
   s.en = fma(0.5, fma(w[0], s.v2, s.b2), w[7] * ph.igm1);
-  s.a2 = (ph.gamma * w[7]) * s.ir;
+  return s;
+}
+
+// the signal speed of a side and what its adjoint needs
+__device__ __forceinline__ void side_speed(double rho, double p, const Phys<double>& ph, SideFwd<double>& s) {
+  s.ir = frcp(rho);
+  s.a2 = (ph.gamma * p) * s.ir;
   s.sum = fma(s.b2, s.ir, s.a2);
   const double disc = fma(-4.0 * (s.a2 * s.ir), s.bn * s.bn, s.sum * s.sum);
   s.clamp = !positive(disc);
   s.sq = fsqrt(s.clamp ? 0.0 : disc);
   s.cf = fsqrt(0.5 * (s.sum + s.sq));
   s.sp = fabs(s.un) + s.cf;
-  return s;
 }
 
 // what both sides of a face share: h fb, d fb, and their sums along the normal
@@ -291,13 +295,19 @@ __device__ __forceinline__ void side_adjoint(const double (&w)[NV], const SideFw
 template <bool NZ = true>
 __device__ __forceinline__ void rusanov_adjoint(const double (&wl)[NV], const double (&wr)[NV], double nx, double ny, double nz, double area,
                                                 const Phys<double>& ph, const double (&fb)[NV], double (&wlb)[NV], double (&wrb)[NV]) {
-  const SideFwd<double> L = side_fwd<NZ>(wl, nx, ny, nz, ph);
-  const SideFwd<double> R = side_fwd<NZ>(wr, nx, ny, nz, ph);
+  SideFwd<double> L = side_fwd<NZ>(wl, nx, ny, nz, ph);
+  SideFwd<double> R = side_fwd<NZ>(wr, nx, ny, nz, ph);
   // lambda = max(max(sp_L, sp_R), c_h); a tie passes the derivative to the first argument
-  const bool selR = greater(R.sp, L.sp);
-  const double lam_s = selR ? R.sp : L.sp;
-  const bool useC = greater(ph.ch, lam_s);
-  const double lam = useC ? ph.ch : lam_s;
+  bool selR = false, useC = true;
+  double lam = ph.ch;
+  if (!(speed_below_ch(wl[0], wl[7], L.un, L.b2, ph) && speed_below_ch(wr[0], wr[7], R.un, R.b2, ph))) {
+    side_speed(wl[0], wl[7], ph, L);
+    side_speed(wr[0], wr[7], ph, R);
+    selR = greater(R.sp, L.sp);
+    const double lam_s = selR ? R.sp : L.sp;
+    useC = greater(ph.ch, lam_s);
+    lam = useC ? ph.ch : lam_s;
+  }
   const double h = 0.5 * area, d = lam * h;
   FaceBar c;
 #pragma unroll

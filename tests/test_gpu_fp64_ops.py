@@ -1,6 +1,7 @@
-"""The FP64 reciprocal and square root of mhd_device.cuh: within one unit in
-the last place of the correctly rounded result over the exponents a state can
-hold, and their edge values."""
+"""The FP64 building blocks of mhd_device.cuh: reciprocal and square root within
+one unit in the last place of the correctly rounded result over the exponents a
+state can hold, with their edge values; and the face's lambda, which forms only
+the signal speeds an FP32 bound leaves open, bit for bit that of both speeds."""
 import ctypes
 import os
 import subprocess
@@ -14,14 +15,19 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 
 
 @pytest.fixture(scope="module")
-def ops(tmp_path_factory):
+def lib(tmp_path_factory):
     from paper_2209_04481_gb300 import build
     out = str(tmp_path_factory.mktemp("ops") / "fp64_ops.so")
     subprocess.run([build.nvcc(), *build.ARCH, *build.COMMON, "-shared", "-o", out,
                     os.path.join(HERE, "fp64_ops_check.cu")], check=True)
     lib = ctypes.CDLL(out)
     lib.run_ops.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_int]
+    lib.run_lambdas.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_double] + [ctypes.c_void_p] * 2 + [ctypes.c_int]
+    return lib
 
+
+@pytest.fixture(scope="module")
+def ops(lib):
     def run(x):
         xd = torch.from_numpy(x).cuda()
         a, b = torch.empty_like(xd), torch.empty_like(xd)
@@ -53,3 +59,42 @@ def test_edge_values(ops):
     _, root = ops(np.array([0.0, -0.0, 5e-324, -1.0, np.nan]))
     assert root[0] == 0.0 and root[1] == 0.0 and root[2] == 0.0
     assert np.isnan(root[3]) and np.isnan(root[4])
+
+
+def _faces(kind, n, rng):
+    """Two primitive states per face; (9, n) each."""
+    if kind == "range":  # every magnitude a unit system could give
+        m = 10.0 ** rng.uniform(-30, 10, (9, n))
+    else:
+        m = 10.0 ** np.array([rng.uniform(-5, 0.5, n)] + [rng.uniform(-4, 0.5, n)] * 3 + [rng.uniform(-4, 0.5, n)] * 3
+                             + [rng.uniform(-7, -0.5, n), rng.uniform(-6, -2, n)])
+    wl = m * np.where(rng.random((9, n)) < 0.5, -1.0, 1.0)
+    wl[0], wl[7] = np.abs(wl[0]), np.abs(wl[7])
+    rel = {"close": 1e-6, "wind": 1e-2, "range": 1.0, "bad": 0.3}[kind]
+    wr = wl * (1.0 + rel * rng.standard_normal((9, n)))
+    if kind == "close":
+        wr[:, ::3] = wl[:, ::3]              # equal sides
+    if kind == "bad":                        # negative, zero, infinite and NaN entries
+        for w in (wl, wr):
+            for v, x in ((0, -1.0), (7, -1.0), (0, 0.0), (7, 0.0), (0, np.nan), (7, np.inf), (5, np.nan), (2, np.inf)):
+                hit = rng.random(n) < 0.05
+                w[v, hit] = x if not np.isfinite(x) else x * w[v, hit]
+    return wl, wr
+
+
+@pytest.mark.parametrize("kind", ["wind", "close", "range", "bad"])
+@pytest.mark.parametrize("ch", [1.0, 0.0, 0.05, 30.0])
+def test_lambda_is_that_of_both_speeds(lib, kind, ch):
+    n = 60000
+    rng = np.random.default_rng(11)
+    wl, wr = _faces(kind, n, rng)
+    nrm = rng.standard_normal((3, n))
+    nrm /= np.linalg.norm(nrm, axis=0)
+    nrm[:, ::7] = np.array([1.0, 0.0, 0.0])[:, None]
+    d = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (wl, wr, nrm)]
+    lam, ref = torch.empty(n, dtype=torch.float64, device="cuda"), torch.empty(n, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    assert lib.run_lambdas(d[0].data_ptr(), d[1].data_ptr(), d[2].data_ptr(), ch, lam.data_ptr(), ref.data_ptr(), n) == 0
+    a, b = lam.cpu().numpy(), ref.cpu().numpy()
+    bad = ~((a == b) | (np.isnan(a) & np.isnan(b)))
+    assert not bad.any(), (int(bad.sum()), a[bad][:4], b[bad][:4], wl[:, bad][:, :2], wr[:, bad][:, :2])
