@@ -38,6 +38,16 @@ extern "C" int run_lambdas(const double* wl, const double* wr, const double* nrm
   return (int)cudaDeviceSynchronize();
 }
 
+__global__ void quotients(const double* a, const double* b, double* q, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) q[i] = crn::quotient(a[i], b[i]);
+}
+
+extern "C" int run_quotients(const double* a, const double* b, double* q, int n) {
+  quotients<<<(n + 255) / 256, 256>>>(a, b, q, n);
+  return (int)cudaDeviceSynchronize();
+}
+
 extern "C" int run_ops(const double* x, double* rcp, double* root, int n) {
   ops<<<(n + 255) / 256, 256>>>(x, rcp, root, n);
   return (int)cudaDeviceSynchronize();

@@ -5,6 +5,7 @@ the signal speeds an FP32 bound leaves open, bit for bit that of both speeds."""
 import ctypes
 import os
 import subprocess
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -22,6 +23,7 @@ def lib(tmp_path_factory):
                     os.path.join(HERE, "fp64_ops_check.cu")], check=True)
     lib = ctypes.CDLL(out)
     lib.run_ops.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_int]
+    lib.run_quotients.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_int]
     lib.run_lambdas.argtypes = [ctypes.c_void_p] * 3 + [ctypes.c_double] + [ctypes.c_void_p] * 2 + [ctypes.c_int]
     return lib
 
@@ -59,6 +61,40 @@ def test_edge_values(ops):
     _, root = ops(np.array([0.0, -0.0, 5e-324, -1.0, np.nan]))
     assert root[0] == 0.0 and root[1] == 0.0 and root[2] == 0.0
     assert np.isnan(root[3]) and np.isnan(root[4])
+
+
+def _quotient(lib, a, b):
+    x, y = torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda()
+    q = torch.empty_like(x)
+    torch.cuda.synchronize()
+    assert lib.run_quotients(x.data_ptr(), y.data_ptr(), q.data_ptr(), a.size) == 0
+    return q.cpu().numpy()
+
+
+def test_quotient_within_one_ulp(lib):
+    rng = np.random.default_rng(4)
+    n = 2000000
+    near1 = 1.0 + rng.integers(0, 2000, n // 4) * 2.0 ** -52
+    near2 = 2.0 - rng.integers(1, 2000, n // 4) * 2.0 ** -52
+    a = np.concatenate([rng.uniform(1, 2, n // 2), near1, near2]) * 2.0 ** rng.integers(-200, 200, n)
+    a *= np.where(rng.random(n) < 0.5, -1.0, 1.0)
+    b = rng.permutation(np.concatenate([rng.uniform(1, 2, n // 2), near1, near2])) * 2.0 ** rng.integers(-200, 200, n)
+    q = _quotient(lib, a, b)
+    assert np.all(np.abs(q - a / b) <= np.spacing(np.abs(a / b)))
+    # 0.51 units of the exact quotient (the values near 1 and 2 give many next to
+    # a rounding boundary, where the correctly rounded one is the neighbour)
+    for i in range(0, n, 101):
+        e = abs(Fraction(q[i]) - Fraction(a[i]) / Fraction(b[i])) / Fraction(np.spacing(abs(q[i])))
+        assert e <= Fraction(51, 100), (a[i], b[i], q[i], float(e))
+    assert np.array_equal(_quotient(lib, b, b), np.ones(n))
+
+
+def test_quotient_edge_values(lib):
+    a = np.array([0.0, -0.0, 5e-324, 1e-300, np.inf, -np.inf, np.nan, 1.0, 3.0])
+    b = np.array([2.0, 2.0, 1.0, 1e300, 2.0, 2.0, 2.0, np.inf, np.nan])
+    q = _quotient(lib, a, b)
+    assert np.all(q[:4] == 0.0) and np.signbit(q[1])
+    assert np.isnan(q[4:9]).all()
 
 
 def _faces(kind, n, rng):
