@@ -388,9 +388,11 @@ int crn_ensemble_create(crn_grid* const* grids, int32_t n, crn_ensemble** out);
 int crn_ensemble_destroy(crn_ensemble* e);
 
 /* Radial planes per work item for every member (their tile shapes are kept);
- * 0 (default) uses each member's own choice (the one its crn_residual uses).
- * crn_ensemble_kchunk returns the last value set for all members, or after
- * crn_ensemble_autotune the chunk of its largest size class. */
+ * 0 (default): each member's own choice (the one its crn_residual uses) while
+ * the members together are small, else chunks balanced over the ensemble
+ * (crn_ensemble_member_config reads them back).  crn_ensemble_kchunk returns
+ * the last value set for all members, or after crn_ensemble_autotune the chunk
+ * of its largest size class. */
 int crn_ensemble_set_kchunk(crn_ensemble* e, int32_t kchunk);
 int32_t crn_ensemble_kchunk(const crn_ensemble* e);
 
@@ -422,7 +424,7 @@ int crn_ensemble_autotune(crn_ensemble* e, const void* const* U_dev, void* const
 
 /* Tile shape (0: 8 x 32, 1: 16 x 16, 2: 8 x 16 (theta, phi) columns per CTA; 2
  * is the own shape of FP64 members and theirs only, 0 of FP32 members) and radial
- * chunk (planes per work item; 0 = the member's own single-launch chunk) of
+ * chunk (planes per work item; 0 = the default of crn_ensemble_set_kchunk) of
  * member m in the persistent launch.  CRN_E_ARG for an index, shape or chunk
  * out of range; a chunk that gives a member more work items than its
  * reduction scratch holds is rejected by the next residual call. */
