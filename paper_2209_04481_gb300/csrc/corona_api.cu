@@ -349,8 +349,7 @@ int crn_grid_create(const crn_grid_desc* d, crn_grid** out) {
     const int per_sm = d->precision == CRN_FP64 ? crn::tiled_ctas_per_sm_fp64(d->limiter)
                                                  : crn::tiled_ctas_per_sm_fp32(d->limiter);
     int kc = crn::choose_radial_chunk(d->n_r, ntiles, std::max(nsm, 1), per_sm, d->precision == CRN_FP64);
-    g->cfg.kchunk_pair =
-        crn::choose_radial_chunk(d->n_r, 2 * ntiles, std::max(nsm, 1), per_sm, d->precision == CRN_FP64);
+    g->cfg.tiled_per_sm = std::max(per_sm, 1);
     if (const char* env = std::getenv("CRN_KCHUNK")) {  // tuning override
       const int v = std::atoi(env);
       if (v >= 1) kc = g->cfg.kchunk_pair = v;
@@ -503,9 +502,9 @@ int crn_pseudo_time_step(crn_grid* g, double* U64_dev, int32_t nsteps, double cf
   }
   for (int s = 0; s < nsteps && e == cudaSuccess; ++s) {
     if (g->d.precision == CRN_FP64)
-      e = crn::launch_residual_fp64(g, U64_dev, (double*)g->rbuf, nullptr, nullptr, st, &nl);
+      e = crn::launch_residual_fp64(g, U64_dev, (double*)g->rbuf, nullptr, g->stats + 9, st, &nl);
     else
-      e = crn::launch_residual_fp32(g, g->shadow, (float*)g->rbuf, nullptr, nullptr, st, &nl);
+      e = crn::launch_residual_fp32(g, g->shadow, (float*)g->rbuf, nullptr, g->stats + 9, st, &nl);
     total += nl;
     if (e != cudaSuccess) break;
     e = crn::launch_update(g, U64_dev, cfl, res_log10_dev ? res_log10_dev + 9 * (size_t)s : nullptr,

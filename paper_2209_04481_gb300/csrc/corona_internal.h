@@ -29,7 +29,8 @@ struct GeoBuf {
 
 struct LaunchCfg {
   int kchunk_tiled = 16;  // radial planes per CTA of the tiled kernel
-  int kchunk_pair = 16;   // the same for two residuals in one launch
+  int kchunk_pair = 0;    // the same for two residuals in one launch (0: chosen by the first)
+  int tiled_per_sm = 2;   // resident CTAs per SM of the tiled kernel
   int num_sms = 152;      // streaming multiprocessors of the grid's device
   int update_per_sm = 2;  // resident blocks per SM of the pseudo-time update
   bool staged = false;    // FP32 residuals use the TMA-staged kernel (on request)
@@ -67,7 +68,9 @@ struct crn_grid {
 
 namespace crn {
 
-// launchers (return cudaGetLastError() of the launch)
+// launchers (return cudaGetLastError() of the launch).  A residual without
+// norms_user and dt_user writes R alone; dt_user = g->stats + 9 keeps the grid's
+// own dtmin.
 cudaError_t launch_residual_fp64(crn_grid* g, const double* U, double* R, double* norms_user,
                                  double* dt_user, cudaStream_t st, int* nlaunch);
 cudaError_t launch_residual_fp32(crn_grid* g, const float* U, float* R, double* norms_user,

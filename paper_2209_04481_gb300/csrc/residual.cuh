@@ -462,11 +462,13 @@ template <class T, int NT> struct MinCtas { static constexpr int value = (sizeof
 
 // One work item of the tiled residual: tile `tile` (row-major over the
 // (theta, phi) tiles) and radial chunk `chunk` of one grid; `bid` / `nblocks`
-// number the items of that grid for its cross-CTA reduction.
+// number the items of that grid for its cross-CTA reduction.  The grid's
+// description is read where it lies (kernel parameters, or the ensemble's copy
+// in shared memory) at each use.
 template <class T, int LIM, int TT, int TP>
 __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, const Phys<T>& ph,
-                                           const double* __restrict__ Br, const T* __restrict__ U,
-                                           T* __restrict__ R, const Reduce& red, int kchunk, int tile,
+                                           const double* const& Br, const T* const& U,
+                                           T* const& R, const Reduce& red, int kchunk, int tile,
                                            int chunk, int bid, int nblocks, unsigned char* smem_raw) {
   using D = TileDims<TT, TP>;
   constexpr int NT = D::NT, HP = D::HP, HC = D::HC, NTV = D::NTV, NFA = D::NFA, NF = D::NF;
@@ -871,9 +873,11 @@ residual_tiled(Shape sh, Geo<T> g, Phys<T> ph, const double* __restrict__ Br,
                const T* __restrict__ U, T* __restrict__ R, Reduce red, int kchunk, const T* __restrict__ U2,
                T* __restrict__ R2) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  tiled_item<T, LIM, TT, TP>(sh, g, ph, Br, blockIdx.z == 0 ? U : U2, blockIdx.z == 0 ? R : R2, red, kchunk,
-                             blockIdx.x, blockIdx.y, blockIdx.y * gridDim.x + blockIdx.x,
-                             gridDim.x * gridDim.y, smem_raw);
+  const double* br = Br;
+  const T* u = blockIdx.z == 0 ? U : U2;
+  T* r = blockIdx.z == 0 ? R : R2;
+  tiled_item<T, LIM, TT, TP>(sh, g, ph, br, u, r, red, kchunk, blockIdx.x, blockIdx.y,
+                             blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y, smem_raw);
 }
 
 // ---------------------------------------------------------------------------

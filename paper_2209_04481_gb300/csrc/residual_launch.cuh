@@ -20,6 +20,7 @@ template <class T> const Phys<T>& phys_of(const crn_grid* g);
 template <> inline const Phys<double>& phys_of<double>(const crn_grid* g) { return g->ph64; }
 template <> inline const Phys<float>& phys_of<float>(const crn_grid* g) { return g->ph32; }
 
+// dt_user = g->stats + 9 asks for the grid's own dtmin (pseudo-time stepping)
 inline Reduce make_reduce(crn_grid* g, double* norms_user, double* dt_user) {
   Reduce r;
   r.partials = g->partials;
@@ -39,7 +40,7 @@ cudaError_t launch_lim(crn_grid* g, const T* U, T* R, double* nu, double* du, cu
   const Shape sh = g->shape;
   const Geo<T>& geo = geo_of<T>(g);
   const Phys<T>& ph = phys_of<T>(g);
-  const Reduce red = make_reduce(g, nu, du);
+  Reduce red = make_reduce(g, nu, du);
   if (g->d.kernel == CRN_KERNEL_CELLWISE) {
     const unsigned nb = (unsigned)((sh.ncell + 255) / 256);
     residual_cellwise<T, LIM><<<nb, 256, 0, st>>>(sh, geo, ph, g->br, U, R, red);
@@ -51,6 +52,9 @@ cudaError_t launch_lim(crn_grid* g, const T* U, T* R, double* nu, double* du, cu
   const int ntiles = ((sh.nt + TT - 1) / TT) * ((sh.np + TP - 1) / TP);
   const int kc = g->cfg.kchunk_tiled;
   const int nch = (sh.nr + kc - 1) / kc;
+  // nobody reads the norms or the step bound: no sums, no last-CTA tail (FP32: 32 x
+  // 16 x 32 16.6 -> 12.6 us, 95 x 45 x 88 39 -> 33 us, 128 x 64 x 128 77 -> 71 us)
+  if (!nu && !du) red.counter = nullptr;
   dim3 grid((unsigned)ntiles, (unsigned)nch);
   residual_tiled<T, LIM, TT, TP><<<grid, D::NT, smem, st>>>(sh, geo, ph, g->br, U, R, red, kc, nullptr, nullptr);
   return cudaGetLastError();
@@ -66,6 +70,8 @@ cudaError_t launch_pair_lim(crn_grid* g, const T* U, T* R, const T* U2, T* R2, c
   constexpr int TT = TileFor<T>::TT, TP = TileFor<T>::TP;
   using D = TileDims<TT, TP>;
   const int ntiles = ((sh.nt + TT - 1) / TT) * ((sh.np + TP - 1) / TP);
+  if (g->cfg.kchunk_pair <= 0)
+    g->cfg.kchunk_pair = choose_radial_chunk(sh.nr, 2ll * ntiles, g->cfg.num_sms, g->cfg.tiled_per_sm, sizeof(T) == 8);
   const int kc = g->cfg.kchunk_pair;
   const dim3 grid((unsigned)ntiles, (unsigned)((sh.nr + kc - 1) / kc), 2);
   residual_tiled<T, LIM, TT, TP><<<grid, D::NT, D::template smem_bytes<T>(), st>>>(
@@ -150,6 +156,7 @@ void ens_fill_t(crn_grid* g, const T* U, T* R, int kchunk, int item0, double* no
   m->U = U;
   m->R = R;
   m->red = make_reduce(g, norms_user, dt_user);
+  if (!norms_user && !dt_user) m->red.counter = nullptr;
   m->kchunk = kchunk;
   m->ntiles = ((g->shape.nt + TT - 1) / TT) * ((g->shape.np + TP - 1) / TP);
   m->nitems = m->ntiles * ((g->shape.nr + kchunk - 1) / kchunk);

@@ -314,6 +314,7 @@ int run(const crn_grid_desc& d, DeviceSlot& slot, const double* Br, const void* 
   red.norms_user = norms;
   red.dt_user = dtmin;
   red.log_out = nullptr;
+  if (!norms && !dtmin) red.counter = nullptr;  // R alone
   // the arrival counter and the error word must start cleared
   cudaError_t e = cudaMemsetAsync(base + kMiscOff, 0, 8, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(base + kMiscOff + 8, 0xff, 8, st);
