@@ -219,14 +219,15 @@ int update_records(crn_ensemble* e, double* const* U64, double* log, cudaStream_
 
 // one persistent launch per tile shape in use; adds the launches to *count
 cudaError_t launch(crn_ensemble* e, cudaStream_t st, int* count = nullptr) {
+  const bool sums = e->kN || e->kD || e->kMarch;  // somebody reads the norms or dtmin
   for (int t = 0; t < crn::kEnsTileCount; ++t) {
     if (e->grp_cnt[t] == 0) continue;
     const void* rec = static_cast<const unsigned char*>(e->d_rec) + (size_t)e->grp_off[t] * e->msz;
     const cudaError_t err =
         e->precision == CRN_FP64
-            ? crn::launch_ensemble_fp64(rec, e->grp_cnt[t], e->grp_items[t], e->next + t, e->limiter, t,
+            ? crn::launch_ensemble_fp64(rec, e->grp_cnt[t], e->grp_items[t], e->next + t, e->limiter, sums, t,
                                         e->nctas[t], st)
-            : crn::launch_ensemble_fp32(rec, e->grp_cnt[t], e->grp_items[t], e->next + t, e->limiter, t,
+            : crn::launch_ensemble_fp32(rec, e->grp_cnt[t], e->grp_items[t], e->next + t, e->limiter, sums, t,
                                         e->nctas[t], st);
     if (err != cudaSuccess) return err;
     if (count) ++*count;

@@ -24,7 +24,7 @@ namespace crn {
 // where the reductions and error reports go
 struct Reduce {
   double* partials;          // [gridDim.x * gridDim.y][16]
-  unsigned int* counter;     // CTA arrival counter, reset by the last CTA; null: no reductions (tiled kernel)
+  unsigned int* counter;     // CTA arrival counter, reset by the last CTA
   double* norms_out;         // [9] L2 norms (always written)
   double* dt_out;            // [1] min V / sum lambda |S| (always written)
   double* norms_user;        // optional copy for the caller
@@ -420,13 +420,36 @@ struct TileDims {
   static constexpr int NF = NV + 1;                             // 9 fluxes + lambda |S|
   static constexpr int NEXTRA_V = 2 * (TT + TP);                // halo cells needing a face value
   static constexpr int NEXTRA_F = TT + TP;                      // faces beyond the own lower faces
+  static constexpr int NUV = NFA + NEXTRA_F;                    // L states, then the R states of those faces
+  static constexpr int NITEM = (3 * NEXTRA_V + 1) & ~1;         // items of three variables of one halo cell
+  // item x -> what it does, packed: source offset in the halo'd planes, target
+  // offset in the face states, theta neighbours (else phi), upper value (else lower)
+  __device__ static unsigned item(int x) {
+    const int e = x % NEXTRA_V, v0 = 3 * (x / NEXTRA_V);
+    int h, dst;
+    unsigned flags;
+    if (e < TP) {                  // theta row -1: upper value -> face row 0
+      h = HP + e + 2; dst = e; flags = 3u;
+    } else if (e < TP + TT) {      // phi col -1 of row r: upper value -> face col 0
+      const int r = e - TP;
+      h = (r + 2) * HP + 1; dst = NTV + r * (TP + 1); flags = 2u;
+    } else if (e < 2 * TP + TT) {  // theta row TT: lower value, R state of face row TT
+      const int c = e - TP - TT;
+      h = (TT + 2) * HP + c + 2; dst = NFA + c; flags = 1u;
+    } else {                       // phi col TP of row r: lower value, R state of face col TP
+      const int r = e - 2 * TP - TT;
+      h = (r + 2) * HP + TP + 2; dst = NFA + TP + r; flags = 0u;
+    }
+    return (unsigned)(h + v0 * HC) | ((unsigned)(dst + v0 * NUV) << 15) | (flags << 30);
+  }
   // per-CTA geometry staged once: theta-face normals, phi-face normals, own
   // r-face normals, own radial unit vectors, theta factors of the areas/volumes
   static constexpr int NGEO = 3 * NTV + 2 * (TP + 1) + 6 * NT + (TT + 1) + 2 * TT;
   static constexpr int NRAD = 8;                                // radial factors of a plane, three planes held
   template <class T>
   static constexpr size_t smem_bytes() {
-    return sizeof(T) * ((size_t)NV * HC + (size_t)NV * NFA + (size_t)NF * NFA + (size_t)NV * NEXTRA_F +
+    return sizeof(unsigned) * (size_t)NITEM +
+           sizeof(T) * ((size_t)NV * HC + (size_t)NV * NUV + (size_t)NF * NFA +
                         (size_t)NV * NHALO + (size_t)3 * NRAD + (size_t)NGEO);
   }
   // halo position h in [0, NHALO) -> halo'd (row, col)
@@ -464,23 +487,24 @@ template <class T, int NT> struct MinCtas { static constexpr int value = (sizeof
 // (theta, phi) tiles) and radial chunk `chunk` of one grid; `bid` / `nblocks`
 // number the items of that grid for its cross-CTA reduction.  The grid's
 // description is read where it lies (kernel parameters, or the ensemble's copy
-// in shared memory) at each use.
-template <class T, int LIM, int TT, int TP>
+// in shared memory) at each use.  SUMS: with the norms and the step bound (their
+// ten running sums per thread are registers the FP32 kernel has to spill for).
+template <class T, int LIM, int TT, int TP, bool SUMS>
 __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, const Phys<T>& ph,
                                            const double* const& Br, const T* const& U,
                                            T* const& R, const Reduce& red, int kchunk, int tile,
                                            int chunk, int bid, int nblocks, unsigned char* smem_raw) {
   using D = TileDims<TT, TP>;
-  constexpr int NT = D::NT, HP = D::HP, HC = D::HC, NTV = D::NTV, NFA = D::NFA, NF = D::NF;
+  constexpr int NT = D::NT, HP = D::HP, HC = D::HC, NTV = D::NTV, NFA = D::NFA, NUV = D::NUV, NF = D::NF;
   constexpr int NX = D::NEXTRA_V, NXF = D::NEXTRA_F;
   static_assert(D::NRAD <= D::NHALO, "the halo threads wait for the radial factors too");
   static_assert(D::NHALO <= NT, "each thread stores at most one halo position");
-  static_assert(NXF <= NT && NT % 32 == 0, "tile shape");
+  static_assert(NXF <= NT && NT % 32 == 0 && NV * HC < (1 << 15) && NV * D::NUV < (1 << 15), "tile shape");
   T* sp = reinterpret_cast<T*>(smem_raw);    // [NV][HC]   primitives of plane k
-  T* uv = sp + NV * HC;                      // [NV][NFA]  L state of each face (upper value of the cell below)
-  T* fx = uv + NV * NFA;                     // [NF][NFA]  flux x area of each face, lambda x area last
-  T* xr = fx + NF * NFA;                     // [NV][NXF]  R states of the faces past the last row / column
-  T* hr = xr + NV * NXF;                     // [NV][NHALO] raw halo cells of plane k + 1
+  T* uv = sp + NV * HC;                      // [NV][NUV]  L state of each face (upper value of the cell below),
+                                             //   then the R states of the faces past the last row / column
+  T* fx = uv + NV * NUV;                     // [NF][NFA]  flux x area of each face, lambda x area last
+  T* hr = fx + NF * NFA;                     // [NV][NHALO] raw halo cells of plane k + 1
   T* s_rad = hr + NV * D::NHALO;             // [3][NRAD] radial factors of planes k .. k + 2
   T* s_nth = s_rad + 3 * D::NRAD;            // [3][NTV]
   T* s_nph = s_nth + 3 * NTV;                // [2][TP + 1]
@@ -489,6 +513,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
   T* s_at = s_rh + 3 * NT;                   // [TT + 1]
   T* s_ar = s_at + (TT + 1);                 // [TT]
   T* s_av = s_ar + TT;                       // [TT]
+  unsigned* s_item = reinterpret_cast<unsigned*>(s_av + TT);  // [NITEM]
 
   const int nr = sh.nr, nt = sh.nt, np = sh.np;
   const int64_t N = sh.ncell, cs = (int64_t)nt * np;
@@ -579,6 +604,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
         rad_slot(k0)[tid] = *rad_at(k0);
         if (k0 + 1 < k1) rad_slot(k0 + 1)[tid] = *rad_at(k0 + 1);
       }
+      for (int x = tid; x < 3 * NX; x += NT) s_item[x] = D::item(x);
       if (tid <= TT) s_at[tid] = g.at[min(j0 + tid, nt)];
       if (tid < TT) {
         s_ar[tid] = g.ar[min(j0 + tid, nt - 1)];
@@ -665,14 +691,16 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
         r[v] = dr[v] + (fx[v * NFA + tl] - fx[v * NFA + tu]) + (fx[v * NFA + pl] - fx[v * NFA + pu]);
       const T lam = dr[NV] + (fx[NV * NFA + tl] + fx[NV * NFA + tu]) + (fx[NV * NFA + pl] + fx[NV * NFA + pu]);
       const T ivol = frcp(rad_slot(kg)[1] * s_av[jj]);
-      const T x = lam * ivol;
-      rate = greater(x, rate) ? x : rate;
+      if (SUMS) {
+        const T x = lam * ivol;
+        rate = greater(x, rate) ? x : rate;
+      }
       T* dst = R + (int64_t)kg * cs + ocol;
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         r[v] *= ivol;
         dst[v * N] = r[v];
-        sq[v] = fmat(r[v], r[v], sq[v]);
+        if (SUMS) sq[v] = fmat(r[v], r[v], sq[v]);
       }
       if (bad || !squares_finite(r)) flag_bad(red, (int64_t)kg * cs + ocol);
     }
@@ -686,36 +714,23 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       const T sf = limited_slope<LIM>(w - q[-1], q[1] - w, ph.eps);
       // explicit FMAs: the same rounding in every kernel inlining this
       tlo[v] = fmat(-half, st, w);
-      uv[v * NFA + tid + TP] = fmat(half, st, w);
+      uv[v * NUV + tid + TP] = fmat(half, st, w);
       plo[v] = fmat(-half, sf, w);
-      uv[v * NFA + NTV + jj * (TP + 1) + ii + 1] = fmat(half, sf, w);
+      uv[v * NUV + NTV + jj * (TP + 1) + ii + 1] = fmat(half, sf, w);
     }
     // halo cells whose face values the tile's boundary faces need: three
     // variables of one cell per item
     for (int x = tid; x < 3 * NX; x += NT) {
-      const int e = x % NX, v0 = 3 * (x / NX);
-      int h, step, dst, stride;
-      T sgn;
-      T* base;
-      if (e < TP) {                  // theta row -1: upper value -> face row 0
-        h = HP + e + 2; step = HP; base = uv; dst = e; stride = NFA; sgn = half;
-      } else if (e < TP + TT) {      // phi col -1 of row r: upper value -> face col 0
-        const int r = e - TP;
-        h = (r + 2) * HP + 1; step = 1; base = uv; dst = NTV + r * (TP + 1); stride = NFA; sgn = half;
-      } else if (e < 2 * TP + TT) {  // theta row TT: lower value, R state of face row TT
-        const int c = e - TP - TT;
-        h = (TT + 2) * HP + c + 2; step = HP; base = xr; dst = c; stride = NXF; sgn = -half;
-      } else {                       // phi col TP of row r: lower value, R state of face col TP
-        const int r = e - 2 * TP - TT;
-        h = (r + 2) * HP + TP + 2; step = 1; base = xr; dst = TP + r; stride = NXF; sgn = -half;
-      }
-      const T* q = sp + v0 * HC + h;
-      T* o = base + v0 * stride + dst;
+      const unsigned it = s_item[x];
+      const int step = (it & (1u << 30)) ? HP : 1;
+      const T sgn = (it & (1u << 31)) ? half : -half;
+      const T* q = sp + (it & 0x7fffu);
+      T* o = uv + ((it >> 15) & 0x7fffu);
 #pragma unroll
       for (int v = 0; v < 3; ++v) {
         const T w = q[v * HC];
         const T s = limited_slope<LIM>(w - q[v * HC - step], q[v * HC + step] - w, ph.eps);
-        o[v * stride] = fmat(sgn, s, w);
+        o[v * NUV] = fmat(sgn, s, w);
       }
     }
     __syncthreads();
@@ -727,7 +742,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       if (jo > 0 && jo < nt && io < np) {
         T wl[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) wl[v] = uv[v * NFA + tid];
+        for (int v = 0; v < NV; ++v) wl[v] = uv[v * NUV + tid];
         rusanov<true>(wl, tlo, s_nth[tid], s_nth[NTV + tid], s_nth[2 * NTV + tid], rbk * s_at[jj], ph, fl, la);
       } else {
 #pragma unroll
@@ -743,7 +758,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       if (jo < nt && io <= np) {
         T wl[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) wl[v] = uv[v * NFA + f];
+        for (int v = 0; v < NV; ++v) wl[v] = uv[v * NUV + f];
         rusanov<false>(wl, plo, s_nph[ii], s_nph[TP + 1 + ii], (T)0, rbk * g.dtheta, ph, fl, la);
       } else {
 #pragma unroll
@@ -775,7 +790,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
         if (live) {
           T wl[NV], wr[NV];
 #pragma unroll
-          for (int v = 0; v < NV; ++v) { wl[v] = uv[v * NFA + f]; wr[v] = xr[v * NXF + e]; }
+          for (int v = 0; v < NV; ++v) { wl[v] = uv[v * NUV + f]; wr[v] = uv[v * NUV + NFA + e]; }
           rusanov<true>(wl, wr, nx, ny, nz, area, ph, fl, la);
         } else {
 #pragma unroll
@@ -852,7 +867,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
     __syncthreads();
   }
   // ---------------- reductions: warp tree in T, then FP64 across warps and CTAs
-  if (red.counter == nullptr) return;  // the caller wants R alone
+  if (!SUMS) return;
   T dtm = (T)INFINITY;
   if (rate > (T)0) dtm = sizeof(T) == 4 ? (T)__frcp_rn((float)rate) : one / rate;
 #pragma unroll
@@ -867,7 +882,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
 
 // one grid: block (x, y) = (tile, radial chunk); with a second state, block z
 // picks the state
-template <class T, int LIM, int TT, int TP>
+template <class T, int LIM, int TT, int TP, bool SUMS>
 __global__ void __launch_bounds__(TT * TP, (MinCtas<T, TT * TP>::value))
 residual_tiled(Shape sh, Geo<T> g, Phys<T> ph, const double* __restrict__ Br,
                const T* __restrict__ U, T* __restrict__ R, Reduce red, int kchunk, const T* __restrict__ U2,
@@ -876,7 +891,7 @@ residual_tiled(Shape sh, Geo<T> g, Phys<T> ph, const double* __restrict__ Br,
   const double* br = Br;
   const T* u = blockIdx.z == 0 ? U : U2;
   T* r = blockIdx.z == 0 ? R : R2;
-  tiled_item<T, LIM, TT, TP>(sh, g, ph, br, u, r, red, kchunk, blockIdx.x, blockIdx.y,
+  tiled_item<T, LIM, TT, TP, SUMS>(sh, g, ph, br, u, r, red, kchunk, blockIdx.x, blockIdx.y,
                              blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y, smem_raw);
 }
 
@@ -903,7 +918,7 @@ struct EnsMember {
 };
 
 
-template <class T, int LIM, int TT, int TP>
+template <class T, int LIM, int TT, int TP, bool SUMS>
 __global__ void __launch_bounds__(TT * TP, (MinCtas<T, TT * TP>::value))
 residual_ensemble(const EnsMember<T>* __restrict__ mem, int nmem, int nitems, unsigned int* __restrict__ next) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -926,7 +941,7 @@ residual_ensemble(const EnsMember<T>* __restrict__ mem, int nmem, int nitems, un
       if (threadIdx.x == 0) s_mem = m;
     }
     const int local = item - M.item0;
-    tiled_item<T, LIM, TT, TP>(M.sh, M.g, M.ph, M.Br, M.U, M.R, M.red, M.kchunk, local % M.ntiles,
+    tiled_item<T, LIM, TT, TP, SUMS>(M.sh, M.g, M.ph, M.Br, M.U, M.R, M.red, M.kchunk, local % M.ntiles,
                                local / M.ntiles, local, M.nitems, smem_raw);
     __syncthreads();  // shared memory and s_item are reused by the next item
   }

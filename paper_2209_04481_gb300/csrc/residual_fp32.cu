@@ -146,8 +146,8 @@ int ens_fill_fp32(crn_grid* g, const void* U, void* R, int kchunk, int item0, do
   return m->nitems;
 }
 cudaError_t launch_ensemble_fp32(const void* dev, int nmem, int nitems, unsigned int* next, int limiter,
-                                  int tile, int nctas, cudaStream_t st) {
-  return launch_ensemble_t<float>(static_cast<const EnsMember<float>*>(dev), nmem, nitems, next, limiter, tile, nctas,
+                                  bool sums, int tile, int nctas, cudaStream_t st) {
+  return launch_ensemble_t<float>(static_cast<const EnsMember<float>*>(dev), nmem, nitems, next, limiter, sums, tile, nctas,
                                 st);
 }
 int ensemble_ctas_per_sm_fp32(int limiter, int tile) { return ensemble_ctas_t<float>(limiter, tile); }

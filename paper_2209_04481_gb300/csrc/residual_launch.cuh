@@ -40,7 +40,7 @@ cudaError_t launch_lim(crn_grid* g, const T* U, T* R, double* nu, double* du, cu
   const Shape sh = g->shape;
   const Geo<T>& geo = geo_of<T>(g);
   const Phys<T>& ph = phys_of<T>(g);
-  Reduce red = make_reduce(g, nu, du);
+  const Reduce red = make_reduce(g, nu, du);
   if (g->d.kernel == CRN_KERNEL_CELLWISE) {
     const unsigned nb = (unsigned)((sh.ncell + 255) / 256);
     residual_cellwise<T, LIM><<<nb, 256, 0, st>>>(sh, geo, ph, g->br, U, R, red);
@@ -54,9 +54,11 @@ cudaError_t launch_lim(crn_grid* g, const T* U, T* R, double* nu, double* du, cu
   const int nch = (sh.nr + kc - 1) / kc;
   // nobody reads the norms or the step bound: no sums, no last-CTA tail (FP32: 32 x
   // 16 x 32 16.6 -> 12.6 us, 95 x 45 x 88 39 -> 33 us, 128 x 64 x 128 77 -> 71 us)
-  if (!nu && !du) red.counter = nullptr;
   dim3 grid((unsigned)ntiles, (unsigned)nch);
-  residual_tiled<T, LIM, TT, TP><<<grid, D::NT, smem, st>>>(sh, geo, ph, g->br, U, R, red, kc, nullptr, nullptr);
+  if (nu || du)
+    residual_tiled<T, LIM, TT, TP, true><<<grid, D::NT, smem, st>>>(sh, geo, ph, g->br, U, R, red, kc, nullptr, nullptr);
+  else
+    residual_tiled<T, LIM, TT, TP, false><<<grid, D::NT, smem, st>>>(sh, geo, ph, g->br, U, R, red, kc, nullptr, nullptr);
   return cudaGetLastError();
 }
 
@@ -65,8 +67,7 @@ cudaError_t launch_lim(crn_grid* g, const T* U, T* R, double* nu, double* du, cu
 template <class T, int LIM>
 cudaError_t launch_pair_lim(crn_grid* g, const T* U, T* R, const T* U2, T* R2, cudaStream_t st) {
   const Shape sh = g->shape;
-  Reduce red = make_reduce(g, nullptr, nullptr);
-  red.counter = nullptr;  // no norms, no dtmin
+  const Reduce red = make_reduce(g, nullptr, nullptr);
   constexpr int TT = TileFor<T>::TT, TP = TileFor<T>::TP;
   using D = TileDims<TT, TP>;
   const int ntiles = ((sh.nt + TT - 1) / TT) * ((sh.np + TP - 1) / TP);
@@ -74,7 +75,7 @@ cudaError_t launch_pair_lim(crn_grid* g, const T* U, T* R, const T* U2, T* R2, c
     g->cfg.kchunk_pair = choose_radial_chunk(sh.nr, 2ll * ntiles, g->cfg.num_sms, g->cfg.tiled_per_sm, sizeof(T) == 8);
   const int kc = g->cfg.kchunk_pair;
   const dim3 grid((unsigned)ntiles, (unsigned)((sh.nr + kc - 1) / kc), 2);
-  residual_tiled<T, LIM, TT, TP><<<grid, D::NT, D::template smem_bytes<T>(), st>>>(
+  residual_tiled<T, LIM, TT, TP, false><<<grid, D::NT, D::template smem_bytes<T>(), st>>>(
       sh, geo_of<T>(g), phys_of<T>(g), g->br, U, R, red, kc, U2, R2);
   return cudaGetLastError();
 }
@@ -106,12 +107,16 @@ template <class T>
 cudaError_t prepare_t() {
   constexpr int TT = TileFor<T>::TT, TP = TileFor<T>::TP;
   const int smem = (int)TileDims<TT, TP>::template smem_bytes<T>();
-  cudaError_t e;
-  e = cudaFuncSetAttribute(residual_tiled<T, 0, TT, TP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(residual_tiled<T, 1, TT, TP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(residual_tiled<T, 2, TT, TP>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  auto set = [&](auto kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  };
+  cudaError_t e = set(residual_tiled<T, 0, TT, TP, true>);
+  if (e == cudaSuccess) e = set(residual_tiled<T, 1, TT, TP, true>);
+  if (e == cudaSuccess) e = set(residual_tiled<T, 2, TT, TP, true>);
+  if (e == cudaSuccess) e = set(residual_tiled<T, 0, TT, TP, false>);
+  if (e == cudaSuccess) e = set(residual_tiled<T, 1, TT, TP, false>);
+  if (e == cudaSuccess) e = set(residual_tiled<T, 2, TT, TP, false>);
+  return e;
 }
 
 template <class T>
@@ -121,11 +126,11 @@ int tiled_ctas_t(int limiter) {
   int n = 0;
   cudaError_t e;
   if (limiter == CRN_LIM_NONE)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 0, TT, TP>, TT * TP, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 0, TT, TP, true>, TT * TP, smem);
   else if (limiter == CRN_LIM_MINMOD)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 1, TT, TP>, TT * TP, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 1, TT, TP, true>, TT * TP, smem);
   else
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 2, TT, TP>, TT * TP, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 2, TT, TP, true>, TT * TP, smem);
   return e == cudaSuccess ? n : 0;
 }
 
@@ -156,7 +161,6 @@ void ens_fill_t(crn_grid* g, const T* U, T* R, int kchunk, int item0, double* no
   m->U = U;
   m->R = R;
   m->red = make_reduce(g, norms_user, dt_user);
-  if (!norms_user && !dt_user) m->red.counter = nullptr;
   m->kchunk = kchunk;
   m->ntiles = ((g->shape.nt + TT - 1) / TT) * ((g->shape.np + TP - 1) / TP);
   m->nitems = m->ntiles * ((g->shape.nr + kchunk - 1) / kchunk);
@@ -166,28 +170,29 @@ void ens_fill_t(crn_grid* g, const T* U, T* R, int kchunk, int item0, double* no
 
 template <class T, int TT, int TP>
 cudaError_t launch_ensemble_shape(const EnsMember<T>* dev, int nmem, int nitems, unsigned int* next, int limiter,
-                                  int nctas, cudaStream_t st) {
+                                  bool sums, int nctas, cudaStream_t st) {
   const size_t smem = TileDims<TT, TP>::template smem_bytes<T>();
   cudaError_t e = cudaMemsetAsync(next, 0, sizeof(unsigned int), st);
   if (e != cudaSuccess) return e;
+  auto go = [&](auto kern) { kern<<<nctas, TT * TP, smem, st>>>(dev, nmem, nitems, next); };
   if (limiter == CRN_LIM_NONE)
-    residual_ensemble<T, 0, TT, TP><<<nctas, TT * TP, smem, st>>>(dev, nmem, nitems, next);
+    sums ? go(residual_ensemble<T, 0, TT, TP, true>) : go(residual_ensemble<T, 0, TT, TP, false>);
   else if (limiter == CRN_LIM_MINMOD)
-    residual_ensemble<T, 1, TT, TP><<<nctas, TT * TP, smem, st>>>(dev, nmem, nitems, next);
+    sums ? go(residual_ensemble<T, 1, TT, TP, true>) : go(residual_ensemble<T, 1, TT, TP, false>);
   else
-    residual_ensemble<T, 2, TT, TP><<<nctas, TT * TP, smem, st>>>(dev, nmem, nitems, next);
+    sums ? go(residual_ensemble<T, 2, TT, TP, true>) : go(residual_ensemble<T, 2, TT, TP, false>);
   return cudaGetLastError();
 }
 
 // the persistent launch over the members of one tile shape
 template <class T>
 cudaError_t launch_ensemble_t(const EnsMember<T>* dev, int nmem, int nitems, unsigned int* next, int limiter,
-                              int tile, int nctas, cudaStream_t st) {
+                              bool sums, int tile, int nctas, cudaStream_t st) {
   if constexpr (sizeof(T) == 8) {
-    if (tile == 2) return launch_ensemble_shape<T, ens_tt(2), ens_tp(2)>(dev, nmem, nitems, next, limiter, nctas, st);
+    if (tile == 2) return launch_ensemble_shape<T, ens_tt(2), ens_tp(2)>(dev, nmem, nitems, next, limiter, sums, nctas, st);
   }
-  if (tile == 0) return launch_ensemble_shape<T, ens_tt(0), ens_tp(0)>(dev, nmem, nitems, next, limiter, nctas, st);
-  return launch_ensemble_shape<T, ens_tt(1), ens_tp(1)>(dev, nmem, nitems, next, limiter, nctas, st);
+  if (tile == 0) return launch_ensemble_shape<T, ens_tt(0), ens_tp(0)>(dev, nmem, nitems, next, limiter, sums, nctas, st);
+  return launch_ensemble_shape<T, ens_tt(1), ens_tp(1)>(dev, nmem, nitems, next, limiter, sums, nctas, st);
 }
 
 template <class T, int TT, int TP>
@@ -199,9 +204,12 @@ int ensemble_ctas_shape(int limiter) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, TT * TP, smem) != cudaSuccess) return 0;
     return n;
   };
-  if (limiter == CRN_LIM_NONE) return setup(residual_ensemble<T, 0, TT, TP>);
-  if (limiter == CRN_LIM_MINMOD) return setup(residual_ensemble<T, 1, TT, TP>);
-  return setup(residual_ensemble<T, 2, TT, TP>);
+  // both kernels of a limiter; the persistent grid fits either
+  if (limiter == CRN_LIM_NONE)
+    return std::min(setup(residual_ensemble<T, 0, TT, TP, true>), setup(residual_ensemble<T, 0, TT, TP, false>));
+  if (limiter == CRN_LIM_MINMOD)
+    return std::min(setup(residual_ensemble<T, 1, TT, TP, true>), setup(residual_ensemble<T, 1, TT, TP, false>));
+  return std::min(setup(residual_ensemble<T, 2, TT, TP, true>), setup(residual_ensemble<T, 2, TT, TP, false>));
 }
 
 // shared-memory opt-in and resident CTAs per SM of one tile shape's kernel

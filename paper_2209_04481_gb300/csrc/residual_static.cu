@@ -249,14 +249,15 @@ template <class T>
 cudaError_t opt_in_smem() {
   constexpr int TT = StaticTile<T>::TT, TP = StaticTile<T>::TP;
   const int smem = (int)crn::TileDims<TT, TP>::template smem_bytes<T>();
-  cudaError_t e = cudaFuncSetAttribute(crn::residual_tiled<T, 0, TT, TP>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(crn::residual_tiled<T, 1, TT, TP>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(crn::residual_tiled<T, 2, TT, TP>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  auto set = [&](auto kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  };
+  cudaError_t e = set(crn::residual_tiled<T, 0, TT, TP, true>);
+  if (e == cudaSuccess) e = set(crn::residual_tiled<T, 1, TT, TP, true>);
+  if (e == cudaSuccess) e = set(crn::residual_tiled<T, 2, TT, TP, true>);
+  if (e == cudaSuccess) e = set(crn::residual_tiled<T, 0, TT, TP, false>);
+  if (e == cudaSuccess) e = set(crn::residual_tiled<T, 1, TT, TP, false>);
+  if (e == cudaSuccess) e = set(crn::residual_tiled<T, 2, TT, TP, false>);
   return e;
 }
 
@@ -279,11 +280,11 @@ int plan(const crn_grid_desc& d, DeviceSlot& slot) {
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const size_t smem = crn::TileDims<TT, TP>::template smem_bytes<T>();
   if (d.limiter == CRN_LIM_NONE)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 0, TT, TP>, TT * TP, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 0, TT, TP, true>, TT * TP, smem);
   else if (d.limiter == CRN_LIM_MINMOD)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 1, TT, TP>, TT * TP, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 1, TT, TP, true>, TT * TP, smem);
   else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 2, TT, TP>, TT * TP, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 2, TT, TP, true>, TT * TP, smem);
   int kc = crn::choose_radial_chunk(d.n_r, ntiles, std::max(nsm, 1), per_sm, sizeof(T) == 8);
   while (ntiles * ((d.n_r + kc - 1) / kc) > kMaxBlocks) kc *= 2;
   slot.plan_desc = d;
@@ -314,7 +315,6 @@ int run(const crn_grid_desc& d, DeviceSlot& slot, const double* Br, const void* 
   red.norms_user = norms;
   red.dt_user = dtmin;
   red.log_out = nullptr;
-  if (!norms && !dtmin) red.counter = nullptr;  // R alone
   // the arrival counter and the error word must start cleared
   cudaError_t e = cudaMemsetAsync(base + kMiscOff, 0, 8, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(base + kMiscOff + 8, 0xff, 8, st);
@@ -325,18 +325,17 @@ int run(const crn_grid_desc& d, DeviceSlot& slot, const double* Br, const void* 
   dim3 grid((unsigned)ntiles, (unsigned)nch);
   const T* u = static_cast<const T*>(U);
   T* r = static_cast<T*>(R);
+  auto go = [&](auto kern) { kern<<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc, nullptr, nullptr); };
+  const bool sums = norms || dtmin;
   switch (d.limiter) {
     case CRN_LIM_NONE:
-      crn::residual_tiled<T, 0, TT, TP><<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc, nullptr,
-                                                                          nullptr);
+      sums ? go(crn::residual_tiled<T, 0, TT, TP, true>) : go(crn::residual_tiled<T, 0, TT, TP, false>);
       break;
     case CRN_LIM_MINMOD:
-      crn::residual_tiled<T, 1, TT, TP><<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc, nullptr,
-                                                                          nullptr);
+      sums ? go(crn::residual_tiled<T, 1, TT, TP, true>) : go(crn::residual_tiled<T, 1, TT, TP, false>);
       break;
     default:
-      crn::residual_tiled<T, 2, TT, TP><<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc, nullptr,
-                                                                          nullptr);
+      sums ? go(crn::residual_tiled<T, 2, TT, TP, true>) : go(crn::residual_tiled<T, 2, TT, TP, false>);
   }
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(CRN_E_CUDA, std::string("residual launch: ") + cudaGetErrorString(e));
