@@ -15,6 +15,9 @@
 namespace crn {
 
 struct Reduce;
+// what a launch of the tiled residual works out besides R: nothing, the step
+// bound, or the norms and the step bound
+enum Sums { SUMS_NONE = 0, SUMS_DT = 1, SUMS_ALL = 2 };
 struct NkWork;                // Newton-Krylov workspace (nk.cu)
 void nk_free(NkWork* w);
 struct HostPipe;              // host-buffer staging (host_io.cu)
@@ -99,12 +102,11 @@ int ens_fill_fp32(crn_grid* g, const void* U, void* R, int kchunk, int item0, do
                   void* dst);
 // work items of a member for a tile shape and radial chunk
 int ens_member_items(const crn_grid* g, int tile, int kchunk);
-// the persistent launch over `nmem` member records of one tile shape; sums: with
-// the members' norms and dtmin
+// the persistent launch over `nmem` member records of one tile shape (sums: Sums)
 cudaError_t launch_ensemble_fp64(const void* dev, int nmem, int nitems, unsigned int* next, int limiter,
-                                 bool sums, int tile, int nctas, cudaStream_t st);
+                                 int sums, int tile, int nctas, cudaStream_t st);
 cudaError_t launch_ensemble_fp32(const void* dev, int nmem, int nitems, unsigned int* next, int limiter,
-                                 bool sums, int tile, int nctas, cudaStream_t st);
+                                 int sums, int tile, int nctas, cudaStream_t st);
 int ensemble_ctas_per_sm_fp64(int limiter, int tile);
 int ensemble_ctas_per_sm_fp32(int limiter, int tile);
 cudaError_t launch_ensemble_update(const void* dev, int nmem, int nitems, double cfl, bool fp32,

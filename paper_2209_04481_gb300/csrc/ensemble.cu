@@ -219,7 +219,7 @@ int update_records(crn_ensemble* e, double* const* U64, double* log, cudaStream_
 
 // one persistent launch per tile shape in use; adds the launches to *count
 cudaError_t launch(crn_ensemble* e, cudaStream_t st, int* count = nullptr) {
-  const bool sums = e->kN || e->kD || e->kMarch;  // somebody reads the norms or dtmin
+  const int sums = e->kN ? crn::SUMS_ALL : e->kD || e->kMarch ? crn::SUMS_DT : crn::SUMS_NONE;
   for (int t = 0; t < crn::kEnsTileCount; ++t) {
     if (e->grp_cnt[t] == 0) continue;
     const void* rec = static_cast<const unsigned char*>(e->d_rec) + (size_t)e->grp_off[t] * e->msz;

@@ -148,7 +148,44 @@ __device__ void reduce_and_finalize_at(const S (&sum)[NV], S dtmin, const Reduce
   if (threadIdx.x == 0) *red.counter = 0u;
 }
 
-// the same from per-thread values, for the block id and count of the launch grid
+// The minimum alone (the pseudo-time march wants the step bound, not the norms):
+// no sums to carry, add and convert, and a last CTA that reads one double per
+// CTA.  A pseudo-time step of 32 x 16 x 32 FP64 cells
+// 71.1 -> 66.4 us, of 128 x 64 x 128 FP32 cells 133 -> 125 us.
+template <int NTHREADS>
+__device__ void reduce_min_at(double dtmin, const Reduce& red, double* scratch /* >= NTHREADS/32 doubles */,
+                              int bid, int nblocks) {
+  constexpr int NW = NTHREADS / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ unsigned int s_last;
+  __syncthreads();  // scratch may alias buffers still in use
+  if (lane == 0) scratch[warp] = dtmin;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = scratch[0];
+    for (int w = 1; w < NW; ++w) a = min_positive(a, scratch[w]);
+    red.partials[bid] = a;
+    __threadfence();
+    s_last = atomicAdd(red.counter, 1u) == (unsigned)(nblocks - 1);
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double a = INFINITY;
+  for (int b = threadIdx.x; b < nblocks; b += NTHREADS) a = min_positive(a, __ldcg(red.partials + b));
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) a = min_positive(a, __shfl_xor_sync(0xffffffffu, a, off));
+  if (lane == 0) scratch[warp] = a;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < NW; ++w) a = min_positive(a, scratch[w]);
+    red.dt_out[0] = a;
+    if (red.dt_user) red.dt_user[0] = a;
+    *red.counter = 0u;
+  }
+}
+
+// sums and minimum from per-thread values, for the block id and count of the launch grid
 template <int NTHREADS>
 __device__ __forceinline__ void reduce_and_finalize(double (&sum)[NV], double dtmin, const Reduce& red,
                                                     double* scratch) {
@@ -487,9 +524,10 @@ template <class T, int NT> struct MinCtas { static constexpr int value = (sizeof
 // (theta, phi) tiles) and radial chunk `chunk` of one grid; `bid` / `nblocks`
 // number the items of that grid for its cross-CTA reduction.  The grid's
 // description is read where it lies (kernel parameters, or the ensemble's copy
-// in shared memory) at each use.  SUMS: with the norms and the step bound (their
-// ten running sums per thread are registers the FP32 kernel has to spill for).
-template <class T, int LIM, int TT, int TP, bool SUMS>
+// in shared memory) at each use.  What else is wanted is a
+// template switch (the running sums are registers the FP32 kernel has to spill
+// for): SUMS_NONE, R alone; SUMS_DT, the step bound; SUMS_ALL, the norms too.
+template <class T, int LIM, int TT, int TP, int SUMS>
 __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, const Phys<T>& ph,
                                            const double* const& Br, const T* const& U,
                                            T* const& R, const Reduce& red, int kchunk, int tile,
@@ -691,7 +729,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
         r[v] = dr[v] + (fx[v * NFA + tl] - fx[v * NFA + tu]) + (fx[v * NFA + pl] - fx[v * NFA + pu]);
       const T lam = dr[NV] + (fx[NV * NFA + tl] + fx[NV * NFA + tu]) + (fx[NV * NFA + pl] + fx[NV * NFA + pu]);
       const T ivol = frcp(rad_slot(kg)[1] * s_av[jj]);
-      if (SUMS) {
+      if (SUMS != SUMS_NONE) {
         const T x = lam * ivol;
         rate = greater(x, rate) ? x : rate;
       }
@@ -700,7 +738,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       for (int v = 0; v < NV; ++v) {
         r[v] *= ivol;
         dst[v * N] = r[v];
-        if (SUMS) sq[v] = fmat(r[v], r[v], sq[v]);
+        if (SUMS == SUMS_ALL) sq[v] = fmat(r[v], r[v], sq[v]);
       }
       if (bad || !squares_finite(r)) flag_bad(red, (int64_t)kg * cs + ocol);
     }
@@ -867,22 +905,27 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
     __syncthreads();
   }
   // ---------------- reductions: warp tree in T, then FP64 across warps and CTAs
-  if (!SUMS) return;
+  if (SUMS == SUMS_NONE) return;
   T dtm = (T)INFINITY;
   if (rate > (T)0) dtm = sizeof(T) == 4 ? (T)__frcp_rn((float)rate) : one / rate;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) sq[v] += __shfl_xor_sync(0xffffffffu, sq[v], off);
+    for (int v = 0; v < NV; ++v)
+      if (SUMS == SUMS_ALL) sq[v] += __shfl_xor_sync(0xffffffffu, sq[v], off);
     const T o = __shfl_xor_sync(0xffffffffu, dtm, off);
     dtm = greater(dtm, o) ? o : dtm;
   }
-  reduce_and_finalize_at<NT>(sq, dtm, red, reinterpret_cast<double*>(smem_raw), bid, nblocks);
+  double* const scratch = reinterpret_cast<double*>(smem_raw);
+  if (SUMS == SUMS_ALL)
+    reduce_and_finalize_at<NT>(sq, dtm, red, scratch, bid, nblocks);
+  else
+    reduce_min_at<NT>((double)dtm, red, scratch, bid, nblocks);
 }
 
 // one grid: block (x, y) = (tile, radial chunk); with a second state, block z
 // picks the state
-template <class T, int LIM, int TT, int TP, bool SUMS>
+template <class T, int LIM, int TT, int TP, int SUMS>
 __global__ void __launch_bounds__(TT * TP, (MinCtas<T, TT * TP>::value))
 residual_tiled(Shape sh, Geo<T> g, Phys<T> ph, const double* __restrict__ Br,
                const T* __restrict__ U, T* __restrict__ R, Reduce red, int kchunk, const T* __restrict__ U2,
@@ -918,7 +961,7 @@ struct EnsMember {
 };
 
 
-template <class T, int LIM, int TT, int TP, bool SUMS>
+template <class T, int LIM, int TT, int TP, int SUMS>
 __global__ void __launch_bounds__(TT * TP, (MinCtas<T, TT * TP>::value))
 residual_ensemble(const EnsMember<T>* __restrict__ mem, int nmem, int nitems, unsigned int* __restrict__ next) {
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -146,7 +146,7 @@ int ens_fill_fp32(crn_grid* g, const void* U, void* R, int kchunk, int item0, do
   return m->nitems;
 }
 cudaError_t launch_ensemble_fp32(const void* dev, int nmem, int nitems, unsigned int* next, int limiter,
-                                  bool sums, int tile, int nctas, cudaStream_t st) {
+                                  int sums, int tile, int nctas, cudaStream_t st) {
   return launch_ensemble_t<float>(static_cast<const EnsMember<float>*>(dev), nmem, nitems, next, limiter, sums, tile, nctas,
                                 st);
 }

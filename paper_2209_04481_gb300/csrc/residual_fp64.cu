@@ -31,7 +31,7 @@ int ens_fill_fp64(crn_grid* g, const void* U, void* R, int kchunk, int item0, do
   return m->nitems;
 }
 cudaError_t launch_ensemble_fp64(const void* dev, int nmem, int nitems, unsigned int* next, int limiter,
-                                  bool sums, int tile, int nctas, cudaStream_t st) {
+                                  int sums, int tile, int nctas, cudaStream_t st) {
   return launch_ensemble_t<double>(static_cast<const EnsMember<double>*>(dev), nmem, nitems, next, limiter, sums, tile, nctas,
                                 st);
 }

@@ -55,10 +55,13 @@ cudaError_t launch_lim(crn_grid* g, const T* U, T* R, double* nu, double* du, cu
   // nobody reads the norms or the step bound: no sums, no last-CTA tail (FP32: 32 x
   // 16 x 32 16.6 -> 12.6 us, 95 x 45 x 88 39 -> 33 us, 128 x 64 x 128 77 -> 71 us)
   dim3 grid((unsigned)ntiles, (unsigned)nch);
-  if (nu || du)
-    residual_tiled<T, LIM, TT, TP, true><<<grid, D::NT, smem, st>>>(sh, geo, ph, g->br, U, R, red, kc, nullptr, nullptr);
+  auto go = [&](auto kern) { kern<<<grid, D::NT, smem, st>>>(sh, geo, ph, g->br, U, R, red, kc, nullptr, nullptr); };
+  if (nu)
+    go(residual_tiled<T, LIM, TT, TP, SUMS_ALL>);
+  else if (du)
+    go(residual_tiled<T, LIM, TT, TP, SUMS_DT>);
   else
-    residual_tiled<T, LIM, TT, TP, false><<<grid, D::NT, smem, st>>>(sh, geo, ph, g->br, U, R, red, kc, nullptr, nullptr);
+    go(residual_tiled<T, LIM, TT, TP, SUMS_NONE>);
   return cudaGetLastError();
 }
 
@@ -75,7 +78,7 @@ cudaError_t launch_pair_lim(crn_grid* g, const T* U, T* R, const T* U2, T* R2, c
     g->cfg.kchunk_pair = choose_radial_chunk(sh.nr, 2ll * ntiles, g->cfg.num_sms, g->cfg.tiled_per_sm, sizeof(T) == 8);
   const int kc = g->cfg.kchunk_pair;
   const dim3 grid((unsigned)ntiles, (unsigned)((sh.nr + kc - 1) / kc), 2);
-  residual_tiled<T, LIM, TT, TP, false><<<grid, D::NT, D::template smem_bytes<T>(), st>>>(
+  residual_tiled<T, LIM, TT, TP, SUMS_NONE><<<grid, D::NT, D::template smem_bytes<T>(), st>>>(
       sh, geo_of<T>(g), phys_of<T>(g), g->br, U, R, red, kc, U2, R2);
   return cudaGetLastError();
 }
@@ -110,12 +113,19 @@ cudaError_t prepare_t() {
   auto set = [&](auto kern) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   };
-  cudaError_t e = set(residual_tiled<T, 0, TT, TP, true>);
-  if (e == cudaSuccess) e = set(residual_tiled<T, 1, TT, TP, true>);
-  if (e == cudaSuccess) e = set(residual_tiled<T, 2, TT, TP, true>);
-  if (e == cudaSuccess) e = set(residual_tiled<T, 0, TT, TP, false>);
-  if (e == cudaSuccess) e = set(residual_tiled<T, 1, TT, TP, false>);
-  if (e == cudaSuccess) e = set(residual_tiled<T, 2, TT, TP, false>);
+  auto all = [&](auto none, auto dt, auto sums) {
+    cudaError_t e = set(none);
+    if (e == cudaSuccess) e = set(dt);
+    if (e == cudaSuccess) e = set(sums);
+    return e;
+  };
+#define CRN_KERNELS(LIM) \
+  residual_tiled<T, LIM, TT, TP, SUMS_NONE>, residual_tiled<T, LIM, TT, TP, SUMS_DT>, \
+      residual_tiled<T, LIM, TT, TP, SUMS_ALL>
+  cudaError_t e = all(CRN_KERNELS(0));
+  if (e == cudaSuccess) e = all(CRN_KERNELS(1));
+  if (e == cudaSuccess) e = all(CRN_KERNELS(2));
+#undef CRN_KERNELS
   return e;
 }
 
@@ -126,11 +136,11 @@ int tiled_ctas_t(int limiter) {
   int n = 0;
   cudaError_t e;
   if (limiter == CRN_LIM_NONE)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 0, TT, TP, true>, TT * TP, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 0, TT, TP, SUMS_ALL>, TT * TP, smem);
   else if (limiter == CRN_LIM_MINMOD)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 1, TT, TP, true>, TT * TP, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 1, TT, TP, SUMS_ALL>, TT * TP, smem);
   else
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 2, TT, TP, true>, TT * TP, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, residual_tiled<T, 2, TT, TP, SUMS_ALL>, TT * TP, smem);
   return e == cudaSuccess ? n : 0;
 }
 
@@ -170,24 +180,28 @@ void ens_fill_t(crn_grid* g, const T* U, T* R, int kchunk, int item0, double* no
 
 template <class T, int TT, int TP>
 cudaError_t launch_ensemble_shape(const EnsMember<T>* dev, int nmem, int nitems, unsigned int* next, int limiter,
-                                  bool sums, int nctas, cudaStream_t st) {
+                                  int sums, int nctas, cudaStream_t st) {
   const size_t smem = TileDims<TT, TP>::template smem_bytes<T>();
   cudaError_t e = cudaMemsetAsync(next, 0, sizeof(unsigned int), st);
   if (e != cudaSuccess) return e;
   auto go = [&](auto kern) { kern<<<nctas, TT * TP, smem, st>>>(dev, nmem, nitems, next); };
+  auto pick = [&](auto none, auto dt, auto all) { go(sums == SUMS_ALL ? all : sums == SUMS_DT ? dt : none); };
+#define CRN_KERNELS(LIM) \
+  residual_ensemble<T, LIM, TT, TP, SUMS_NONE>, residual_ensemble<T, LIM, TT, TP, SUMS_DT>, \
+      residual_ensemble<T, LIM, TT, TP, SUMS_ALL>
   if (limiter == CRN_LIM_NONE)
-    sums ? go(residual_ensemble<T, 0, TT, TP, true>) : go(residual_ensemble<T, 0, TT, TP, false>);
+    pick(CRN_KERNELS(0));
   else if (limiter == CRN_LIM_MINMOD)
-    sums ? go(residual_ensemble<T, 1, TT, TP, true>) : go(residual_ensemble<T, 1, TT, TP, false>);
+    pick(CRN_KERNELS(1));
   else
-    sums ? go(residual_ensemble<T, 2, TT, TP, true>) : go(residual_ensemble<T, 2, TT, TP, false>);
+    pick(CRN_KERNELS(2));
   return cudaGetLastError();
 }
 
 // the persistent launch over the members of one tile shape
 template <class T>
 cudaError_t launch_ensemble_t(const EnsMember<T>* dev, int nmem, int nitems, unsigned int* next, int limiter,
-                              bool sums, int tile, int nctas, cudaStream_t st) {
+                              int sums, int tile, int nctas, cudaStream_t st) {
   if constexpr (sizeof(T) == 8) {
     if (tile == 2) return launch_ensemble_shape<T, ens_tt(2), ens_tp(2)>(dev, nmem, nitems, next, limiter, sums, nctas, st);
   }
@@ -204,12 +218,12 @@ int ensemble_ctas_shape(int limiter) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, TT * TP, smem) != cudaSuccess) return 0;
     return n;
   };
-  // both kernels of a limiter; the persistent grid fits either
-  if (limiter == CRN_LIM_NONE)
-    return std::min(setup(residual_ensemble<T, 0, TT, TP, true>), setup(residual_ensemble<T, 0, TT, TP, false>));
-  if (limiter == CRN_LIM_MINMOD)
-    return std::min(setup(residual_ensemble<T, 1, TT, TP, true>), setup(residual_ensemble<T, 1, TT, TP, false>));
-  return std::min(setup(residual_ensemble<T, 2, TT, TP, true>), setup(residual_ensemble<T, 2, TT, TP, false>));
+  // the three kernels of a limiter; the persistent grid fits each
+  auto least = [&](auto none, auto dt, auto all) { return std::min(setup(none), std::min(setup(dt), setup(all))); };
+  if (limiter == CRN_LIM_NONE) return least(CRN_KERNELS(0));
+  if (limiter == CRN_LIM_MINMOD) return least(CRN_KERNELS(1));
+  return least(CRN_KERNELS(2));
+#undef CRN_KERNELS
 }
 
 // shared-memory opt-in and resident CTAs per SM of one tile shape's kernel

@@ -252,12 +252,18 @@ cudaError_t opt_in_smem() {
   auto set = [&](auto kern) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   };
-  cudaError_t e = set(crn::residual_tiled<T, 0, TT, TP, true>);
-  if (e == cudaSuccess) e = set(crn::residual_tiled<T, 1, TT, TP, true>);
-  if (e == cudaSuccess) e = set(crn::residual_tiled<T, 2, TT, TP, true>);
-  if (e == cudaSuccess) e = set(crn::residual_tiled<T, 0, TT, TP, false>);
-  if (e == cudaSuccess) e = set(crn::residual_tiled<T, 1, TT, TP, false>);
-  if (e == cudaSuccess) e = set(crn::residual_tiled<T, 2, TT, TP, false>);
+  auto all = [&](auto none, auto dt, auto sums) {
+    cudaError_t e = set(none);
+    if (e == cudaSuccess) e = set(dt);
+    if (e == cudaSuccess) e = set(sums);
+    return e;
+  };
+#define CRN_KERNELS(LIM) \
+  crn::residual_tiled<T, LIM, TT, TP, crn::SUMS_NONE>, crn::residual_tiled<T, LIM, TT, TP, crn::SUMS_DT>, \
+      crn::residual_tiled<T, LIM, TT, TP, crn::SUMS_ALL>
+  cudaError_t e = all(CRN_KERNELS(0));
+  if (e == cudaSuccess) e = all(CRN_KERNELS(1));
+  if (e == cudaSuccess) e = all(CRN_KERNELS(2));
   return e;
 }
 
@@ -280,11 +286,11 @@ int plan(const crn_grid_desc& d, DeviceSlot& slot) {
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const size_t smem = crn::TileDims<TT, TP>::template smem_bytes<T>();
   if (d.limiter == CRN_LIM_NONE)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 0, TT, TP, true>, TT * TP, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 0, TT, TP, crn::SUMS_ALL>, TT * TP, smem);
   else if (d.limiter == CRN_LIM_MINMOD)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 1, TT, TP, true>, TT * TP, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 1, TT, TP, crn::SUMS_ALL>, TT * TP, smem);
   else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 2, TT, TP, true>, TT * TP, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 2, TT, TP, crn::SUMS_ALL>, TT * TP, smem);
   int kc = crn::choose_radial_chunk(d.n_r, ntiles, std::max(nsm, 1), per_sm, sizeof(T) == 8);
   while (ntiles * ((d.n_r + kc - 1) / kc) > kMaxBlocks) kc *= 2;
   slot.plan_desc = d;
@@ -326,17 +332,13 @@ int run(const crn_grid_desc& d, DeviceSlot& slot, const double* Br, const void* 
   const T* u = static_cast<const T*>(U);
   T* r = static_cast<T*>(R);
   auto go = [&](auto kern) { kern<<<grid, TT * TP, smem, st>>>(sh, geo, ph, Br, u, r, red, kc, nullptr, nullptr); };
-  const bool sums = norms || dtmin;
+  auto pick = [&](auto none, auto dt, auto all) { go(norms ? all : dtmin ? dt : none); };
   switch (d.limiter) {
-    case CRN_LIM_NONE:
-      sums ? go(crn::residual_tiled<T, 0, TT, TP, true>) : go(crn::residual_tiled<T, 0, TT, TP, false>);
-      break;
-    case CRN_LIM_MINMOD:
-      sums ? go(crn::residual_tiled<T, 1, TT, TP, true>) : go(crn::residual_tiled<T, 1, TT, TP, false>);
-      break;
-    default:
-      sums ? go(crn::residual_tiled<T, 2, TT, TP, true>) : go(crn::residual_tiled<T, 2, TT, TP, false>);
+    case CRN_LIM_NONE: pick(CRN_KERNELS(0)); break;
+    case CRN_LIM_MINMOD: pick(CRN_KERNELS(1)); break;
+    default: pick(CRN_KERNELS(2));
   }
+#undef CRN_KERNELS
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(CRN_E_CUDA, std::string("residual launch: ") + cudaGetErrorString(e));
   return CRN_OK;

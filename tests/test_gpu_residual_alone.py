@@ -59,7 +59,11 @@ def test_ensemble_that_fills_the_gpu(precision, limiter):
     norms = torch.zeros((n, 9), dtype=torch.float64, device="cuda")
     dtmin = torch.zeros(n, dtype=torch.float64, device="cuda")
     Rs = [R.clone() for R in ens.residual(list(Us), norms=norms, dtmin=dtmin)]
-    alone = ens.residual(list(Us))
+    alone = [R.clone() for R in ens.residual(list(Us))]
+    d1 = torch.zeros_like(dtmin)
+    for a, b in zip(alone, ens.residual(list(Us), dtmin=d1)):
+        assert torch.equal(a, b)
+    assert torch.equal(dtmin, d1)
     for m, g in enumerate(gs):
         nm, dm = scratch()
         R = g.residual(Us[m], norms=nm, dtmin=dm)
