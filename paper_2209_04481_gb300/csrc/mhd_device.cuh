@@ -79,6 +79,11 @@ template <class T> __device__ __forceinline__ T fmat(T a, T b, T c);
 template <> __device__ __forceinline__ double fmat<double>(double a, double b, double c) { return fma(a, b, c); }
 template <> __device__ __forceinline__ float fmat<float>(float a, float b, float c) { return fmaf(a, b, c); }
 
+// a product that is rounded by itself in FP64 (not contracted into a sum), so that
+// a kept one and one formed in place are the same number
+__device__ __forceinline__ double product(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float product(float a, float b) { return a * b; }
+
 // Reciprocal and square root.  The FP64 pipe runs at 1/64 of the FP32 rate, so
 // their FP64 operations are counted: both start from the approximate PTX
 // instructions (about 20 bits, not on the FP64 pipe) and take one cubic step.
@@ -162,6 +167,17 @@ __device__ __forceinline__ bool greater(float x, float y) { return x > y; }
 __device__ __forceinline__ bool greater(double x, double y) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   return b > (unsigned long long)__double_as_longlong(y) && b <= 0x7ff0000000000000ull;
+}
+
+// x / 2 and 2 x of a normal x >= 0 (or 0) by its exponent, on the integer pipe;
+// infinities and NaNs stay
+__device__ __forceinline__ double halved(double x) {
+  const int hi = __double2hiint(x), e = hi & 0x7ff00000;
+  return __hiloint2double(e != 0 && e != 0x7ff00000 ? hi - 0x00100000 : hi, __double2loint(x));
+}
+__device__ __forceinline__ double doubled(double x) {
+  const int hi = __double2hiint(x), e = hi & 0x7ff00000;
+  return __hiloint2double(e != 0 && e != 0x7ff00000 ? hi + 0x00100000 : hi, __double2loint(x));
 }
 
 // |x| to FP32, cut off (not rounded), by integer instructions: 0 below the FP32
@@ -514,9 +530,9 @@ __device__ __forceinline__ void rusanov(const double (&wl)[NV], const double (&w
     }
     lam = greater(lam, ph.ch) ? lam : ph.ch;
   }
-  const double h = 0.5 * area;
-  lam_area = lam * area;
+  const double h = halved(area);
   const double d = lam * h;
+  lam_area = doubled(d);
   const double ul = h * L.un, ur = h * R.un, bl = h * L.bn, br = h * R.bn;
   const double ml = wl[0] * ul, mr = wr[0] * ur;
   const double pt = h * (L.pt + R.pt), ps = h * (wl[8] + wr[8]);

@@ -483,11 +483,12 @@ struct TileDims {
   // r-face normals, own radial unit vectors, theta factors of the areas/volumes
   static constexpr int NGEO = 3 * NTV + 2 * (TP + 1) + 6 * NT + (TT + 1) + 2 * TT;
   static constexpr int NRAD = 8;                                // radial factors of a plane, three planes held
+  static constexpr int NROW = 6 * (TT + 1);                     // factors of the tile's rows in one plane (1 / V: two)
   template <class T>
   static constexpr size_t smem_bytes() {
     return sizeof(unsigned) * (size_t)NITEM +
            sizeof(T) * ((size_t)NV * HC + (size_t)NV * NUV + (size_t)NF * NFA +
-                        (size_t)NV * NHALO + (size_t)3 * NRAD + (size_t)NGEO);
+                        (size_t)NV * NHALO + (size_t)3 * NRAD + (size_t)NROW + (size_t)NGEO);
   }
   // halo position h in [0, NHALO) -> halo'd (row, col)
   __device__ static void halo_rc(int h, int& row, int& col) {
@@ -544,7 +545,9 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
   T* fx = uv + NV * NUV;                     // [NF][NFA]  flux x area of each face, lambda x area last
   T* hr = fx + NF * NFA;                     // [NV][NHALO] raw halo cells of plane k + 1
   T* s_rad = hr + NV * D::NHALO;             // [3][NRAD] radial factors of planes k .. k + 2
-  T* s_nth = s_rad + 3 * D::NRAD;            // [3][NTV]
+  T* s_row = s_rad + 3 * D::NRAD;            // [6][TT + 1] by row: r and theta face areas, V, gravity x V of plane k,
+                                             //   1 / V of planes k and k - 1
+  T* s_nth = s_row + D::NROW;                // [3][NTV]
   T* s_nph = s_nth + 3 * NTV;                // [2][TP + 1]
   T* s_nr = s_nph + 2 * (TP + 1);            // [3][NT]
   T* s_rh = s_nr + 3 * NT;                   // [3][NT]
@@ -588,6 +591,11 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
   T rL[NV];           // L state of r face k + 1/2 (upper r value of plane k)
   T frl[NF];          // flux x area of r face k - 1/2, lambda x area last
   T pf_own[NV];       // raw own cell of plane k + 2
+  // FP64: the forward difference of plane k, which is the backward one of plane
+  // k + 1 (the same two cells over the same distance).  FP32 forms it again: its
+  // registers are full.
+  constexpr bool CARRY = sizeof(T) == 8;
+  T fwd[CARRY ? NV : 1];
   // radial factor tid of plane p: r_b, r_v and gravity of p, face area factor of
   // its upper face, slope and face distances of plane p + 1.  They come in with
   // the halo cells, two planes ahead: a global load where they are used would
@@ -682,7 +690,8 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       const T im = g.inv_dm[k0], ip = g.inv_dp[k0], hm = g.hm[k0], hp = g.hp[k0];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const T s = limited_slope<LIM>((wc[v] - wm1[v]) * im, (w1[v] - wc[v]) * ip, ph.eps);
+        const T s = limited_slope<LIM>(product(wc[v] - wm1[v], im), product(w1[v] - wc[v], ip), ph.eps);
+        if constexpr (CARRY) fwd[v] = product(w1[v] - wc[v], ip);
         wr[v] = fmat(-s, hm, wc[v]);
         rL[v] = fmat(s, hp, wc[v]);
       }
@@ -694,7 +703,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       const T im = g.inv_dm[k0 - 1], ip = g.inv_dp[k0 - 1], hp = g.hp[k0 - 1];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const T s = limited_slope<LIM>((wm1[v] - wm2[v]) * im, (wc[v] - wm1[v]) * ip, ph.eps);
+        const T s = limited_slope<LIM>(product(wm1[v] - wm2[v], im), product(wc[v] - wm1[v], ip), ph.eps);
         wl[v] = fmat(s, hp, wm1[v]);
       }
     }
@@ -715,6 +724,12 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
   for (int v = 0; v < NV; ++v) sq[v] = (T)0;
   T rate = (T)0;      // largest lambda |S| / V of the thread's cells
   T dr[NF];           // r faces' contribution to the cell being gathered
+  // FP64: the plane's factors of each row once, by one thread per row: a product
+  // or a reciprocal in every thread is an operation of the FP64 pipe per warp.
+  // FP32 forms them in place (with the table the ensemble was 1 % slower).
+  constexpr bool ROWS = sizeof(T) == 8;
+  T* const row_ar = s_row, * const row_at = s_row + (TT + 1), * const row_v = s_row + 2 * (TT + 1);
+  T* const row_gv = s_row + 3 * (TT + 1), * const row_iv = s_row + 4 * (TT + 1);
   bool bad = false;   // rho <= 0 or p <= 0 in that cell
 
   for (int k = k0;; ++k) {
@@ -727,9 +742,9 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
 #pragma unroll
       for (int v = 0; v < NV; ++v)
         r[v] = dr[v] + (fx[v * NFA + tl] - fx[v * NFA + tu]) + (fx[v * NFA + pl] - fx[v * NFA + pu]);
-      const T lam = dr[NV] + (fx[NV * NFA + tl] + fx[NV * NFA + tu]) + (fx[NV * NFA + pl] + fx[NV * NFA + pu]);
-      const T ivol = frcp(rad_slot(kg)[1] * s_av[jj]);
+      const T ivol = ROWS ? row_iv[(kg & 1) * (TT + 1) + jj] : frcp(rad_slot(kg)[1] * s_av[jj]);
       if (SUMS != SUMS_NONE) {
+        const T lam = dr[NV] + (fx[NV * NFA + tl] + fx[NV * NFA + tu]) + (fx[NV * NFA + pl] + fx[NV * NFA + pu]);
         const T x = lam * ivol;
         rate = greater(x, rate) ? x : rate;
       }
@@ -743,6 +758,18 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       if (bad || !squares_finite(r)) flag_bad(red, (int64_t)kg * cs + ocol);
     }
     if (k >= k1) break;
+    if (ROWS && tid >= NT - 32 && tid - (NT - 32) <= TT) {
+      const int q = tid - (NT - 32);
+      const T* rad = rad_slot(k);
+      row_at[q] = rad[0] * s_at[q];
+      if (q < TT) {
+        const T vol = rad[1] * s_av[q];
+        row_ar[q] = rad[3] * s_ar[q];
+        row_v[q] = vol;
+        row_gv[q] = -(rad[2] * vol);
+        row_iv[(k & 1) * (TT + 1) + q] = frcp(vol);
+      }
+    }
     T tlo[NV], plo[NV];  // the cell's lower theta and phi face values
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -781,14 +808,14 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
         T wl[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) wl[v] = uv[v * NUV + tid];
-        rusanov<true>(wl, tlo, s_nth[tid], s_nth[NTV + tid], s_nth[2 * NTV + tid], rbk * s_at[jj], ph, fl, la);
+        rusanov<true>(wl, tlo, s_nth[tid], s_nth[NTV + tid], s_nth[2 * NTV + tid], ROWS ? row_at[jj] : rbk * s_at[jj], ph, fl, la);
       } else {
 #pragma unroll
         for (int v = 0; v < NV; ++v) fl[v] = (T)0;
       }
 #pragma unroll
       for (int v = 0; v < NV; ++v) fx[v * NFA + tid] = fl[v];
-      fx[NV * NFA + tid] = la;
+      if (SUMS != SUMS_NONE) fx[NV * NFA + tid] = la;
     }
     {  // lower phi face of the own cell
       const int f = NTV + jj * (TP + 1) + ii;
@@ -804,7 +831,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       }
 #pragma unroll
       for (int v = 0; v < NV; ++v) fx[v * NFA + f] = fl[v];
-      fx[NV * NFA + f] = la;
+      if (SUMS != SUMS_NONE) fx[NV * NFA + f] = la;
     }
     if (tid >= NT - ((NXF + 31) / 32) * 32) {  // the faces past the last row and column: the last warps
       const int e = tid - (NT - ((NXF + 31) / 32) * 32);
@@ -816,7 +843,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
           f = TT * TP + e;
           live = j0 + TT < nt && i0 + e < np;
           nx = s_nth[f]; ny = s_nth[NTV + f]; nz = s_nth[2 * NTV + f];
-          area = rbk * s_at[TT];
+          area = ROWS ? row_at[TT] : rbk * s_at[TT];
         } else {
           const int r = e - TP;
           f = NTV + r * (TP + 1) + TP;
@@ -836,7 +863,7 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
         }
 #pragma unroll
         for (int v = 0; v < NV; ++v) fx[v * NFA + f] = fl[v];
-        fx[NV * NFA + f] = la;
+        if (SUMS != SUMS_NONE) fx[NV * NFA + f] = la;
       }
     }
     // r face k + 1/2 and the plane k + 1 that follows
@@ -852,7 +879,14 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
         const T im = rad[4], ip = rad[5], hm = rad[6], hp = rad[7];
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-          const T s = limited_slope<LIM>((w1[v] - wc[v]) * im, (w2[v] - w1[v]) * ip, ph.eps);
+          T s;
+          if constexpr (CARRY) {
+            const T b = product(w2[v] - w1[v], ip);
+            s = limited_slope<LIM>(fwd[v], b, ph.eps);
+            fwd[v] = b;
+          } else {
+            s = limited_slope<LIM>(product(w1[v] - wc[v], im), product(w2[v] - w1[v], ip), ph.eps);
+          }
           rR[v] = fmat(-s, hm, w1[v]);
           rLn[v] = fmat(s, hp, w1[v]);
         }
@@ -862,14 +896,14 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       }
       if (own) {
         T f[NV], la;
-        rusanov<true>(rL, rR, s_nr[tid], s_nr[NT + tid], s_nr[2 * NT + tid], rad[3] * s_ar[jj], ph, f, la);
+        rusanov<true>(rL, rR, s_nr[tid], s_nr[NT + tid], s_nr[2 * NT + tid], ROWS ? row_ar[jj] : rad[3] * s_ar[jj], ph, f, la);
 #pragma unroll
         for (int v = 0; v < NV; ++v) { dr[v] = frl[v] - f[v]; frl[v] = f[v]; }
         dr[NV] = frl[NV] + la;
         frl[NV] = la;
         // the sources in flux units (x V): gravity [Sect. 2.2] and GLM damping
-        const T vol = rad[1] * s_av[jj];
-        const T a = -(rad[2] * vol) * wc[0];
+        const T vol = ROWS ? row_v[jj] : rad[1] * s_av[jj];
+        const T a = (ROWS ? row_gv[jj] : -(rad[2] * vol)) * wc[0];
         const T ex = s_rh[tid], ey = s_rh[NT + tid], ez = s_rh[2 * NT + tid];
         dr[1] = fmat(a, ex, dr[1]);
         dr[2] = fmat(a, ey, dr[2]);
