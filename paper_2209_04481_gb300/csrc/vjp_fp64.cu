@@ -6,8 +6,17 @@ cudaError_t launch_vjp_fp64(crn_grid* g, const double* U, const double* Rb, doub
                             cudaStream_t st, int* nl) {
   return vjp_t<double>(g, U, Rb, Ub, Brb, st, nl);
 }
-size_t vjp_scratch_bytes(const crn_grid* g) {
-  if (!vjp_uses_scratch(g)) return 0;
-  return vjp_scratch_elems(g->shape, g->d.precision == CRN_FP64) * (g->d.precision == CRN_FP64 ? 8 : 4);
+// The scratch of the slope/face/cell passes, if this grid runs them, at its first
+// VJP.  1.15 kB per FP64 cell, where the kernels that formed the slopes at the
+// faces took 0.94: a shell that fitted then and does not now runs the tiled VJP.
+cudaError_t vjp_ensure_scratch(crn_grid* g) {
+  if (g->vjp_buf || g->vjp_no_room || !vjp_uses_scratch(g)) return cudaSuccess;
+  const bool fp64 = g->d.precision == CRN_FP64;
+  const cudaError_t e = cudaMalloc(&g->vjp_buf, vjp_scratch_elems(g->shape, fp64) * (fp64 ? 8 : 4));
+  if (e != cudaErrorMemoryAllocation || !fp64) return e;
+  cudaGetLastError();
+  g->vjp_buf = nullptr;
+  g->vjp_no_room = true;
+  return cudaSuccess;
 }
 }  // namespace crn
