@@ -123,8 +123,9 @@ template <> __device__ __forceinline__ float fsqrt<float>(float x) { return sqrt
 // and warp, against four FP64 operations): Newton's series y0 (1 + e + e^2) for
 // 2^63 / d's significand from an FP32 reciprocal y0 (24 bits, e < 2^-22, so that
 // e^3 is below the last bit kept), times n's significand, rounded once: within
-// 0.51 units in the last place (truncations of 2^-60 at most before it).  A quotient below the normal range and one of a
-// subnormal n are 0; an infinite or NaN operand gives a NaN.
+// 0.51 units in the last place (truncations of 2^-60 at most before it).  A
+// quotient below the normal range and one of a subnormal n are 0; an infinite or
+// NaN operand gives a NaN.  128 x 64 x 128 FP64: 1906 -> 1668 us.
 __device__ __forceinline__ float quotient(float n, float d) { return n * frcp(d); }
 __device__ __forceinline__ double quotient(double n, double d) {
   typedef unsigned long long u64;
@@ -371,7 +372,8 @@ __device__ __forceinline__ T limited_slope(T a, T b, T eps) {
 // slowest pipe, so its operations are counted: h = |S|/2 is multiplied into
 // u_n, B_n and rho u_n once per side instead of into each of the nine sums, and
 // the pressure and GLM gradient terms of both sides are added before they meet
-// the normal (159 operations and 4 for the square roots against about 200; every FMA explicit).  FP32
+// the normal: 109 operations, and 24 for each fast speed that is formed, against
+// about 200 in all (every FMA explicit).  FP32
 // keeps the sums by side: there the regrouping saved 3 % and moved the momentum
 // of the polar cells, whose opposite faces nearly cancel, by 1e-7 per step.
 // ---------------------------------------------------------------------------

@@ -4,17 +4,18 @@
 // on how the CTAs fall on the SMs, so the launch of every candidate chunk is
 // simulated: CTAs start in launch order (all tiles of chunk 0, then chunk 1,
 // ...) on the first free slot, the first `nsm` of them on SMs of their own.
-// Measured on 152 SMs (152 x {1, 2} CTAs of 256 FP32 or 128 FP64 threads):
-//   * an FP32 CTA alone on its SM takes 2.7 us per plane, two on one SM 4.8 us
-//     each; FP64 42 us and 74 us: two CTAs run at 0.57 of the rate of one;
+// Measured on 152 SMs, norms included (152 x {1, 2} CTAs of 256 FP32 or 128 FP64 threads):
+//   * two CTAs on one SM take 4.8 us per plane where one takes 2.7 (FP32), 74
+//     where one takes 42 (FP64): two CTAs run at 0.57 of the rate of one;
 //   * the preamble (first loads, the redundant r face at the chunk's start, and
 //     the closing reduction) takes about 1.5 planes in FP32 and 0.5 in FP64,
 //     and since it is latency it does not slow down beside another CTA.
 // The chunk it picks was the fastest of those timed on every grid swept: 14 of
-// 128 planes on 128 x 64 x 128 in FP32 (76 us; 13: 109, 16: 83) and 9 in FP64
-// (2.10 ms; 8: 2.23, 16: 2.39), 6 on 95 x 45 x 88 (39 us; 12: 48), 2 on
-// 64 x 32 x 64 (21 us; 4: 25), 1 on 32 x 16 x 32 (16.5 us against 23 with 4
-// planes; FP64 73 us against 198), 12 on 96 x 48 x 96 FP64 (0.75 ms).
+// 128 planes on 128 x 64 x 128 in FP32 (64 us; 7: 68, 12: 84, 16: 71) and 9 in
+// FP64 (1.53 ms; 7 to 16: 1.65 to 1.86 before the last 4 %), 6 on 95 x 45 x 88
+// (31 us; 12: 39), 2 on 64 x 32 x 64 (17 us; 4: 19), 1 on 32 x 16 x 32 (12 us
+// against 19 with 4 planes; FP64 60 us against 176), 12 on 96 x 48 x 96 FP64
+// (0.63 ms; 16: 0.87).
 #include <algorithm>
 #include <queue>
 #include <vector>

@@ -25,8 +25,8 @@ namespace crn {
 struct Reduce {
   double* partials;          // [gridDim.x * gridDim.y][16]
   unsigned int* counter;     // CTA arrival counter, reset by the last CTA
-  double* norms_out;         // [9] L2 norms (always written)
-  double* dt_out;            // [1] min V / sum lambda |S| (always written)
+  double* norms_out;         // [9] L2 norms, where the kernel forms them
+  double* dt_out;            // [1] min V / sum lambda |S|, likewise
   double* norms_user;        // optional copy for the caller
   double* dt_user;           // optional copy for the caller
   unsigned int* err_flags;   // bit 0: non-physical or non-finite cell
@@ -440,12 +440,13 @@ __device__ __forceinline__ bool squares_finite(const double (&r)[NV]) {
 //      plane k + 1 replaces plane k in shared memory; the loads of the own
 //      cell of plane k + 3 and the halo of plane k + 2 are issued
 //
-// FP32 is bound by instruction issue at 16 warps per SM (128 registers): 61 %
-// of the slots at 1575 instructions per cell, 920 of them on the FMA pipe.
-// 128 x 64 x 128: 77 us, against 87 us for three phases per plane with a ring
-// of three planes, both face values in shared memory and a global load per
-// radial factor (55 % of the slots, 1660 instructions).  FP64 is bound by the
-// FP64 pipe: about 1020 operations per cell, 2.10 ms (2.65 ms with 1208).
+// FP32 is bound by instruction issue at 16 warps per SM (128 registers): 66 %
+// of the slots at 1545 instructions per cell.  128 x 64 x 128, R alone: 64 us
+// (90 us with three phases per plane, a ring of three planes, both face values
+// in shared memory, a global load per radial factor and the sums always; 72 us
+// with the halo items worked out from their number on every plane).  FP64 is
+// bound by the FP64 pipe (88 % busy): about 790 operations per cell, 1.53 ms
+// (2.65 ms with 1208).
 template <int TT, int TP>
 struct TileDims {
   static constexpr int NT = TT * TP;                            // threads = own columns
@@ -784,7 +785,8 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       uv[v * NUV + NTV + jj * (TP + 1) + ii + 1] = fmat(half, sf, w);
     }
     // halo cells whose face values the tile's boundary faces need: three
-    // variables of one cell per item
+    // variables of one cell per item, the items packed once per CTA (worked out
+    // from x on every plane they took 8 us of 72 in FP32 and 75 of 1670 in FP64)
     for (int x = tid; x < 3 * NX; x += NT) {
       const unsigned it = s_item[x];
       const int step = (it & (1u << 30)) ? HP : 1;

@@ -26,8 +26,9 @@
 //               of the recovery and of the sources
 // The first version evaluated the slopes and their derivatives at each of the
 // six faces that use them and stored 36 values per face: 3350 FP64 operations
-// per cell, 5.67 ms on 128 x 64 x 128; now about 2250 and 3.87 ms (64 x 32 x 64:
-// 0.75 -> 0.53 ms, of it slopes 0.18, faces 0.22, cells 0.13).
+// per cell, 5.67 ms on 128 x 64 x 128; now about 2100 and 3.62 ms (64 x 32 x 64:
+// 0.75 -> 0.50 ms, of it slopes 0.18, faces 0.19, cells 0.13; 3.87 and 0.53 ms
+// before the FP32 bound of the fast speeds).
 // Non-smooth points follow the oracle's conventions: max(a, b) passes the
 // derivative to a on a tie, d|x|/dx = +1 at 0, the clamp of the fast-speed
 // discriminant at 0 has zero derivative.
