@@ -61,8 +61,8 @@ typedef enum { CRN_LIM_NONE = 0, CRN_LIM_MINMOD = 1, CRN_LIM_VANALBADA = 2 } crn
  * FP64).  STAGED (FP32_BULK only): each plane's own 8 x 32 block arrives by a
  * TMA tensor copy and the halo by cp.async; it needs n_theta a multiple of 8,
  * n_phi a multiple of 32 and a 16-byte aligned state, else the tiled kernel
- * runs.  It computes the same residual and is slower on GB300 (127 us against
- * 86 us on 128 x 64 x 128).  CELLWISE: a simple reference kernel, one thread
+ * runs.  It computes the same residual and is slower on GB300 (121 us against
+ * 64 us on 128 x 64 x 128).  CELLWISE: a simple reference kernel, one thread
  * per cell.  crn_last_kernel reports the kernel that ran. */
 typedef enum {
   CRN_KERNEL_TILED = 0,
@@ -181,8 +181,8 @@ int crn_residual(crn_grid* g, const void* U_dev, void* R_dev, double* norms9_dev
  * passes, one thread per cell, per face and per cell again, 3 launches (2 with
  * FP32, which forms its slopes where they are used), with a scratch of about 144
  * values of the grid's type per cell (54 with FP32) allocated by the grid's
- * first VJP call: make that call before
- * any stream capture.  The environment variable CRN_VJP_KERNEL ("tiled" or
+ * first VJP call: make that call before any stream capture.  An FP64 grid whose
+ * scratch does not fit in device memory runs the tiled passes.  The environment variable CRN_VJP_KERNEL ("tiled" or
  * "faces"), read at each call, overrides the choice.  Ubar_dev must not
  * overlap U_dev or Rbar_dev (CRN_E_ARG).  Asynchronous. */
 int crn_residual_vjp(crn_grid* g, const void* U_dev, const void* Rbar_dev, void* Ubar_dev,

@@ -90,8 +90,9 @@ int member_chunk(const crn_ensemble* e, int m) {
 // here the members fill the GPU together.  For each target length every member
 // takes the even split next to it, the items are list-scheduled longest first
 // (the order the records are laid out in) onto the resident CTAs, and the target
-// with the shortest makespan wins.  Eight shells of 4.9 M cells: 362 us against
-// 419 us with the own chunks of 2 to 26 planes.  Ensembles of fewer than four
+// with the shortest makespan wins.  Eight FP32 shells of 4.9 M cells:
+// 310 us, the best single chunk for all 346 us; when the kernel was slower 362 us
+// against 419 us with the own chunks of 2 to 26 planes.  Ensembles of fewer than four
 // (tile, plane) pairs per CTA keep the members' own chunks.
 void plan_chunks(crn_ensemble* e) {
   const bool fp64 = e->precision == CRN_FP64;
