@@ -446,6 +446,11 @@ struct StepMin {
   unsigned int* bits;      // [2] minima as FP32 bit patterns (0x7f800000 between launches)
   unsigned int* counter;
 };
+// the counter and the minima before the first launch
+__global__ void sync_init_kernel(unsigned int* sync) {
+  sync[0] = 0u;
+  sync[1] = sync[2] = 0x7f800000u;
+}
 constexpr int NKE = 128;  // threads per block: long threads, and a small shell has few cells
 template <class TV>
 __global__ void __launch_bounds__(NKE)
@@ -950,7 +955,9 @@ bool use_basis32(const crn_nk_options& o) {
   return o.basis_fp32 == 1 || (o.basis_fp32 == -1 && o.lin_rtol >= 1e-4);
 }
 
-cudaError_t ensure_work(crn_grid* g, int m) {
+// st: the stream of the call, which also sets the kernels' counters up (a host copy
+// on another stream could still be under way when the first kernel reads them)
+cudaError_t ensure_work(crn_grid* g, int m, cudaStream_t st) {
   NkWork* w = g->nk;
   const int64_t N = g->shape.ncell, n = 9 * N;
   if (w && w->m >= m) return cudaSuccess;
@@ -979,8 +986,8 @@ cudaError_t ensure_work(crn_grid* g, int m) {
   if (e == cudaSuccess) e = cudaMallocHost(&w->host, sizeof(double) * w->rows);
   if (e == cudaSuccess) e = cudaMalloc(&w->sync, 3 * sizeof(unsigned int));
   if (e == cudaSuccess) {
-    const unsigned int init[3] = {0u, 0x7f800000u, 0x7f800000u};
-    e = cudaMemcpy(w->sync, init, sizeof(init), cudaMemcpyHostToDevice);
+    sync_init_kernel<<<1, 1, 0, st>>>(w->sync);
+    e = cudaGetLastError();
   }
   if (e != cudaSuccess) { nk_free(w); g->nk = nullptr; }
   return e;
@@ -1332,7 +1339,7 @@ double default_b(const crn_grid* g, bool central) {
 int nk_step(crn_grid* g, double* U, double cfl, const crn_nk_options& o, crn_nk_stats* out,
             cudaStream_t st, int& launches, double stop_below, bool& stopped) {
   stopped = false;
-  cudaError_t e = ensure_work(g, o.krylov_dim);
+  cudaError_t e = ensure_work(g, o.krylov_dim, st);
   if (e == cudaSuccess && use_basis32(o)) e = ensure_basis32(g->nk);
   if (e == cudaSuccess && o.fd_central != 0) e = ensure_central(g);
   if (e != cudaSuccess) return report(CRN_E_CUDA, std::string("Newton-Krylov workspace: ") + cudaGetErrorString(e));
@@ -1619,7 +1626,7 @@ int adjoint_fgmres(Ctx& c, const double* U, const double* gbar, double* lam, dou
 // passes.
 int adjoint_pseudo_time(crn_grid* g, const double* U, const double* gbar, double* lambda, double* sens,
                         const crn_nk_options& o, crn_nk_stats* out, cudaStream_t st, int& launches) {
-  cudaError_t e = ensure_work(g, o.krylov_dim);
+  cudaError_t e = ensure_work(g, o.krylov_dim, st);
   if (e == cudaSuccess) e = vjp_ensure_scratch(g);
   if (e == cudaSuccess && !g->nk->adj) e = cudaMalloc(&g->nk->adj, sizeof(double) * 2 * g->nk->n);
   if (e != cudaSuccess) return report(CRN_E_CUDA, std::string("adjoint workspace: ") + cudaGetErrorString(e));
@@ -1720,7 +1727,7 @@ int adjoint_pseudo_time(crn_grid* g, const double* U, const double* gbar, double
 int adjoint_solve(crn_grid* g, const double* U, const double* gbar, double* lambda, double* sens,
                   const crn_nk_options& o, crn_nk_stats* out, cudaStream_t st, int& launches) {
   if (o.adjoint_cfl > 0.0) return adjoint_pseudo_time(g, U, gbar, lambda, sens, o, out, st, launches);
-  cudaError_t e = ensure_work(g, o.krylov_dim);
+  cudaError_t e = ensure_work(g, o.krylov_dim, st);
   if (e == cudaSuccess) e = vjp_ensure_scratch(g);
   if (e != cudaSuccess) return report(CRN_E_CUDA, std::string("adjoint workspace: ") + cudaGetErrorString(e));
   Ctx c(g, st);
