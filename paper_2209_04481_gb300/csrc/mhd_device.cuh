@@ -88,21 +88,25 @@ __device__ __forceinline__ float product(float a, float b) { return a * b; }
 // their FP64 operations are counted: both start from the approximate PTX
 // instructions (about 20 bits, not on the FP64 pipe) and take one cubic step.
 //   1/x: y0 (1 + e + e^2) with e = 1 - x y0 (Newton's series cut after e^2:
-//        error e^3 ~ 2^-60), 3 operations, within one unit in the last place;
-//        x finite and nonzero.
+//        error e^3 ~ 2^-60), 3 operations, within one unit in the last place.
+//        Where y0 is 0, infinite or NaN it is the result (1/0, 1/inf; on the
+//        integer pipe): the step would make it NaN.
 //   sqrt x: Goldschmidt's step on g = x y0 and h = y0 / 2 (y0 ~ 1 / sqrt x), then
 //        Newton's with the exact remainder x - g^2: 6 operations (h halves an
 //        exponent), correctly rounded but for values next to a rounding
 //        boundary.  In particular the square root of a rounded square is its
 //        base: with it a face state of negative pressure and B_n = 0 keeps c_f = 0
 //        where a last place less would make q + sqrt(q^2) negative.  0 below
-//        the normal range, NaN for x < 0.
+//        the normal range, +inf for +inf (an overflowing speed has to stay the
+//        larger one), NaN for x < 0.
 template <class T> __device__ __forceinline__ T frcp(T x);
 template <> __device__ __forceinline__ double frcp<double>(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+  const double r = fma(y, fma(e, e, e), y);
+  const unsigned ey = (unsigned)__double2hiint(y) & 0x7ff00000u;
+  return ey - 0x00100000u < 0x7fe00000u ? r : y;
 }
 template <> __device__ __forceinline__ float frcp<float>(float x) { return __fdividef(1.0f, x); }
 template <class T> __device__ __forceinline__ T fsqrt(T x);
@@ -114,7 +118,8 @@ template <> __device__ __forceinline__ double fsqrt<double>(double x) {
   const double e = fma(-h, g, 0.5);
   const double g1 = fma(g, e, g);
   const double r = fma(fma(-g1, g1, x), fma(h, e, h), g1);
-  return (__double2hiint(x) & 0x7ff00000) == 0 ? 0.0 : r;
+  const int hx = __double2hiint(x);
+  return (hx & 0x7ff00000) == 0 ? 0.0 : hx == 0x7ff00000 ? x : r;
 }
 template <> __device__ __forceinline__ float fsqrt<float>(float x) { return sqrtf(x); }
 
