@@ -438,26 +438,40 @@ scale_cells_kernel(const TV* __restrict__ v, const double* __restrict__ dtau, in
 // last term within p / 4.  eps and 1 / eps go to eps_out[0] and [1] (1 if z = 0).
 // The step needs the ratios' magnitude only: they are formed in FP32 wherever
 // the entries fit (a conversion on the integer pipe and an FP32 reciprocal in
-// place of two slots of the FP64 pipe), the pressures in FP64.  The minima are
-// combined by integer minima of their bit patterns, and the last block forms
-// eps: 38 us on 96 x 48 x 96, where FP64 ratios, nine divisions per thread for
+// place of two slots of the FP64 pipe), the pressures in FP64; the ratios of
+// entries that do not (a time step of 1e60 makes such directions) stay FP64, in
+// minima of their own.  The minima are combined by integer minima of their bit
+// patterns, and the last block forms eps: 38 us on 96 x 48 x 96, where FP64 ratios, nine divisions per thread for
 // the floors and two more kernels for the minima and eps took 134 + 8 us.
-struct StepMin {
-  unsigned int* bits;      // [2] minima as FP32 bit patterns (0x7f800000 between launches)
-  unsigned int* counter;
+// words the kernels of one grid share: minima of the entry and the pressure
+// ratios as bit patterns (+inf between launches), FP32 and FP64, and the
+// arrival counter of last_block (0 between launches)
+struct NkSync {
+  unsigned long long wide[2];
+  unsigned int bits[2];
+  unsigned int counter;
+  __device__ void clear_minima() {
+    bits[0] = bits[1] = 0x7f800000u;
+    wide[0] = wide[1] = 0x7ff0000000000000ull;
+  }
 };
-// the counter and the minima before the first launch
-__global__ void sync_init_kernel(unsigned int* sync) {
-  sync[0] = 0u;
-  sync[1] = sync[2] = 0x7f800000u;
+__global__ void sync_init_kernel(NkSync* sync) {
+  sync->clear_minima();
+  sync->counter = 0u;
+}
+// the smaller of the two minima q
+__device__ __forceinline__ double step_minimum(const NkSync* sync, int q) {
+  return fmin((double)__uint_as_float(__ldcg(sync->bits + q)), __longlong_as_double((long long)__ldcg(sync->wide + q)));
 }
 constexpr int NKE = 128;  // threads per block: long threads, and a small shell has few cells
 template <class TV>
 __global__ void __launch_bounds__(NKE)
 direction_kernel(const TV* __restrict__ v, const double* __restrict__ dtau, int64_t N, double* __restrict__ z,
                  const double* __restrict__ U, const double* __restrict__ floors, double gm1, double b,
-                 StepMin sm, double* __restrict__ eps_out) {
+                 NkSync* __restrict__ sync, double* __restrict__ eps_out) {
   float m = INFINITY, mp = INFINITY;
+  double md = INFINITY, mpd = INFINITY;  // the same where FP32 does not hold the ratio's terms
+  bool wide = false;                     // any of those
   float fl[NV];
 #pragma unroll
   for (int q = 0; q < NV; ++q) fl[q] = narrow_f64(floors[q]);
@@ -483,12 +497,12 @@ direction_kernel(const TV* __restrict__ v, const double* __restrict__ dtau, int6
       zf[q] = narrow_f64(zz[q]);
       uf[q] = narrow_f64(u[q]);
       const float az = fabsf(zf[q]), au = fabsf(uf[q]) + fl[q];
-      float r;
       if (az > 1e-30f && az < 1e30f && au > 1e-30f && au < 1e30f)
-        r = __fdividef(au, az);
-      else  // zero, or beyond the range of FP32 arithmetic
-        r = zz[q] != 0.0 ? narrow_f64((fabs(u[q]) + floors[q]) * rcp_coarse(fabs(zz[q]))) : INFINITY;
-      m = fminf(m, r);
+        m = fminf(m, __fdividef(au, az));
+      else if (zz[q] != 0.0) {  // beyond the range of FP32 arithmetic
+        md = fmin(md, (fabs(u[q]) + floors[q]) * rcp_coarse(fabs(zz[q])));
+        wide = true;
+      }
     }
     const double ir = rcp_coarse(u[0]);
     const double vx = u[1] * ir, vy = u[2] * ir, vz = u[3] * ir;
@@ -502,8 +516,10 @@ direction_kernel(const TV* __restrict__ v, const double* __restrict__ dtau, int6
     const float pf = narrow_f64(pe), df = fabsf(narrow_f64(dpe));
     if (df > 1e-30f && df < 1e30f && fabsf(pf) > 1e-30f && fabsf(pf) < 1e30f)
       mp = fminf(mp, __fdividef(pf, df));
-    else if (dpe != 0.0)
-      mp = fminf(mp, narrow_f64(pe * rcp_coarse(fabs(dpe))));
+    else if (dpe != 0.0) {
+      mpd = fmin(mpd, pe * rcp_coarse(fabs(dpe)));
+      wide = true;
+    }
     const float rf = uf[0], fx = narrow_f64(vx), fy = narrow_f64(vy), fz = narrow_f64(vz);
     const float wx = zf[1] - fx * zf[0], wy = zf[2] - fy * zf[0], wz = zf[3] - fz * zf[0];
     const float Q = 0.5f * (zf[4] * zf[4] + zf[5] * zf[5] + zf[6] * zf[6]) +
@@ -514,7 +530,10 @@ direction_kernel(const TV* __restrict__ v, const double* __restrict__ dtau, int6
       const double dx = zz[1] - vx * zz[0], dy = zz[2] - vy * zz[0], dz = zz[3] - vz * zz[0];
       const double Qd = 0.5 * (zz[4] * zz[4] + zz[5] * zz[5] + zz[6] * zz[6]) +
                         0.5 * (dx * dx + dy * dy + dz * dz) * ir;
-      if (Qd > 0.0) mp = fminf(mp, narrow_f64(2.0 * sqrt(pe * rcp_coarse(Qd))));
+      if (Qd > 0.0) {
+        mpd = fmin(mpd, 2.0 * sqrt(pe * rcp_coarse(Qd)));
+        wide = true;
+      }
     }
   }
   // a negative pressure gives a negative ratio: it orders below every other
@@ -524,17 +543,21 @@ direction_kernel(const TV* __restrict__ v, const double* __restrict__ dtau, int6
   const unsigned bm = __reduce_min_sync(0xffffffffu, __float_as_uint(m));
   const unsigned bp = __reduce_min_sync(0xffffffffu, __float_as_uint(mp));
   if ((threadIdx.x & 31) == 0) {
-    atomicMin(sm.bits, bm);
-    atomicMin(sm.bits + 1, bp);
+    atomicMin(sync->bits, bm);
+    atomicMin(sync->bits + 1, bp);
   }
-  if (!last_block(sm.counter)) return;
+  if (wide) {
+    atomicMin(sync->wide, (unsigned long long)__double_as_longlong(fmax(md, 0.0)));
+    atomicMin(sync->wide + 1, (unsigned long long)__double_as_longlong(fmax(mpd, 0.0)));
+  }
+  if (!last_block(&sync->counter)) return;
   if (threadIdx.x == 0) {
-    const double me = b * (double)__uint_as_float(__ldcg(sm.bits));
-    const double e = fmin(me, 0.25 * (double)__uint_as_float(__ldcg(sm.bits + 1)));
+    const double me = b * step_minimum(sync, 0);
+    const double e = fmin(me, 0.25 * step_minimum(sync, 1));
     const double eps = isfinite(e) && e > 0.0 ? e : (isfinite(me) && me > 0.0 ? me : 1.0);
     eps_out[0] = eps;
     eps_out[1] = 1.0 / eps;
-    sm.bits[0] = sm.bits[1] = 0x7f800000u;
+    sync->clear_minima();
   }
 }
 
@@ -898,7 +921,7 @@ struct NkWork {
   double* out = nullptr;   // rows reduced values
   double* coef = nullptr;  // m + 2 coefficients
   double* host = nullptr;  // pinned mirror of out
-  unsigned int* sync = nullptr;  // arrival counter, then the two minima of direction_kernel
+  NkSync* sync = nullptr;  // arrival counter and the minima of direction_kernel
   double* adj = nullptr;   // 2n: the pseudo-time adjoint's lambda and residual (first use)
   double* fv = nullptr;    // (mf + 1) n: outer FGMRES basis of the pseudo-time adjoint
   double* fz = nullptr;    // mf n: its preconditioned directions
@@ -984,7 +1007,7 @@ cudaError_t ensure_work(crn_grid* g, int m, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaMalloc(&w->out, sizeof(double) * w->rows);
   if (e == cudaSuccess) e = cudaMalloc(&w->coef, sizeof(double) * (m + 2));
   if (e == cudaSuccess) e = cudaMallocHost(&w->host, sizeof(double) * w->rows);
-  if (e == cudaSuccess) e = cudaMalloc(&w->sync, 3 * sizeof(unsigned int));
+  if (e == cudaSuccess) e = cudaMalloc(&w->sync, sizeof(NkSync));
   if (e == cudaSuccess) {
     sync_init_kernel<<<1, 1, 0, st>>>(w->sync);
     e = cudaGetLastError();
@@ -1023,7 +1046,7 @@ struct Ctx {
     if (err == cudaSuccess) err = cudaStreamSynchronize(st);
   }
   GsOut gs() const {
-    return GsOut{w->out, w->out + rows.ww, w->out + rows.after, w->out + rows.inv, w->coef, w->out + rows.redo, w->sync};
+    return GsOut{w->out, w->out + rows.ww, w->out + rows.after, w->out + rows.inv, w->coef, w->out + rows.redo, &w->sync->counter};
   }
   // blocks of the Gram-Schmidt kernels: one per SM, fewer for a short vector
   unsigned gs_blocks(int per) const {
@@ -1167,15 +1190,14 @@ struct Ctx {
   // w_out = v - J (dtau . v), J by a forward or central difference
   template <class TV>
   void apply_op(const TV* v, TV* wout, const double* U, double b_rel, bool central) {
-    const StepMin sm{w->sync + 1, w->sync};
     double* e = w->out + rows.eps;
     const double gm1 = g->d.gamma - 1.0;
     const unsigned nb = (unsigned)std::min<int64_t>((N + NKE - 1) / NKE, 8 * (int64_t)g->cfg.num_sms);
     if (precond == 1) {
       line_solve(v, w->z);
-      direction_kernel<double><<<nb, NKE, 0, st>>>(w->z, nullptr, N, w->z, U, w->out + rows.floors, gm1, b_rel, sm, e);
+      direction_kernel<double><<<nb, NKE, 0, st>>>(w->z, nullptr, N, w->z, U, w->out + rows.floors, gm1, b_rel, w->sync, e);
     } else {
-      direction_kernel<TV><<<nb, NKE, 0, st>>>(v, w->dtau, N, w->z, U, w->out + rows.floors, gm1, b_rel, sm, e);
+      direction_kernel<TV><<<nb, NKE, 0, st>>>(v, w->dtau, N, w->z, U, w->out + rows.floors, gm1, b_rel, w->sync, e);
     }
     ++launches;
     if (g->d.precision == CRN_FP64)
@@ -1371,7 +1393,7 @@ int nk_step(crn_grid* g, double* U, double cfl, const crn_nk_options& o, crn_nk_
     c.line_factor();
   }
   floors_kernel<<<(unsigned)std::min<int64_t>((c.N + NKB - 1) / NKB, w->nblk), NKB, 0, st>>>(
-      U, c.N, w->part, w->out, c.rows.floors, w->sync);
+      U, c.N, w->part, w->out, c.rows.floors, &w->sync->counter);
   ++c.launches;
   const bool outer64 = g->d.precision == CRN_FP32_BULK && o.outer_fp64 != 0;
   if (outer64) {  // the FP64 tiled kernels' shared-memory opt-in (an FP32-bulk grid skips it)

@@ -1,9 +1,12 @@
 """The Newton-Krylov workspace and its finite-difference step at the ends of
-their ranges: the first step of a grid on a stream of its own."""
+their ranges: the first step of a grid on a stream of its own, and directions
+beyond the range of FP32."""
+import numpy as np
 import pytest
 
 import coronal_inputs as ci
-from _util import problem
+import oracle
+from _util import oracle_grid, problem
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -32,3 +35,24 @@ def test_first_step_on_a_side_stream(precision):
         out.append((U64, st))
         g.close()
     assert torch.equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
+
+
+@pytest.mark.parametrize("cfl", [1e42, 1e60, 1e-60])
+@pytest.mark.parametrize("m", [2, 5])
+def test_directions_beyond_fp32(cfl, m):
+    """z = dtau . v with entries far outside FP32 (precond 0, FP64 basis): the
+    linear residual reported is the true one of the step returned."""
+    shape = (5, 7, 16)
+    g, U, Br = make(shape)
+    U64 = torch.from_numpy(U.copy()).cuda()
+    dU = torch.zeros_like(U64)
+    st = g.newton_krylov_step(U64, cfl, dU=dU, krylov_dim=m, lin_rtol=1e-12, basis_fp32=0, precond=0)
+    og = oracle_grid(shape, inner_bc="low_e_wp", vr_star=VR)
+    x = dU.cpu().numpy()
+    R = oracle.residual(og, U, Br)["R"]
+    _, Jx = oracle.residual_jvp(og, U, Br, x, np.zeros_like(Br))
+    r = R - x / (cfl * oracle.local_dt(og, U))[None] + Jx
+    rel = np.linalg.norm(r) / np.linalg.norm(R)
+    # the bar of the steps at ordinary directions: 1e-5 per finite-difference product
+    assert abs(rel - st["lin_rel"]) <= 1e-5 * np.sqrt(m) + 1e-3 * st["lin_rel"], (rel, st)
+    g.close()
