@@ -906,9 +906,8 @@ struct NkWork {
   double* z = nullptr;     // n: preconditioned direction, then dU
   double* x = nullptr;     // n: GMRES solution y
   double* b = nullptr;     // n: R(U) in FP64
-  double* w = nullptr;     // n: Arnoldi vector
+  double* w = nullptr;     // n: residual vectors; during a product with J, U - eps z of a central difference
   void* ut = nullptr;      // n of T: cast state / U + eps z
-  void* um = nullptr;      // n of T: U - eps z (allocated by the first central difference)
   void* rt = nullptr;      // n of T: perturbed residual
   void* rb = nullptr;      // n of T: base residual (FP32 grids) / R(U - eps z) (FP64 grids)
   void* rm = nullptr;      // n of T: R(U - eps z) (FP32 grids)
@@ -933,7 +932,7 @@ void nk_free(NkWork* w) {
   cudaFree(w->V); cudaFree(w->z); cudaFree(w->x); cudaFree(w->b); cudaFree(w->w);
   cudaFree(w->ut); cudaFree(w->rt); cudaFree(w->rb); cudaFree(w->rm); cudaFree(w->dtau);
   cudaFree(w->line);
-  cudaFree(w->Vf); cudaFree(w->um); cudaFree(w->sync);
+  cudaFree(w->Vf); cudaFree(w->sync);
   cudaFree(w->part); cudaFree(w->out); cudaFree(w->coef);
   cudaFree(w->adj);
   cudaFree(w->fv); cudaFree(w->fz);
@@ -965,13 +964,6 @@ int report(int code, const std::string& msg) { return report_error(code, msg.c_s
 cudaError_t ensure_basis32(NkWork* w) {
   if (w->Vf) return cudaSuccess;
   return cudaMalloc(&w->Vf, sizeof(float) * (size_t)(w->m + 1) * w->n);
-}
-
-// the second perturbed state of a central difference (allocated on first use)
-cudaError_t ensure_central(crn_grid* g) {
-  NkWork* w = g->nk;
-  if (w->um) return cudaSuccess;
-  return cudaMalloc(&w->um, (size_t)(g->d.precision == CRN_FP64 ? 8 : 4) * w->n);
 }
 
 bool use_basis32(const crn_nk_options& o) {
@@ -1206,13 +1198,15 @@ struct Ctx {
       difference<float>(v, wout, U, central, w->rb, w->rm);
   }
   // the finite difference along z: base R(U) for the forward one, the second
-  // residual in `other` for the central one
+  // residual in `other` for the central one, whose second state lies in w->w:
+  // nothing reads that vector before the product is written (wout may be it)
   template <class T, class TV>
   void difference(const TV* v, TV* wout, const double* U, bool central, const void* base, void* other) {
     const double* e = w->out + rows.eps;
-    perturb_kernel<T><<<grid, NKB, 0, st>>>(U, w->z, e, n, (T*)w->ut, central ? (T*)w->um : nullptr);
+    T* um = central ? reinterpret_cast<T*>(w->w) : nullptr;
+    perturb_kernel<T><<<grid, NKB, 0, st>>>(U, w->z, e, n, (T*)w->ut, um);
     if (central)
-      residual_pair(w->ut, w->rt, w->um, other);
+      residual_pair(w->ut, w->rt, um, other);
     else
       residual(w->ut, w->rt);
     jvp_combine_kernel<T, TV, TV><<<cells(), NKB, 0, st>>>(v, (const T*)w->rt, (const T*)(central ? other : base), e + 1,
@@ -1363,7 +1357,6 @@ int nk_step(crn_grid* g, double* U, double cfl, const crn_nk_options& o, crn_nk_
   stopped = false;
   cudaError_t e = ensure_work(g, o.krylov_dim, st);
   if (e == cudaSuccess && use_basis32(o)) e = ensure_basis32(g->nk);
-  if (e == cudaSuccess && o.fd_central != 0) e = ensure_central(g);
   if (e != cudaSuccess) return report(CRN_E_CUDA, std::string("Newton-Krylov workspace: ") + cudaGetErrorString(e));
   Ctx c(g, st);
   c.precond = o.precond;

@@ -1,6 +1,6 @@
 """The Newton-Krylov workspace and its finite-difference step at the ends of
-their ranges: the first step of a grid on a stream of its own, and directions
-beyond the range of FP32."""
+their ranges: the first step of a grid on a stream of its own, directions
+beyond the range of FP32, and the memory a central difference takes."""
 import numpy as np
 import pytest
 
@@ -56,3 +56,19 @@ def test_directions_beyond_fp32(cfl, m):
     # the bar of the steps at ordinary directions: 1e-5 per finite-difference product
     assert abs(rel - st["lin_rel"]) <= 1e-5 * np.sqrt(m) + 1e-3 * st["lin_rel"], (rel, st)
     g.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_central_difference_takes_no_memory_of_its_own(precision):
+    """9.4 (4.7) MB of a second perturbed state on 64 x 32 x 64 would show."""
+    used = {}
+    for central in (0, 1):
+        g, U, _ = make((64, 32, 64), precision)
+        U64 = torch.from_numpy(U.copy()).cuda()
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        g.newton_krylov_step(U64, 1.0, krylov_dim=2, fd_central=central)
+        torch.cuda.synchronize()
+        used[central] = before - torch.cuda.mem_get_info()[0]
+        g.close()
+    assert used[0] > 0 and used[1] <= used[0]
