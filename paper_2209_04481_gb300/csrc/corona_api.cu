@@ -374,8 +374,12 @@ int crn_grid_create(const crn_grid_desc* d, crn_grid** out) {
         tiled_blocks = std::max<int64_t>(tiled_blocks, st * ((d->n_r + kcs - 1) / kcs));
       }
     }
-    const int64_t cell_blocks = (g->shape.ncell + 255) / 256;
-    g->max_blocks = (size_t)std::max<int64_t>(std::max<int64_t>(tiled_blocks, cell_blocks), 4 * 152 * 8);
+    // one partial per work item: the launches above, the cell-wise kernel's, and in
+    // an ensemble any chunk the caller sets, which the own tile's columns cut into
+    // (FP64: half the columns of FP32, twice the items of a chunk)
+    const int64_t cell_blocks = (g->shape.ncell + tt * tp - 1) / (tt * tp);
+    const int64_t least = 4 * 152 * 8 * (256 / (tt * tp));
+    g->max_blocks = (size_t)std::max<int64_t>(std::max<int64_t>(tiled_blocks, cell_blocks), least);
   }
   rc = upload_geometry(h, g->g64);
   if (rc == CRN_OK) rc = upload_geometry(h, g->g32);

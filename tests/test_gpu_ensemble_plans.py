@@ -1,0 +1,46 @@
+"""The ensemble's chunks and tiles where the defaults and the launches' limits
+meet: the shortest chunks of large members."""
+import pytest
+
+import coronal_inputs as ci
+from _util import problem
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def make(shapes, precision):
+    import paper_2209_04481_gb300 as pg
+    gs, Us, cache = [], [], {}
+    for shape in shapes:
+        if shape not in cache:
+            U, Br = problem(shape, perturb=3)
+            cache[shape] = torch.from_numpy(U), torch.from_numpy(Br).cuda()
+        U, Br = cache[shape]
+        g = pg.Grid(*shape, precision=precision, p_b=ci.parker_sound_speed2())
+        g.set_inner_boundary(Br)
+        gs.append(g)
+        Us.append(U.to("cuda", g.dtype))
+    return gs, Us, pg.Ensemble(gs)
+
+
+def close(gs, ens):
+    gs[0].sync_status()
+    ens.close()
+    for g in gs:
+        g.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("kchunk", [1, 2])
+def test_shortest_chunks(precision, kchunk):
+    gs, Us, ens = make([(80, 64, 128), (5, 8, 16)], precision)
+    norms = torch.zeros((2, 9), dtype=torch.float64, device="cuda")
+    ens.kchunk = kchunk
+    Rs = ens.residual(Us, norms=norms)
+    for g, U, R in zip(gs, Us, Rs):
+        assert torch.equal(R, g.residual(U))
+    ref = torch.stack([torch.linalg.vector_norm(R.double().reshape(9, -1), dim=1) for R in Rs])
+    # FP32 sums of at most 2 squares a thread and a 5-level tree; FP64 elsewhere
+    torch.testing.assert_close(norms, ref, rtol=1e-6 if precision == "fp32" else 1e-12, atol=0)
+    close(gs, ens)
