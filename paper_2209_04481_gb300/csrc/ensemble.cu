@@ -93,7 +93,9 @@ int member_chunk(const crn_ensemble* e, int m) {
 // with the shortest makespan wins.  Eight FP32 shells of 4.9 M cells:
 // 310 us, the best single chunk for all 346 us; when the kernel was slower 362 us
 // against 419 us with the own chunks of 2 to 26 planes.  Ensembles of fewer than four
-// (tile, plane) pairs per CTA keep the members' own chunks.
+// (tile, plane) pairs per CTA keep the members' own chunks; where even whole columns
+// of the tallest member leave eight items per CTA and more, every member is taken
+// whole: the items are many, and no preamble is paid twice.
 void plan_chunks(crn_ensemble* e) {
   const bool fp64 = e->precision == CRN_FP64;
   const int t = crn::own_tile(fp64), n = (int)e->g.size();
@@ -109,8 +111,8 @@ void plan_chunks(crn_ensemble* e) {
   }
   if (planes < 4 * slots) return;
   const double pre = fp64 ? 0.5 : 1.5;
-  const int k_lo = (int)std::max<long long>(1, planes / (8 * slots));
   const int k_hi = (int)std::min<long long>(nr_max, planes / slots + 1);
+  const int k_lo = (int)std::max<long long>(1, std::min<long long>(k_hi, planes / (8 * slots)));
   double best = 0.0;
   std::vector<int> kc(n), order(n);
   std::vector<double> heap;
@@ -120,6 +122,10 @@ void plan_chunks(crn_ensemble* e) {
       const int parts = std::max(1, (2 * nr + k) / (2 * k));
       kc[m] = (nr + parts - 1) / parts;
       order[m] = m;
+    }
+    if (k_lo == k_hi) {  // nothing to compare
+      e->plan = kc;
+      return;
     }
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return kc[a] > kc[b]; });
     heap.assign((size_t)slots, 0.0);

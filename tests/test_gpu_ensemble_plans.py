@@ -1,5 +1,6 @@
-"""The ensemble's chunks and tiles where the defaults and the launches' limits
-meet: the shortest chunks of large members."""
+"""The ensemble's chunks, tiles and tuner where the defaults and the launches'
+limits meet: the shortest chunks of large members, and more members than the
+longest chunk can balance."""
 import pytest
 
 import coronal_inputs as ci
@@ -43,4 +44,17 @@ def test_shortest_chunks(precision, kchunk):
     ref = torch.stack([torch.linalg.vector_norm(R.double().reshape(9, -1), dim=1) for R in Rs])
     # FP32 sums of at most 2 squares a thread and a 5-level tree; FP64 elsewhere
     torch.testing.assert_close(norms, ref, rtol=1e-6 if precision == "fp32" else 1e-12, atol=0)
+    close(gs, ens)
+
+
+@pytest.mark.parametrize("precision,n", [("fp32", 100), ("fp64", 50)])
+def test_more_members_than_chunks_can_balance(precision, n):
+    """Many flat shells: more (tile, plane) pairs than eight items per CTA of the
+    tallest member's full height.  Every member is taken whole."""
+    shapes = [(8, 64, 128) if m % 3 else (5, 64, 128) for m in range(n)]
+    gs, Us, ens = make(shapes, precision)
+    assert [ens.member_config(m)[1] for m in range(n)] == [s[0] for s in shapes]
+    Rs = ens.residual(Us)
+    for m in (0, 1, n - 1):
+        assert torch.equal(Rs[m], gs[m].residual(Us[m])), m
     close(gs, ens)
