@@ -524,8 +524,11 @@ class Ensemble:
         _check(_lib.crn_ensemble_member_config(self._h, int(m), ctypes.byref(t), ctypes.byref(k)))
         return self.TILES[t.value], k.value
 
-    def set_member_config(self, m, tile=(8, 32), kchunk=0):
-        """Tile shape ((8, 32), (16, 16) or, in FP64, (8, 16)) and radial chunk (0: the member's own) of member m."""
+    def set_member_config(self, m, tile=None, kchunk=0):
+        """Tile shape ((8, 32), (16, 16) or, in FP64, (8, 16); None: that of the
+        member's own launch) and radial chunk (0: the default) of member m."""
+        if tile is None:
+            tile = (8, 16) if self.grids[0].desc.precision == FP64 else (8, 32)
         code = {v: c for c, v in self.TILES.items()}[tuple(tile)]
         _check(_lib.crn_ensemble_set_member_config(self._h, int(m), code, int(kchunk)))
 

@@ -1,6 +1,6 @@
 """The ensemble's chunks, tiles and tuner where the defaults and the launches'
-limits meet: the shortest chunks of large members, and more members than the
-longest chunk can balance."""
+limits meet: the shortest chunks of large members, more members than the
+longest chunk can balance, and a chunk set without a tile."""
 import pytest
 
 import coronal_inputs as ci
@@ -57,4 +57,17 @@ def test_more_members_than_chunks_can_balance(precision, n):
     Rs = ens.residual(Us)
     for m in (0, 1, n - 1):
         assert torch.equal(Rs[m], gs[m].residual(Us[m])), m
+    close(gs, ens)
+
+
+@pytest.mark.parametrize("precision,own", [("fp64", (8, 16)), ("fp32", (8, 32))])
+def test_chunk_without_a_tile_keeps_the_own_tile(precision, own):
+    gs, Us, ens = make([(12, 8, 32), (9, 24, 64)], precision)
+    assert ens.member_config(0)[0] == own
+    ens.set_member_config(0, kchunk=3)
+    assert ens.member_config(0) == (own, 3)
+    ens.set_member_config(0, tile=(16, 16), kchunk=5)
+    assert ens.member_config(0) == ((16, 16), 5)
+    ens.set_member_config(0)
+    assert ens.member_config(0)[0] == own
     close(gs, ens)
