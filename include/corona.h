@@ -412,13 +412,17 @@ int crn_ensemble_pseudo_time_step(crn_ensemble* e, double* const* U64_dev, int32
 /* Tile autotuner.  Members are grouped in size classes (equal n_theta and
  * n_phi).  For each class it times the persistent launch over that class's
  * members alone (one warm-up, three timed launches, CUDA events) for each tile
- * shape (8 x 32 and 16 x 16 (theta, phi) columns per CTA) and each radial chunk
- * (the members' own, 4, 6, 8, 12, 16, 24, 32, 48 planes per item), and keeps
- * the fastest pair for the class's members (crn_ensemble_member_config reads
- * it back).  *kchunk_out receives the chunk chosen for the class with the most
- * cells.  R is the same for every tile shape and chunk up to rounding (the
- * first r face of a chunk is evaluated on the CTA's preamble path).
- * Synchronises `stream`; R_dev is overwritten. */
+ * shape (8 x 32 and 16 x 16 (theta, phi) columns per CTA; for FP64 members that
+ * together fill the GPU also their own 8 x 16) and each radial chunk (the
+ * default of crn_ensemble_set_kchunk, 4, 6, 8, 12, 16, 24, 32, 48 planes per
+ * item), and keeps the fastest pair for the class's members
+ * (crn_ensemble_member_config reads it back).  Then it times the whole ensemble
+ * with these choices and with the defaults, and returns to the defaults unless
+ * the choices beat them by 2 % (FP64 members that do not fill the GPU keep the
+ * choices).  *kchunk_out receives the chunk chosen for the class with the most
+ * cells, 0 with the defaults.  R is the same for every tile shape and chunk up
+ * to rounding (the first r face of a chunk is evaluated on the CTA's preamble
+ * path).  Synchronises `stream`; R_dev is overwritten. */
 int crn_ensemble_autotune(crn_ensemble* e, const void* const* U_dev, void* const* R_dev, void* stream,
                           int32_t* kchunk_out);
 

@@ -559,7 +559,8 @@ class Ensemble:
         return U64s
 
     def autotune(self, Us, Rs, stream=None):
-        """Time the candidate radial chunks and keep the fastest; returns it."""
+        """Time the candidate tiles and radial chunks and keep the fastest, the
+        defaults unless they are beaten; returns the chunk (0: the defaults)."""
         self._check_states(Us, "U")
         self._check_states(Rs, "R")
         k = ctypes.c_int32()

@@ -414,8 +414,32 @@ int crn_ensemble_autotune(crn_ensemble* e, const void* const* U_dev, void* const
   cudaEvent_t a, b;
   cudaEventCreate(&a);
   cudaEventCreate(&b);
+  auto done = [&](int code, const std::string& msg) {
+    cudaEventDestroy(a);
+    cudaEventDestroy(b);
+    return report(code, msg);
+  };
   int launches = 0, big_class = 0;
   int64_t big_cells = -1;
+  // three launches of the current configuration after one to warm up, of all
+  // members or those in `sub`; ms stays as it is if a chunk overflows a member's scratch
+  auto time_launches = [&](const std::vector<int>* sub, float& ms) {
+    ++e->cfg_version;
+    if (residual_records(e, U_dev, R_dev, nullptr, nullptr, st, sub) != CRN_OK) return cudaSuccess;
+    int nl = 0;
+    cudaError_t err = launch(e, st, &nl);
+    if (err == cudaSuccess) err = cudaEventRecord(a, st);
+    for (int r = 0; r < 3 && err == cudaSuccess; ++r) err = launch(e, st, &nl);
+    if (err == cudaSuccess) err = cudaEventRecord(b, st);
+    if (err == cudaSuccess) err = cudaEventSynchronize(b);
+    if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, a, b);
+    launches += nl;
+    return err;
+  };
+  const int own = crn::own_tile(e->precision == CRN_FP64);
+  // Tile shapes 0 and 1, and the own shape of FP64 members (2) where the members
+  // together fill the GPU; a smaller FP64 ensemble chooses between the two.
+  const bool with_own = own < 2 || !e->plan.empty();
   std::vector<int> best_k(classes.size(), 0);
   for (size_t c = 0; c < classes.size(); ++c) {
     const std::vector<int>& mem = classes[c];
@@ -428,43 +452,56 @@ int crn_ensemble_autotune(crn_ensemble* e, const void* const* U_dev, void* const
     if (cells > big_cells) { big_cells = cells; big_class = (int)c; }
     float best_ms = INFINITY;
     int best_tile = 0, bestk = 0;
-    for (int tile = 0; tile < 2; ++tile)
+    for (int tile = 0; tile < crn::kEnsTileCount; ++tile) {
+      if (tile == 2 && !(own == 2 && with_own)) continue;
       for (int k : cand) {
         if (k > 0 && k > nr_max) continue;
         for (int m : mem) { e->tile[m] = tile; e->kc[m] = k; }
-        ++e->cfg_version;
-        rc = residual_records(e, U_dev, R_dev, nullptr, nullptr, st, &mem);
-        if (rc != CRN_OK) continue;  // this chunk overflows a member's scratch
-        int nl = 0;
-        cudaError_t err = launch(e, st, &nl);  // warm-up
-        if (err == cudaSuccess) err = cudaEventRecord(a, st);
-        for (int r = 0; r < 3 && err == cudaSuccess; ++r) err = launch(e, st, &nl);
-        if (err == cudaSuccess) err = cudaEventRecord(b, st);
-        if (err == cudaSuccess) err = cudaEventSynchronize(b);
-        float ms = 0.f;
-        if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, a, b);
-        if (err != cudaSuccess) {
-          cudaEventDestroy(a);
-          cudaEventDestroy(b);
-          return report(CRN_E_CUDA, std::string("crn_ensemble_autotune: ") + cudaGetErrorString(err));
-        }
-        launches += nl;
+        float ms = INFINITY;
+        const cudaError_t err = time_launches(&mem, ms);
+        if (err != cudaSuccess)
+          return done(CRN_E_CUDA, std::string("crn_ensemble_autotune: ") + cudaGetErrorString(err));
         if (ms < best_ms) { best_ms = ms; best_tile = tile; bestk = k; }
       }
-    if (!(best_ms < INFINITY)) {
-      cudaEventDestroy(a);
-      cudaEventDestroy(b);
-      return report(CRN_E_ARG, "no radial chunk fits the reduction scratch of every member of a size class");
     }
+    if (!(best_ms < INFINITY))
+      return done(CRN_E_ARG, "no radial chunk fits the reduction scratch of every member of a size class");
     for (int m : mem) { e->tile[m] = best_tile; e->kc[m] = bestk; }
     best_k[c] = bestk;
+  }
+  e->kchunk = best_k[big_class];
+  // A class timed alone says little of it among the others, whose items fill its
+  // tail: the default (own tiles, balanced chunks, one launch) stays unless the
+  // classes' choices beat it together.  Four FP32 shells of 2.0 M cells: default
+  // 75 us, the classes' choices 89; FP64 1.44 ms and 1.57 (without shape 2).
+  if (with_own) {
+    const std::vector<int> tile = e->tile, kc = e->kc;
+    float tuned = INFINITY, plain = INFINITY;
+    for (int r = 0; r < 2; ++r) {
+      float ms = INFINITY;
+      cudaError_t err = time_launches(nullptr, ms);
+      tuned = std::min(tuned, ms);
+      e->tile.assign(n, own);
+      e->kc.assign(n, 0);
+      ms = INFINITY;
+      if (err == cudaSuccess) err = time_launches(nullptr, ms);
+      plain = std::min(plain, ms);
+      e->tile = tile;
+      e->kc = kc;
+      if (err != cudaSuccess)
+        return done(CRN_E_CUDA, std::string("crn_ensemble_autotune: ") + cudaGetErrorString(err));
+    }
+    if (!(tuned < 0.98f * plain)) {  // 2 %: what the runs of one configuration differ by
+      e->tile.assign(n, own);
+      e->kc.assign(n, 0);
+      e->kchunk = 0;
+    }
   }
   cudaEventDestroy(a);
   cudaEventDestroy(b);
   ++e->cfg_version;
   e->kSub = nullptr;
   e->kU.clear();  // the next call rebuilds the full table
-  e->kchunk = best_k[big_class];
   if (kchunk_out) *kchunk_out = e->kchunk;
   e->last_launches = launches;
   return CRN_OK;

@@ -1,6 +1,7 @@
 """The ensemble's chunks, tiles and tuner where the defaults and the launches'
-limits meet: the shortest chunks of large members, more members than the
-longest chunk can balance, and a chunk set without a tile."""
+limits meet: one-plane chunks of FP64 members, more members than the longest
+chunk can balance, a chunk set without a tile, and a tuner that leaves the
+default where the default is faster."""
 import pytest
 
 import coronal_inputs as ci
@@ -70,4 +71,36 @@ def test_chunk_without_a_tile_keeps_the_own_tile(precision, own):
     assert ens.member_config(0) == ((16, 16), 5)
     ens.set_member_config(0)
     assert ens.member_config(0)[0] == own
+    close(gs, ens)
+
+
+def _time(ens, Us, Rs):
+    for _ in range(3):
+        ens.residual(Us, Rs)
+    best = float("inf")
+    for _ in range(5):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(10):
+            ens.residual(Us, Rs)
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_tuned_is_never_slower_than_the_default(precision):
+    """Shells that fill the GPU.  3 % for the runs of one configuration."""
+    gs, Us, ens = make([(64, 32, 96), (47, 40, 80), (96, 30, 64), (60, 48, 128)], precision)
+    Rs = [torch.empty_like(U) for U in Us]
+    default = _time(ens, Us, Rs)
+    ref = [R.clone() for R in Rs]
+    k = ens.autotune(Us, Rs)
+    assert ens.kchunk == k
+    tuned = _time(ens, Us, Rs)
+    assert tuned <= 1.03 * default, (tuned, default, [ens.member_config(m) for m in range(4)])
+    tol = 1e-13 if precision == "fp64" else 1e-6
+    for a, b in zip(ref, Rs):
+        assert torch.all((a - b).abs() <= tol * a.abs().amax(dim=(1, 2, 3), keepdim=True))
     close(gs, ens)
