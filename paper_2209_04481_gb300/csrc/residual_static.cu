@@ -64,14 +64,21 @@ static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
 namespace {
 
+// the radial chunk chosen for a launch's sizes, precision and limiter
+struct Plan {
+  int32_t nr, nt, np, precision, limiter;
+  int kchunk;
+};
+constexpr int kPlans = 64;
+
 struct DeviceSlot {
   bool ready = false;
   unsigned char* base = nullptr;  // device address of g_scratch on this device
   bool geo_valid = false;
   crn_grid_desc geo_desc{};
   bool captured = false;  // a call on this device was recorded in a graph
-  crn_grid_desc plan_desc{};  // sizes, precision and limiter the radial chunk was chosen for
-  int kchunk = 0;             // (0: none yet)
+  Plan plans[kPlans];  // a simulated launch takes 1 to 2 ms of host time: kept for the last kPlans launches
+  int nplans = 0;      // ever made; the oldest gives way
 };
 
 std::mutex g_mu;
@@ -275,10 +282,11 @@ bool same_geometry(const crn_grid_desc& a, const crn_grid_desc& b) {
 // the radial chunk of a launch, as crn_grid_create chooses it
 template <class T>
 int plan(const crn_grid_desc& d, DeviceSlot& slot) {
-  const crn_grid_desc& p = slot.plan_desc;
-  if (slot.kchunk > 0 && p.n_r == d.n_r && p.n_theta == d.n_theta && p.n_phi == d.n_phi &&
-      p.precision == d.precision && p.limiter == d.limiter)
-    return slot.kchunk;
+  for (int q = 0; q < std::min(slot.nplans, kPlans); ++q) {
+    const Plan& p = slot.plans[q];
+    if (p.nr == d.n_r && p.nt == d.n_theta && p.np == d.n_phi && p.precision == d.precision && p.limiter == d.limiter)
+      return p.kchunk;
+  }
   constexpr int TT = StaticTile<T>::TT, TP = StaticTile<T>::TP;
   const int64_t ntiles = (int64_t)((d.n_theta + TT - 1) / TT) * ((d.n_phi + TP - 1) / TP);
   int nsm = 0, per_sm = 0, dev = 0;
@@ -293,8 +301,8 @@ int plan(const crn_grid_desc& d, DeviceSlot& slot) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, crn::residual_tiled<T, 2, TT, TP, crn::SUMS_ALL>, TT * TP, smem);
   int kc = crn::choose_radial_chunk(d.n_r, ntiles, std::max(nsm, 1), per_sm, sizeof(T) == 8);
   while (ntiles * ((d.n_r + kc - 1) / kc) > kMaxBlocks) kc *= 2;
-  slot.plan_desc = d;
-  slot.kchunk = kc;
+  slot.plans[slot.nplans % kPlans] = Plan{d.n_r, d.n_theta, d.n_phi, d.precision, d.limiter, kc};
+  slot.nplans = slot.nplans + 1 < 2 * kPlans ? slot.nplans + 1 : kPlans;
   return kc;
 }
 
