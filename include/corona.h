@@ -182,9 +182,12 @@ int crn_residual(crn_grid* g, const void* U_dev, void* R_dev, double* norms9_dev
  * FP32, which forms its slopes where they are used), with a scratch of about 144
  * values of the grid's type per cell (54 with FP32) allocated by the grid's
  * first VJP call: make that call before any stream capture.  An FP64 grid whose
- * scratch does not fit in device memory runs the tiled passes.  The environment variable CRN_VJP_KERNEL ("tiled" or
- * "faces"), read at each call, overrides the choice.  Ubar_dev must not
- * overlap U_dev or Rbar_dev (CRN_E_ARG).  Asynchronous. */
+ * scratch does not fit in device memory, or is larger than the environment
+ * variable CRN_VJP_SCRATCH_LIMIT (bytes), runs the tiled passes (2 launches,
+ * other rounding), and asks again at its next call outside a capture.  The
+ * environment variable CRN_VJP_KERNEL ("tiled" or "faces") overrides the choice.
+ * Both are read at each call.  Ubar_dev must not overlap U_dev or Rbar_dev
+ * (CRN_E_ARG).  Asynchronous. */
 int crn_residual_vjp(crn_grid* g, const void* U_dev, const void* Rbar_dev, void* Ubar_dev,
                      double* Brbar_dev, void* stream);
 

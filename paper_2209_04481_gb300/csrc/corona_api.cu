@@ -472,7 +472,7 @@ int crn_residual_vjp(crn_grid* g, const void* U_dev, const void* Rbar_dev, void*
       (Brbar_dev && !is_device_ptr(Brbar_dev)))
     return fail(CRN_E_ARG, "VJP arguments must be device pointers");
   {
-    const cudaError_t es = crn::vjp_ensure_scratch(g);  // first VJP call
+    const cudaError_t es = crn::vjp_ensure_scratch(g, (cudaStream_t)stream);  // first VJP call
     if (es != cudaSuccess) return cuda_fail(es, "cudaMalloc(VJP scratch)");
   }
   int nl = 0;

@@ -60,7 +60,7 @@ struct crn_grid {
   unsigned long long* err_cell = nullptr;
   void* rbuf = nullptr;            // residual scratch for pseudo-time stepping (9N of T)
   void* vjp_buf = nullptr;         // VJP slopes and face cotangents (allocated by the first VJP call)
-  bool vjp_no_room = false;        // that allocation failed: the tiled VJP, which needs none
+  bool vjp_no_room = false;        // that allocation failed last time: the tiled VJP, which needs none
   float* shadow = nullptr;         // FP32 shadow of the master state (FP32_BULK)
   crn::NkWork* nk = nullptr;       // Newton-Krylov workspace (allocated by the first NK call)
   crn::HostPipe* pipe = nullptr;   // host-buffer staging (allocated by the first host batch)
@@ -92,7 +92,7 @@ cudaError_t launch_vjp_fp64(crn_grid* g, const double* U, const double* Rb, doub
                             cudaStream_t st, int* nlaunch);
 cudaError_t launch_vjp_fp32(crn_grid* g, const float* U, const float* Rb, float* Ub, double* Brb,
                             cudaStream_t st, int* nlaunch);
-cudaError_t vjp_ensure_scratch(crn_grid* g);
+cudaError_t vjp_ensure_scratch(crn_grid* g, cudaStream_t st);
 // ensemble records (EnsMember<T> of residual.cuh, opaque here) and launches
 size_t ens_member_bytes_fp64();
 size_t ens_member_bytes_fp32();

@@ -966,6 +966,25 @@ cudaError_t ensure_basis32(NkWork* w) {
   return cudaMalloc(&w->Vf, sizeof(float) * (size_t)(w->m + 1) * w->n);
 }
 
+// the outer FGMRES basis of the pseudo-time adjoint (allocated on first use)
+cudaError_t ensure_fgmres(NkWork* w, int mf) {
+  if (w->mf >= mf) return cudaSuccess;
+  cudaFree(w->fv);
+  cudaFree(w->fz);
+  w->fv = w->fz = nullptr;
+  w->mf = 0;
+  cudaError_t e = cudaMalloc(&w->fv, sizeof(double) * (size_t)(mf + 1) * w->n);
+  if (e == cudaSuccess) e = cudaMalloc(&w->fz, sizeof(double) * (size_t)mf * w->n);
+  if (e == cudaSuccess) {
+    w->mf = mf;
+  } else {
+    cudaFree(w->fv);
+    cudaFree(w->fz);
+    w->fv = w->fz = nullptr;
+  }
+  return e;
+}
+
 bool use_basis32(const crn_nk_options& o) {
   return o.basis_fp32 == 1 || (o.basis_fp32 == -1 && o.lin_rtol >= 1e-4);
 }
@@ -1551,21 +1570,6 @@ int adjoint_fgmres(Ctx& c, const double* U, const double* gbar, double* lam, dou
     if (c.err == cudaSuccess) c.err = e;
   };
   const int mf = std::min(o.adjoint_fgmres, o.krylov_dim);
-  if (w->mf < mf) {
-    cudaFree(w->fv);
-    cudaFree(w->fz);
-    w->fv = w->fz = nullptr;
-    w->mf = 0;
-    cudaError_t e = cudaMalloc(&w->fv, sizeof(double) * (size_t)(mf + 1) * c.n);
-    if (e == cudaSuccess) e = cudaMalloc(&w->fz, sizeof(double) * (size_t)mf * c.n);
-    if (e != cudaSuccess) {
-      cudaFree(w->fv);
-      cudaFree(w->fz);
-      w->fv = w->fz = nullptr;
-      return report(CRN_E_CUDA, std::string("adjoint FGMRES basis: ") + cudaGetErrorString(e));
-    }
-    w->mf = mf;
-  }
   std::vector<double> H((size_t)(mf + 1) * mf), cs(mf), sn(mf), gv(mf + 1), y(mf), h(mf + 1);
   auto Hat = [&](int i, int j) -> double& { return H[(size_t)i * mf + j]; };
   for (;;) {
@@ -1642,8 +1646,10 @@ int adjoint_fgmres(Ctx& c, const double* U, const double* gbar, double* lam, dou
 int adjoint_pseudo_time(crn_grid* g, const double* U, const double* gbar, double* lambda, double* sens,
                         const crn_nk_options& o, crn_nk_stats* out, cudaStream_t st, int& launches) {
   cudaError_t e = ensure_work(g, o.krylov_dim, st);
-  if (e == cudaSuccess) e = vjp_ensure_scratch(g);
   if (e == cudaSuccess && !g->nk->adj) e = cudaMalloc(&g->nk->adj, sizeof(double) * 2 * g->nk->n);
+  if (e == cudaSuccess && o.adjoint_fgmres > 0) e = ensure_fgmres(g->nk, std::min(o.adjoint_fgmres, o.krylov_dim));
+  // last: the VJP does without its scratch where nothing is left for it
+  if (e == cudaSuccess) e = vjp_ensure_scratch(g, st);
   if (e != cudaSuccess) return report(CRN_E_CUDA, std::string("adjoint workspace: ") + cudaGetErrorString(e));
   Ctx c(g, st);
   c.mode = 1;
@@ -1743,7 +1749,7 @@ int adjoint_solve(crn_grid* g, const double* U, const double* gbar, double* lamb
                   const crn_nk_options& o, crn_nk_stats* out, cudaStream_t st, int& launches) {
   if (o.adjoint_cfl > 0.0) return adjoint_pseudo_time(g, U, gbar, lambda, sens, o, out, st, launches);
   cudaError_t e = ensure_work(g, o.krylov_dim, st);
-  if (e == cudaSuccess) e = vjp_ensure_scratch(g);
+  if (e == cudaSuccess) e = vjp_ensure_scratch(g, st);
   if (e != cudaSuccess) return report(CRN_E_CUDA, std::string("adjoint workspace: ") + cudaGetErrorString(e));
   Ctx c(g, st);
   c.mode = 1;
