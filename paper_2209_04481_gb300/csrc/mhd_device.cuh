@@ -496,11 +496,13 @@ __device__ __forceinline__ void rusanov(const float (&wl)[NV], const float (&wr)
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const bool on = NZ || c < 2;
-    // momentum
+    // momentum: of the two products the pressure's is the exact one (explicit FMAs;
+    // left to the compiler it was the mass flux's, and the mean error of the
+    // momentum of a shell's cells 1.5 % larger)
     float a = ml * wl[1 + c], b = mr * wr[1 + c];
-    if (on) { a += L.pt * n[c]; b += R.pt * n[c]; }
-    a -= wl[4 + c] * L.bn;
-    b -= wr[4 + c] * R.bn;
+    if (on) { a = fmaf(L.pt, n[c], a); b = fmaf(R.pt, n[c], b); }
+    a = fmaf(-wl[4 + c], L.bn, a);
+    b = fmaf(-wr[4 + c], R.bn, b);
     f[1 + c] = h * (a + b) - d * (wr[0] * wr[1 + c] - wl[0] * wl[1 + c]);
     // induction with the GLM gradient term
     float p = L.un * wl[4 + c] - L.bn * wl[1 + c], q = R.un * wr[4 + c] - R.bn * wr[1 + c];
