@@ -748,14 +748,15 @@ __device__ __forceinline__ void tiled_item(const Shape& sh, const Geo<T>& g, con
       for (int v = 0; v < NV; ++v)
         r[v] = dr[v] + (fx[v * NFA + tl] - fx[v * NFA + tu]) + (fx[v * NFA + pl] - fx[v * NFA + pu]);
       const T vol = ROWS ? one : rad_slot(kg)[1] * s_av[jj];
-      const T ivol = ROWS ? row_iv[(kg & 1) * (TT + 1) + jj] : frcp(vol);
+      // (FP32: rounded as the including file's flags have it, approximate but in the static entry)
+      const T ivol = ROWS ? row_iv[(kg & 1) * (TT + 1) + jj] : one / vol;
       if (SUMS != SUMS_NONE) {
         const T lam = dr[NV] + (fx[NV * NFA + tl] + fx[NV * NFA + tu]) + (fx[NV * NFA + pl] + fx[NV * NFA + pu]);
         if constexpr (ROWS) {
           const T x = lam * ivol;
           rate = greater(x, rate) ? x : rate;
         } else {
-          const T x = quotient(vol, lam);
+          const T x = vol / lam;
           bound = x < bound ? x : bound;
         }
       }
