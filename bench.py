@@ -739,7 +739,7 @@ def run_ensemble(torch, pg, ci, device, stream, nsteps=200):
                 "ms_per_step": 1e3 * sec / nsteps, "launches_per_step": ens.last_launch_count,
                 "timing": "one CUDA graph of all timed steps, CUDA events"}
 
-    before = timed_residual()                 # every member: 8 x 32 tiles, its own radial chunk
+    before = timed_residual()                 # the defaults: 8 x 32 tiles, balanced radial chunks
     with torch.cuda.stream(stream):
         stream.synchronize()
         t0 = time.perf_counter()

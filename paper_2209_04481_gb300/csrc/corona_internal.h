@@ -96,7 +96,7 @@ cudaError_t vjp_ensure_scratch(crn_grid* g, cudaStream_t st);
 // ensemble records (EnsMember<T> of residual.cuh, opaque here) and launches
 size_t ens_member_bytes_fp64();
 size_t ens_member_bytes_fp32();
-// tile: the member's (theta, phi) tile shape, 0: 8 x 32, 1: 16 x 16
+// tile: the member's (theta, phi) tile shape, 0: 8 x 32, 1: 16 x 16, 2: 8 x 16 (FP64)
 int ens_fill_fp64(crn_grid* g, const void* U, void* R, int kchunk, int item0, double* nu, double* du, int tile,
                   void* dst);
 int ens_fill_fp32(crn_grid* g, const void* U, void* R, int kchunk, int item0, double* nu, double* du, int tile,

@@ -49,8 +49,8 @@ __device__ __forceinline__ double as_double(double x) { return x; }
 // warp issues at one per 16 clocks: eight sums of 32 lanes take 9 adds by
 // recursive halving (40 with a shuffle tree each), the grid is one block per SM
 // so that few partials remain, and the last block adds those.  A Krylov step's
-// products with V on 32 x 16 x 32: five launches of 20 us and five of 5 us over
-// their partials before, four of 13 us (cold) now; the step 33 -> 6.4 ms in all.
+// products with V on 32 x 16 x 32: four launches of 13 us (cold), where sums over
+// one vector at a time took five of 20 us and five of 5 us over their partials.
 struct GsOut {
   double* h;             // [m + 1] the column: h_t
   double* ww;            // [1] |w|^2 before the first pass

@@ -29,7 +29,7 @@
 // Gram-Schmidt dots and updates of an FP32 Krylov basis (basis_fp32);
 // reductions go through per-block partials summed in a fixed order, so a
 // solve is bitwise reproducible.  The host runs the GMRES recurrences (Hessenberg, Givens) and
-// synchronises the stream once or twice per Krylov step to read the dots.
+// synchronises the stream once per Krylov step to read the column of the Hessenberg matrix.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>

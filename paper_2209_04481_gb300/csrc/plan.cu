@@ -4,18 +4,19 @@
 // on how the CTAs fall on the SMs, so the launch of every candidate chunk is
 // simulated: CTAs start in launch order (all tiles of chunk 0, then chunk 1,
 // ...) on the first free slot, the first `nsm` of them on SMs of their own.
-// Measured on 152 SMs, norms included (152 x {1, 2} CTAs of 256 FP32 or 128 FP64 threads):
+// Measured on 152 SMs with 152 x {1, 2} CTAs of 256 FP32 or 128 FP64 threads, norms
+// included:
 //   * two CTAs on one SM take 4.8 us per plane where one takes 2.7 (FP32), 74
 //     where one takes 42 (FP64): two CTAs run at 0.57 of the rate of one;
 //   * the preamble (first loads, the redundant r face at the chunk's start, and
 //     the closing reduction) takes about 1.5 planes in FP32 and 0.5 in FP64,
 //     and since it is latency it does not slow down beside another CTA.
-// The chunk it picks was the fastest of those timed on every grid swept: 14 of
-// 128 planes on 128 x 64 x 128 in FP32 (64 us; 7: 68, 12: 84, 16: 71) and 9 in
-// FP64 (1.53 ms; 7 to 16: 1.65 to 1.86 before the last 4 %), 6 on 95 x 45 x 88
-// (31 us; 12: 39), 2 on 64 x 32 x 64 (17 us; 4: 19), 1 on 32 x 16 x 32 (12 us
-// against 19 with 4 planes; FP64 60 us against 176), 12 on 96 x 48 x 96 FP64
-// (0.63 ms; 16: 0.87).
+// What it picks against a sweep of 1 to 16 planes (R alone, van Albada).  FP32, the
+// fastest on each: 14 planes on 128 x 64 x 128 (61.5 us; 7: 65.4, 12: 81.9, 16: 68.3),
+// 6 on 95 x 45 x 88 (30.8 us; 5: 39.0, 12: 39.0), 2 on 64 x 32 x 64 (16.4 us; 4: 18.6),
+// 1 on 32 x 16 x 32 (12.4 us; 4: 18.5).  FP64, within 3 % of the fastest: 9 on
+// 128 x 64 x 128 (1.53 ms; 7: 1.58, 12: 1.68, 16: 1.79), 12 on 95 x 45 x 88 (0.71 ms;
+// 6: 0.69, 9: 0.86), 1 on 32 x 16 x 32 (60 us; 4: 172).
 #include <algorithm>
 #include <queue>
 #include <vector>
